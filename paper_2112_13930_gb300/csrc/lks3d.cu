@@ -79,6 +79,7 @@ struct Params3 {
     C Ks[3];                   // (1 - 1/(2 tau_f)) 3 F w for |e|^2 = 0, 1, 2 (source term)
     C cB[3];                   // 4.5 w (-1) 2 B0 for |e|^2 = 0, 1, 2 (Maxwell stress, e_y = +1)
     C omW0, omW1, omW1x4;      // w_m W_0, w_m W, 4 w_m W (D3Q7)
+    C ov, cm, gE;              // FP64 collision: w v (v = 1/36), 4.5 w v, 4 w_m W / 3
     Wall3<C> bot, top;
     C rs_back, rs_front;       // duct: tangential-component ratios of the side walls z = -b, z = +b
 };
@@ -109,6 +110,9 @@ Params3<C> make_params3(const lks3_params& p, double c_bot, double c_top, double
     q.omW0 = (C)(0.25 / p.tau_m);
     q.omW1 = (C)(0.125 / p.tau_m);
     q.omW1x4 = (C)(0.5 / p.tau_m);
+    q.ov = (C)(1.0 / p.tau_f / 36.0);
+    q.cm = (C)(0.125 / p.tau_f);
+    q.gE = (C)(0.5 / 3.0 / p.tau_m);
     const double a = 0.5 * p.ny;
     auto wall = [&](double c, double U, double ey) {
         Wall3<C> w;
@@ -213,6 +217,140 @@ __device__ __forceinline__ V tree_sum3(V (&v)[N]) {
     return v[0];
 }
 
+// FP64 form of collide3 (as lks::collide_pairs in 2D): the FP64 pipe's instruction rate is the step's
+// time, so opposite directions share the even part T and the odd part O of their equilibrium and
+// source, the quadratic forms of u and B are built from six products each, and the three
+// antisymmetric products u_d B_i - u_i B_d serve both components.  Weights are multiples of v = 1/36
+// (12, 2, 1), the velocity enters as 3 u, and A = 3 (1 - w/2) F = 0 leaves the force terms out.
+template <bool FORCE, typename In, typename Out>
+__device__ __forceinline__ void collide3_pairs(const Params3<double>& p, In F, Out out) {
+    using lks::ffma;
+    using lks::fmul;
+    const double f0 = F(0);
+    double f[19], s[10], d[10];
+#pragma unroll
+    for (int k = 1; k < 10; ++k) {  // pair k: directions 2 k - 1 and 2 k
+        f[2 * k - 1] = F(2 * k - 1);
+        f[2 * k] = F(2 * k);
+        s[k] = f[2 * k - 1] + f[2 * k];
+        d[k] = f[2 * k - 1] - f[2 * k];
+    }
+    const double drho = (((s[1] + s[2]) + (s[3] + s[4])) + ((s[5] + s[6]) + (s[7] + s[8]))) + (s[9] + f0);
+    double jx = d[1] + ((d[4] + d[5]) + (d[6] + d[7]));
+    const double jy = d[2] + ((d[4] - d[5]) + (d[8] + d[9]));
+    const double jz = d[3] + ((d[6] - d[7]) + (d[8] - d[9]));
+    if (FORCE) jx = jx + p.hFx;
+    const double rho = 1.0 + drho;
+    const double r = lks::recip_seed(rho), e = ffma(-rho, r, 1.0), r3 = fmul(3.0, r);
+    const double inv3 = ffma(r3, ffma(e, e, e), r3);  // 3/rho, as lks::recip
+    const double x3 = fmul(jx, inv3), y3 = fmul(jy, inv3), z3 = fmul(jz, inv3);
+    double g[21], dB[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+#pragma unroll
+        for (int a = 0; a < 7; ++a) g[7 * i + a] = F(19 + 7 * i + a);
+        const double* q = g + 7 * i;
+        dB[i] = ((q[1] + q[2]) + (q[3] + q[4])) + ((q[5] + q[6]) + q[0]);
+    }
+    const double bx = dB[0], dby = dB[1], bz = dB[2], by = p.B0 + dby;
+    // b_a = 4.5 (e.u)^2 - 1.5 u^2 per pair
+    const double xx = fmul(fmul(1.0 / 6.0, x3), x3), yy = fmul(fmul(1.0 / 6.0, y3), y3),
+                 zz = fmul(fmul(1.0 / 6.0, z3), z3);
+    const double h = (xx + yy) + zz;
+    const double xy = fmul(x3, y3), xz = fmul(x3, z3), yz = fmul(y3, z3);
+    double b[10];
+    b[1] = ffma(3.0, xx, -h);
+    b[2] = ffma(3.0, yy, -h);
+    b[3] = ffma(3.0, zz, -h);
+    const double cxy = ffma(3.0, yy, b[1]), cxz = ffma(3.0, zz, b[1]), cyz = ffma(3.0, zz, b[2]);
+    b[4] = cxy + xy;
+    b[5] = cxy - xy;
+    b[6] = cxz + xz;
+    b[7] = cxz - xz;
+    b[8] = cyz + yz;
+    b[9] = cyz - yz;
+    double Q = fmul(p.ov, drho), kx = 0.0;
+    const double kv = p.Ks[2];
+    if (FORCE) {
+        kx = fmul(kv, x3);
+        Q = ffma(-1.0 / 3.0, kx, Q);
+    }
+    const double P = p.ov + Q, P2 = fmul(2.0, P);
+    // Maxwell stress, products times 4.5 w v
+    const double bxs = fmul(p.cm, bx), bzs = fmul(p.cm, bz);
+    const double bxx = fmul(bxs, bx), bxy = fmul(bxs, by), bxz = fmul(bxs, bz), byz = fmul(bzs, by), bzz = fmul(bzs, bz);
+    const double dyy = fmul(fmul(p.cm, dby), p.B0 + by);
+    const double q = (bxx + dyy) + bzz;
+    const double S = ffma(-1.0 / 6.0, q, Q), R2 = ffma(2.0 / 3.0, q, fmul(2.0, Q));
+    double T[10];
+    T[1] = ffma(b[1], P2, ffma(-2.0, bxx, FORCE ? ffma(2.0, kx, R2) : R2));
+    T[2] = ffma(b[2], P2, ffma(-2.0, dyy, R2));
+    T[3] = ffma(b[3], P2, ffma(-2.0, bzz, R2));
+    double Dxy = S + bzz, Dxz = S + dyy;
+    const double Dyz = S + bxx;
+    if (FORCE) {
+        Dxy = Dxy + kx;
+        Dxz = Dxz + kx;
+        const double exy = ffma(-2.0, bxy, fmul(kv, y3)), exz = ffma(-2.0, bxz, fmul(kv, z3));
+        T[4] = ffma(b[4], P, Dxy + exy);
+        T[5] = ffma(b[5], P, Dxy - exy);
+        T[6] = ffma(b[6], P, Dxz + exz);
+        T[7] = ffma(b[7], P, Dxz - exz);
+    } else {
+        T[4] = ffma(b[4], P, ffma(-2.0, bxy, Dxy));
+        T[5] = ffma(b[5], P, ffma(2.0, bxy, Dxy));
+        T[6] = ffma(b[6], P, ffma(-2.0, bxz, Dxz));
+        T[7] = ffma(b[7], P, ffma(2.0, bxz, Dxz));
+    }
+    T[8] = ffma(b[8], P, ffma(-2.0, byz, Dyz));
+    T[9] = ffma(b[9], P, ffma(2.0, byz, Dyz));
+    const double X = FORCE ? ffma(x3, P, kv) : fmul(x3, P), Y = fmul(y3, P), Z = fmul(z3, P);
+    double O[10];
+    O[1] = X;
+    O[2] = Y;
+    O[3] = Z;
+    O[4] = X + Y;
+    O[5] = X - Y;
+    O[6] = X + Z;
+    O[7] = X - Z;
+    O[8] = Y + Z;
+    O[9] = Y - Z;
+    if (FORCE) {
+        O[1] = ffma(kv, b[1], O[1]);
+#pragma unroll
+        for (int k = 4; k < 8; ++k) O[k] = ffma(kv, b[k], O[k]);
+    }
+    const double om1 = p.om1f;
+    out(0, ffma(12.0, ffma(-h, P, S), fmul(om1, f0)));
+#pragma unroll
+    for (int k = 1; k < 10; ++k) {
+        out(2 * k - 1, ffma(om1, f[2 * k - 1], k < 4 ? ffma(2.0, O[k], T[k]) : T[k] + O[k]));
+        out(2 * k, ffma(om1, f[2 * k], k < 4 ? ffma(-2.0, O[k], T[k]) : T[k] - O[k]));
+    }
+    // g: E_di = u_d B_i - u_i B_d (times 3), + for the direction +d, - for -d
+    const double o1 = p.om1m, gE = p.gE;
+    const double Exy = ffma(x3, by, -fmul(y3, bx)), Exz = ffma(x3, bz, -fmul(z3, bx)), Eyz = ffma(y3, bz, -fmul(z3, by));
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const double* gi = g + 7 * i;
+        const int k0 = 19 + 7 * i;
+        const double b1 = fmul(p.omW1, dB[i]);
+        out(k0, ffma(o1, gi[0], fmul(p.omW0, dB[i])));
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            double up = b1, dn = b1;
+            if (c != i) {
+                const int lo = c < i ? c : i, hi = c < i ? i : c;
+                const double E = lo == 0 ? (hi == 1 ? Exy : Exz) : Eyz;
+                up = ffma(c < i ? gE : -gE, E, b1);
+                dn = ffma(c < i ? -gE : gE, E, b1);
+            }
+            out(k0 + 1 + 2 * c, ffma(o1, gi[1 + 2 * c], up));
+            out(k0 + 2 + 2 * c, ffma(o1, gi[2 + 2 * c], dn));
+        }
+    }
+}
+
 // Moments, equilibria, source and collision of one node or of a pair of nodes.  F(k) returns
 // the streamed value of slot k (wall terms included), out(k, v) takes the post-collision value of
 // slot k.  With the rest (rho = 1, u = 0, B = (0, B0, 0)) subtracted, per direction a of D3Q19
@@ -222,6 +360,13 @@ __device__ __forceinline__ V tree_sum3(V (&v)[N]) {
 //   g'_ai = (1 - w_m) g_ai + w_m W_a (dB_i + 4 e_ad E_di),  E_di = u_d B_i - B_d u_i  (E_ii = 0).
 template <typename V, typename C, typename In, typename Out>
 __device__ __forceinline__ void collide3(const Params3<C>& p, In F, Out out) {
+    if constexpr (std::is_same<V, double>::value) {
+        if (p.Fx != 0.0)
+            collide3_pairs<true>(p, F, out);
+        else
+            collide3_pairs<false>(p, F, out);
+        return;
+    }
     using namespace lks;
     typedef VecOf<V> K;
     V f[19];
@@ -409,10 +554,11 @@ __global__ void __launch_bounds__(256) step3_kernel(const S* __restrict__ fin, c
     step3_node<S, C, false>(fin, gin, fout, gout, p, x, blockIdx.y, blockIdx.z);
 }
 
-// The duct: one node per thread over the flattened node index n = (z ny + y) nx + x, so that a warp
-// covers consecutive nodes (coalesced) whatever nx is -- a fully developed duct flow has nx = 1.
-template <typename S, typename C>
-__global__ void __launch_bounds__(256) step3_duct_kernel(const S* __restrict__ fin, const S* __restrict__ gin,
+// One node per thread over the flattened node index n = (z ny + y) nx + x, so that a warp covers
+// consecutive nodes (coalesced) whatever nx is: the duct (SIDE; a fully developed duct flow has
+// nx = 1), and the FP64 channel, whose blocks are small (lks::block_f64).
+template <typename S, typename C, bool SIDE>
+__global__ void __launch_bounds__(256) step3_flat_kernel(const S* __restrict__ fin, const S* __restrict__ gin,
                                                          S* __restrict__ fout, S* __restrict__ gout,
                                                          const Params3<C> p) {
     const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -421,7 +567,7 @@ __global__ void __launch_bounds__(256) step3_duct_kernel(const S* __restrict__ f
     const int x = (int)(n - t * p.nx);
     const int z = (int)(t / p.ny);
     const int y = (int)(t - (int64_t)z * p.ny);
-    step3_node<S, C, true>(fin, gin, fout, gout, p, x, y, z);
+    step3_node<S, C, SIDE>(fin, gin, fout, gout, p, x, y, z);
 }
 
 // 16-bit storage staged through shared memory by the bulk-copy engine.  A task is R whole rows
@@ -903,7 +1049,8 @@ cudaError_t launch_step3(lks3_handle* h) {
         const int64_t N = (int64_t)p.nx * p.ny * p.nz;
         LKS3_DISPATCH(p.storage, {
             const Params3<C> q = make_params3<C>(p, h->c_bot, h->c_top, h->u_bot, h->u_top, h->c_back, h->c_front);
-            step3_duct_kernel<S, C><<<(unsigned)((N + 255) / 256), 256, 0, h->stream>>>(
+            const unsigned block = sizeof(C) == 8 ? lks::block_f64(N) : 256;
+            step3_flat_kernel<S, C, true><<<(unsigned)((N + block - 1) / block), block, 0, h->stream>>>(
                 (const S*)h->f[src], (const S*)h->g[src], (S*)h->f[src ^ 1], (S*)h->g[src ^ 1], q);
         });
         return cudaGetLastError();
@@ -917,8 +1064,17 @@ cudaError_t launch_step3(lks3_handle* h) {
     }
     LKS3_DISPATCH(p.storage, {
         const Params3<C> q = make_params3<C>(p, h->c_bot, h->c_top, h->u_bot, h->u_top);
-        step3_kernel<S, C><<<grid, 256, 0, h->stream>>>((const S*)h->f[src], (const S*)h->g[src], (S*)h->f[src ^ 1],
-                                                        (S*)h->g[src ^ 1], q);
+        const S* fi = (const S*)h->f[src];
+        const S* gi = (const S*)h->g[src];
+        S* fo = (S*)h->f[src ^ 1];
+        S* go = (S*)h->g[src ^ 1];
+        if constexpr (sizeof(C) == 8) {
+            const unsigned block = lks::block_f64(q.N);
+            step3_flat_kernel<S, C, false><<<(unsigned)((q.N + block - 1) / block), block, 0, h->stream>>>(fi, gi, fo,
+                                                                                                           go, q);
+        } else {
+            step3_kernel<S, C><<<grid, 256, 0, h->stream>>>(fi, gi, fo, go, q);
+        }
     });
     return cudaGetLastError();
 }

@@ -154,6 +154,9 @@ StepParams<double> make_step_params(int nx, int ny, int closure, double tau_f, d
     s.sw1 = s.src_coef * 3.0 * Fx * (1.0 / 9.0);
     s.sw5 = s.src_coef * 3.0 * Fx * (1.0 / 36.0);
     s.src3 = 3.0 * s.src_coef;
+    s.ov = s.omega_f / 36.0;
+    s.kv = 3.0 * s.src_coef * Fx / 36.0;
+    s.cm = 0.25 * s.omega_f;
     s.coupling = coupling;
     s.bot = wall_coef(closure, a, tau_m, B0, c_bot, u_bot, +1.0);
     s.top = wall_coef(closure, a, tau_m, B0, c_top, u_top, -1.0);

@@ -10,6 +10,7 @@ namespace lks {
 
 template <typename C>
 inline StepParams<C> convert_params(const StepParams<double>& d) {
+    static_assert(sizeof(C) == 4, "FP64 steps take the FP64 parameters as they are");
     StepParams<C> o;
     o.nx = d.nx;
     o.ny = d.ny;
@@ -47,6 +48,14 @@ inline StepParams<C> convert_params(const StepParams<double>& d) {
 // channel; c = INFINITY selects each closure's perfectly conducting limit.
 StepParams<double> make_step_params(int nx, int ny, int closure, double tau_f, double tau_m, double B0, double Fx,
                                     double c_bot, double c_top, double u_bot, double u_top, int coupling = 0);
+
+// Threads per block of the FP64 step kernels.  An FP64 warp instruction holds its SM sub-partition's
+// FP64 unit for 64 clocks, so warps that share a sub-partition add up: a 4 x 65 channel took 9.8 us of
+// FP64 work a step as 2 blocks of 256 (4 warps deep on 2 SMs).  Blocks of 64 put one or two warps on
+// an SM as long as every SM gets one block at most; blocks of 128 have one warp per sub-partition.  With
+// them and the shorter collision: 4 x 65 channel 12.7 -> 5.2 us a step, 128 x 128 duct 28.7 -> 14.3;
+// large lattices take the same time with blocks of 64, 128 and 256.
+inline unsigned block_f64(int64_t N) { return N <= 152 * 64 ? 64 : 128; }
 
 // Bytes per stored population for each lks_storage value.
 inline size_t storage_bytes(int storage) { return storage == 0 ? 8 : (storage == 1 ? 4 : 2); }

@@ -213,13 +213,13 @@ static cudaError_t launch_pair(const void* fin, const void* gin, void* fout, voi
 
 template <typename S, typename C, bool R2>
 static void launch_typed_grid(const S* fi, const S* gi, S* fo, S* go, const StepParams<C>& p, int closure,
-                              dim3 grid, cudaStream_t st) {
+                              dim3 grid, unsigned block, cudaStream_t st) {
     if (p.coupling == 0) {
-        if (closure == 0) step_kernel<S, C, 0, 0, R2><<<grid, 256, 0, st>>>(fi, gi, fo, go, p);
-        else step_kernel<S, C, 1, 0, R2><<<grid, 256, 0, st>>>(fi, gi, fo, go, p);
+        if (closure == 0) step_kernel<S, C, 0, 0, R2><<<grid, block, 0, st>>>(fi, gi, fo, go, p);
+        else step_kernel<S, C, 1, 0, R2><<<grid, block, 0, st>>>(fi, gi, fo, go, p);
     } else {
-        if (closure == 0) step_kernel<S, C, 0, 1, R2><<<grid, 256, 0, st>>>(fi, gi, fo, go, p);
-        else step_kernel<S, C, 1, 1, R2><<<grid, 256, 0, st>>>(fi, gi, fo, go, p);
+        if (closure == 0) step_kernel<S, C, 0, 1, R2><<<grid, block, 0, st>>>(fi, gi, fo, go, p);
+        else step_kernel<S, C, 1, 1, R2><<<grid, block, 0, st>>>(fi, gi, fo, go, p);
     }
 }
 
@@ -227,16 +227,18 @@ template <typename S, typename C>
 static cudaError_t launch_typed(const void* fin, const void* gin, void* fout, void* gout, const StepParams<C>& p,
                                 int closure, cudaStream_t st) {
     // FP64 is bound by the FP64 pipe, where the grid shape changes nothing (3.55 GLUPS at 4096^2
-    // either way): it keeps the 1D grid, and its 2D kernels are not instantiated
+    // either way): it keeps the 1D grid, and its 2D kernels are not instantiated.  Its blocks are
+    // small (block_f64), so that small lattices use as many SMs as they can
     if constexpr (sizeof(C) == 4) {
         if (rows2d(p.nx, p.ny)) {
             launch_typed_grid<S, C, true>((const S*)fin, (const S*)gin, (S*)fout, (S*)gout, p, closure,
-                                          dim3((p.nx + 255) / 256, p.ny), st);
+                                          dim3((p.nx + 255) / 256, p.ny), 256, st);
             return cudaGetLastError();
         }
     }
+    const unsigned block = sizeof(C) == 8 ? block_f64(p.N) : 256;
     launch_typed_grid<S, C, false>((const S*)fin, (const S*)gin, (S*)fout, (S*)gout, p, closure,
-                                   dim3((unsigned)((p.N + 255) / 256)), st);
+                                   dim3((unsigned)((p.N + block - 1) / block)), block, st);
     return cudaGetLastError();
 }
 

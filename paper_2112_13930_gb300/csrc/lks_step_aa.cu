@@ -227,26 +227,29 @@ __global__ void __launch_bounds__(256, (CLOSURE == 0 || PHASE == 0) ? 3 : 4) ste
 }
 
 template <typename S, typename C, int PHASE, bool R2>
-static void launch_aa_grid(S* f, S* g, const StepParams<C>& p, int closure, dim3 grid, cudaStream_t st) {
+static void launch_aa_grid(S* f, S* g, const StepParams<C>& p, int closure, dim3 grid, unsigned block,
+                           cudaStream_t st) {
     if (p.coupling == 0) {
-        if (closure == 0) step_kernel_aa<S, C, 0, 0, PHASE, R2><<<grid, 256, 0, st>>>(f, g, p);
-        else step_kernel_aa<S, C, 1, 0, PHASE, R2><<<grid, 256, 0, st>>>(f, g, p);
+        if (closure == 0) step_kernel_aa<S, C, 0, 0, PHASE, R2><<<grid, block, 0, st>>>(f, g, p);
+        else step_kernel_aa<S, C, 1, 0, PHASE, R2><<<grid, block, 0, st>>>(f, g, p);
     } else {
-        if (closure == 0) step_kernel_aa<S, C, 0, 1, PHASE, R2><<<grid, 256, 0, st>>>(f, g, p);
-        else step_kernel_aa<S, C, 1, 1, PHASE, R2><<<grid, 256, 0, st>>>(f, g, p);
+        if (closure == 0) step_kernel_aa<S, C, 0, 1, PHASE, R2><<<grid, block, 0, st>>>(f, g, p);
+        else step_kernel_aa<S, C, 1, 1, PHASE, R2><<<grid, block, 0, st>>>(f, g, p);
     }
 }
 
 template <typename S, typename C, int PHASE>
 static cudaError_t launch_aa_typed(void* f, void* g, const StepParams<C>& p, int closure, cudaStream_t st) {
-    // as in the two-buffer step: FP64 is FP64-pipe-bound and keeps the 1D grid
+    // as in the two-buffer step: FP64 is FP64-pipe-bound and keeps the 1D grid of small blocks
     if constexpr (sizeof(C) == 4) {
         if (p.nx >= 64 && p.ny <= 65535) {
-            launch_aa_grid<S, C, PHASE, true>((S*)f, (S*)g, p, closure, dim3((p.nx + 255) / 256, p.ny), st);
+            launch_aa_grid<S, C, PHASE, true>((S*)f, (S*)g, p, closure, dim3((p.nx + 255) / 256, p.ny), 256, st);
             return cudaGetLastError();
         }
     }
-    launch_aa_grid<S, C, PHASE, false>((S*)f, (S*)g, p, closure, dim3((unsigned)((p.N + 255) / 256)), st);
+    const unsigned block = sizeof(C) == 8 ? block_f64(p.N) : 256;
+    launch_aa_grid<S, C, PHASE, false>((S*)f, (S*)g, p, closure, dim3((unsigned)((p.N + block - 1) / block)), block,
+                                       st);
     return cudaGetLastError();
 }
 
