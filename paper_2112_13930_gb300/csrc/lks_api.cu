@@ -21,12 +21,13 @@ using lks::WallCoef;
 namespace {
 
 thread_local std::string g_last_error = "";
-// Captured graphs of 64, 32, ..., 2 steps (even, so a graph returns the state to the buffer it started
-// in), one per size and starting buffer, built on first use: lks_step(n) runs n as a few graph
-// launches (n = 100: 64 + 32 + 4) plus at most one direct launch, which matters for small lattices
-// whose steps cost less than a launch.
+// Captured graphs of 64, 32, ..., 2 launches (even, so a graph returns the state to the buffer it
+// started in), one per size and starting buffer, built on first use: lks_step(n) runs its launches
+// as a few graphs (100: 64 + 32 + 4) plus at most one direct launch, which matters for small lattices
+// whose steps cost less than a launch.  A launch is one step, or lks::kRowSteps of them where the
+// fused kernel applies (the n % kRowSteps steps left over are then launched one by one).
 constexpr int kGraphSizes = 6;
-constexpr int64_t kGraphSteps[kGraphSizes] = {64, 32, 16, 8, 4, 2};
+constexpr int64_t kGraphLaunches[kGraphSizes] = {64, 32, 16, 8, 4, 2};
 constexpr size_t kAlign = 256;
 
 inline size_t align_up(size_t x) { return (x + kAlign - 1) & ~(kAlign - 1); }
@@ -202,6 +203,7 @@ struct lks_handle {
     int* flag = nullptr;
     bool staged = false;              // 16-bit, nx % 8 == 0, nx >= 1024: the staged kernels
     lks::StagedStep ss = {nullptr, 0};
+    lks::RowsPlan rows = {0, 0, 0};     // strip > 0: kRowSteps steps per launch
     double c_bot = 0.0, c_top = 0.0, u_bot = 0.0, u_top = 0.0;
     StepParams<double> sp;
     int64_t steps = 0;
@@ -260,15 +262,24 @@ cudaError_t step_once(lks_handle* h, int src, cudaStream_t st) {
                             h->staged ? &h->ss : nullptr);
 }
 
-// Capture kGraphSteps[size] steps starting from buffer `start` into an executable graph.
+// Steps per launch of a graph, and one such launch from buffer (in place: phase) `src`.
+int launch_steps(const lks_handle* h) { return h->rows.strip ? lks::kRowSteps : 1; }
+cudaError_t launch_once(lks_handle* h, int src, cudaStream_t st) {
+    if (h->rows.strip)
+        return lks::launch_rows(h->p.storage, h->p.closure, h->f[src], h->g[src], h->f[src ^ 1], h->g[src ^ 1], h->sp,
+                                h->rows, st);
+    return step_once(h, src, st);
+}
+
+// Capture kGraphLaunches[size] launches starting from buffer `start` into an executable graph.
 cudaError_t build_graph(lks_handle* h, int size, int start) {
     cudaGraph_t graph = nullptr;
     cudaError_t e = cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return e;
     int src = start;
     cudaError_t le = cudaSuccess;
-    for (int64_t k = 0; k < kGraphSteps[size] && le == cudaSuccess; ++k) {
-        le = step_once(h, src, h->cap_stream);
+    for (int64_t k = 0; k < kGraphLaunches[size] && le == cudaSuccess; ++k) {
+        le = launch_once(h, src, h->cap_stream);
         src ^= 1;
     }
     e = cudaStreamEndCapture(h->cap_stream, &graph);
@@ -413,6 +424,8 @@ lks_status lks_create(const lks_params* p, lks_handle** out) {
         h->ss.err = h->flag;
         h->staged = e == cudaSuccess;
     }
+    if (e == cudaSuccess && !p->inplace)
+        e = lks::plan_rows(p->storage, p->closure, p->coupling, p->nx, p->ny, &h->rows);
     if (e != cudaSuccess) {
         lks_destroy(h);
         return cuda_fail(nullptr, e, "lks_create");
@@ -449,8 +462,10 @@ lks_status lks_step(lks_handle* h, int64_t n) {
     if (!h) return fail(nullptr, LKS_EINVAL, "handle is NULL");
     if (n < 0) return fail(h, LKS_EINVAL, "n must be >= 0");
     if (h->p.inplace && (n & 1)) return fail(h, LKS_EINVAL, "an in-place handle steps in pairs: n must be even");
+    const int64_t per = launch_steps(h);
+    int64_t left = n / per;  // launches of `per` steps
     for (int g = 0; g < kGraphSizes && !h->graphs_disabled; ++g) {
-        while (n >= kGraphSteps[g] && !h->graphs_disabled) {
+        while (left >= kGraphLaunches[g] && !h->graphs_disabled) {
             if (!h->graph[g][h->cur]) {
                 cudaError_t e = build_graph(h, g, h->cur);
                 if (e != cudaSuccess) {
@@ -461,11 +476,17 @@ lks_status lks_step(lks_handle* h, int64_t n) {
             }
             cudaError_t e = cudaGraphLaunch(h->graph[g][h->cur], h->stream);
             if (e != cudaSuccess) return cuda_fail(h, e, "cudaGraphLaunch");
-            n -= kGraphSteps[g];
-            h->steps += kGraphSteps[g];
+            left -= kGraphLaunches[g];
+            h->steps += per * kGraphLaunches[g];
         }
     }
-    for (int64_t k = 0; k < n; ++k) {
+    for (; left > 0; --left) {
+        cudaError_t e = launch_once(h, h->cur, h->stream);
+        if (e != cudaSuccess) return cuda_fail(h, e, "step kernel launch");
+        h->cur ^= 1;
+        h->steps += per;
+    }
+    for (n %= per; n > 0; --n) {
         cudaError_t e = step_once(h, h->cur, h->stream);
         if (e != cudaSuccess) return cuda_fail(h, e, "step kernel launch");
         h->cur ^= 1;

@@ -1,0 +1,520 @@
+// lks_step_rows.cu -- kRowSteps steps of one lattice per pass over memory (two-buffer handles, FP32
+// and 16-bit storage).
+//
+// A single FP32 step moves 152 bytes a node and runs at the HBM rate, so more steps per second need
+// fewer bytes per step: a block takes a strip of columns and marches up its rows, computing
+// level 1 (the first step) of row r from global memory, level 2 of row r - 1 from the level-1
+// rows it has just made, and so on; only the last level is stored.  Every level is the ordinary
+// step (pull, wall closures, collision, rounding to the storage type), so the state after kRowSteps
+// steps has the bits of as many single steps.
+//
+// What the next level pulls from a level: populations with e_x = 0 come from the thread's own
+// column and stay in registers (as storage words: the row above needs none of them back, the
+// own row one, the row below two rows' worth); the ten with e_x != 0 pass through shared memory,
+// in rings of three rows.  One block barrier per level and row orders them: a slot is written again
+// two barriers after its last read.
+//
+// A strip carries kRowSteps - 1 extra columns on each side, and a chunk of rows as many extra rows
+// at each end, recomputed by the neighbouring block; a row that fits one block wraps around
+// instead.
+#include <algorithm>
+#include <type_traits>
+
+#include "lks_device.cuh"
+#include "lks_internal.h"
+#include "lks_packed.cuh"
+#include "lks_pair.cuh"
+
+namespace lks {
+namespace {
+
+// Rows of the first and last chunk, whose blocks test every row for a wall and run about 1.5 times as
+// long a row, as a share of the others'.
+constexpr double kEdgeShare = 0.65;
+// Fewest rows of a chunk: each block also computes kRowSteps - 1 rows beyond either end, so that short
+// chunks lose to single steps (FP32 at 1000 x 513, 7 rows: 53.6 GLUPS against 57.4, 512^2, 4 rows: 43 against
+// 49; at 1000^2, 12 rows: 75 against 43.  FP16 at 512^2, 3 rows: 34 against 50, 1000^2, 9 rows: 69 against 68).
+constexpr int kRowMinChunk = 8;
+// Rows fetched into L2 ahead of their first use (no prefetch: FP16 92.8 instead of 100.3 GLUPS).
+constexpr int kAhead = 2;
+
+// One node per thread: a word is a stored population.
+template <typename S>
+struct OneNode {
+    typedef S W;
+    typedef float V;
+    static constexpr int kNodes = 1;
+    static __device__ __forceinline__ V unpack(W w) { return Loader<S, float, false>::ld(&w); }
+    static __device__ __forceinline__ W pack(V v) {
+        W w;
+        store_s<S, float>(&w, v);
+        return w;
+    }
+    // the population pulled from x - 1 (x + 1), given the words of the left (right) and own columns
+    static __device__ __forceinline__ W from_left(W left, W) { return left; }
+    static __device__ __forceinline__ W from_right(W, W right) { return right; }
+    static constexpr bool kOwn = false;  // own word unused by the two above
+};
+
+// Two x-adjacent nodes per thread (16-bit storage): a word holds both.
+template <typename S>
+struct TwoNodes {
+    typedef uint32_t W;
+    typedef float2 V;
+    static constexpr int kNodes = 2;
+    static __device__ __forceinline__ V unpack(W w) { return Packed<S>::pair(w); }
+    static __device__ __forceinline__ W pack(V v) { return Packed<S>::pack(v.x, v.y); }
+    static __device__ __forceinline__ W from_left(W left, W own) { return __byte_perm(left, own, 0x5432); }
+    static __device__ __forceinline__ W from_right(W own, W right) { return __byte_perm(own, right, 0x5432); }
+    static constexpr bool kOwn = true;
+};
+
+// FP16 words hold deviations times kHalfScale.  With the Maxwell coupling the two-node kernel leaves them
+// scaled: the parameters that produce populations are scaled once on the host (scaled_params), and only
+// the five moments are brought back.  A power of two commutes with every rounding here, so the bits are
+// those of the unscaled form, for 5 multiplications a pair instead of 38 (FP16 107 -> 117 GLUPS at 4096^2).
+template <typename S>
+struct TwoNodesScaled : TwoNodes<S> {
+    typedef uint32_t W;
+    typedef float2 V;
+    static __device__ __forceinline__ V unpack(W w) { return __half22float2(*reinterpret_cast<const __half2*>(&w)); }
+    static __device__ __forceinline__ W pack(V v) {
+        const __half2 h = __floats2half2_rn(v.x, v.y);
+        return *reinterpret_cast<const uint32_t*>(&h);
+    }
+};
+template <typename N> struct IsScaled { static constexpr bool value = false; };
+template <typename S> struct IsScaled<TwoNodesScaled<S>> { static constexpr bool value = true; };
+
+// Parameters of the scaled form: everything a population is made of that is not another population.
+// The moment closure runs unscaled and keeps its kx.
+StepParams<float> scaled_params(StepParams<float> p, int closure) {
+    for (float* v : {&p.owf0, &p.owf1, &p.owf5, &p.owm0, &p.owm1, &p.sw0, &p.sw1, &p.sw5, &p.bot.du, &p.top.du})
+        *v *= kHalfScale;
+    if (closure == 0) p.bot.kx *= kHalfScale, p.top.kx *= kHalfScale;
+    return p;
+}
+
+// collide_node and collide_g on scaled populations with scaled_params: the same operations in the same
+// order, the moments unscaled.
+__device__ __forceinline__ void collide_scaled(float2 f[9], float2 gx[5], float2 gy[5], const StepParams<float>& p) {
+    const float un = kHalfUnscale, half = 0.5f, three = 3.0f, four5 = 4.5f, one5 = 1.5f;
+    const auto drho = fmul(un, ((f[0] + f[1]) + (f[2] + f[3])) + ((f[4] + f[5]) + (f[6] + f[7])) + f[8]);
+    const auto rho = 1.0f + drho;
+    const auto jx = fmul(un, (f[1] - f[3]) + (f[5] - f[6]) + (f[8] - f[7]));
+    const auto jy = fmul(un, (f[2] - f[4]) + (f[5] + f[6]) - (f[7] + f[8]));
+    const auto inv_rho = recip(rho);
+    const auto ux = fmul(ffma(half, p.Fx, jx), inv_rho);
+    const auto uy = fmul(jy, inv_rho);
+    const auto bx = fmul(un, ((gx[0] + gx[1]) + (gx[2] + gx[3])) + gx[4]);
+    const auto dby = fmul(un, ((gy[0] + gy[1]) + (gy[2] + gy[3])) + gy[4]);
+    const auto by = p.B0 + dby;
+    const auto q = fmul(dby, p.B0 + by);
+    const auto om13 = fmul(p.owf1, fmul(2.25f, ffma(-bx, bx, q)));
+    const auto omxy = fmul(p.owf5, fmul(fmul(9.0f, bx), by));
+    const auto usq = fmul(one5, ffma(ux, ux, fmul(uy, uy)));
+    const auto s0 = fmul(p.sw0, -ux);
+    const auto s1p = fmul(p.sw1, 1.0f - ux), s1z = fmul(p.sw1, -ux), s1m = fmul(p.sw1, -1.0f - ux);
+    const auto s5p = fmul(p.sw5, 1.0f - ux), s5m = fmul(p.sw5, -1.0f - ux);
+    auto dir = [&](int a, float2 eu, float ow, float2 omag, float2 sa) {
+        const auto bm1 = ffma(ffma(four5, eu, three), eu, -usq);
+        const auto ofeq = ffma(ow, ffma(rho, bm1, drho), omag);
+        f[a] = ffma(p.om1f, f[a], ofeq + ffma(sa, bm1, sa));
+    };
+    const float2 zero = make_float2(0.0f, 0.0f);
+    dir(0, zero, p.owf0, zero, s0);
+    dir(1, ux, p.owf1, om13, s1p);
+    dir(2, uy, p.owf1, -om13, s1z);
+    dir(3, -ux, p.owf1, om13, s1m);
+    dir(4, -uy, p.owf1, -om13, s1z);
+    dir(5, ux + uy, p.owf5, -omxy, s5p);
+    dir(6, uy - ux, p.owf5, omxy, s5m);
+    dir(7, -ux - uy, p.owf5, -omxy, s5m);
+    dir(8, ux - uy, p.owf5, omxy, s5p);
+    collide_g<float>(gx, gy, ux, uy, bx, by, dby, p);
+}
+
+// The wall closure of a scaled moment-closed row, unscaled, and the scaled collision.
+template <int CLOSURE>
+__device__ __forceinline__ void close_collide_scaled(float2 f[9], float2 gx[5], float2 gy[5],
+                                                     const StepParams<float>& p, bool bottom, bool top) {
+    if (CLOSURE == 1 && (bottom || top)) {
+        auto all = [&](float c) {
+#pragma unroll
+            for (int a = 0; a < 9; ++a) f[a] = fmul(c, f[a]);
+#pragma unroll
+            for (int a = 0; a < 5; ++a) gx[a] = fmul(c, gx[a]), gy[a] = fmul(c, gy[a]);
+        };
+        all(kHalfUnscale);
+        if (bottom) moment_closure_bottom<float, 0>(f, gx, gy, p.bot, p);
+        if (top) moment_closure_top<float, 0>(f, gx, gy, p.top, p);
+        all(kHalfScale);
+    }
+    collide_scaled(f, gx, gy, p);
+}
+
+template <int CLOSURE, int COUPLING>
+__device__ __forceinline__ void close_collide(float f[9], float gx[5], float gy[5], const StepParams<float>& p,
+                                              bool bottom, bool top) {
+    if (CLOSURE == 1) {
+        if (bottom) moment_closure_bottom<float, COUPLING>(f, gx, gy, p.bot, p);
+        if (top) moment_closure_top<float, COUPLING>(f, gx, gy, p.top, p);
+    }
+    collide<float, COUPLING>(f, gx, gy, p);
+}
+template <int CLOSURE, int COUPLING>
+__device__ __forceinline__ void close_collide(float2 f[9], float2 gx[5], float2 gy[5], const StepParams<float>& p,
+                                              bool bottom, bool top) {
+    close_collide_pair<CLOSURE, COUPLING, true>(f, gx, gy, p, bottom, top);
+}
+
+// What a thread keeps of a level for the next one, as storage words: of the row before, the e_x = 0
+// populations (f0, gx0, gy0; f2, gx2, gy2; and, for a bottom link wall, f4, gx4, gy4), and of the
+// row before that the upward ones (f2, gx2, gy2; f5, f6 as the node pulls them).
+template <typename W>
+struct Kept {
+    W a0[3], a2[3], a4[3], b2[3], b5, b6;
+};
+
+__device__ __forceinline__ int ey9(int a) { return a == 2 || a == 5 || a == 6 ? 1 : (a == 4 || a == 7 || a == 8 ? -1 : 0); }
+__device__ __forceinline__ int ey5(int a) { return a == 2 ? 1 : (a == 4 ? -1 : 0); }
+
+// The planes of both buffers (f0..8, gx0..4, gy0..4).  As kernel parameters their addresses are uniform
+// operands of the loads and stores, to which a thread adds 32-bit offsets: computing 64-bit addresses
+// took 40 of 296 instructions per node and step.
+struct RowPlanes {
+    const char* in[19];
+    char* out[19];
+};
+
+// Ring entries of a level: f1 f3 gx1 gx3 gy1 gy3 f5 f6 f7 f8 (the populations with e_x != 0).
+constexpr int kRing = 10;
+
+template <typename S, typename N, int CLOSURE, int COUPLING, int T, int TB, int MINB>
+__global__ void __launch_bounds__(TB, MINB) rows_kernel(const __grid_constant__ RowPlanes io,
+                                                        const __grid_constant__ StepParams<float> p, int strip,
+                                                        int chunk, int edge) {
+    typedef typename N::W W;
+    typedef typename N::V V;
+    extern __shared__ __align__(16) unsigned char rows_sm[];
+    const int t = threadIdx.x;
+    const int ncol = p.nx / N::kNodes, ny = p.ny;   // columns of words
+    const unsigned pitch = (unsigned)ncol * (unsigned)sizeof(W);  // bytes of a row
+    const int x0 = blockIdx.x * strip, w = min(strip, ncol - x0);
+    const bool wrap = strip >= ncol;                // the whole row in one block
+    const int halo = wrap ? 0 : T - 1;
+    const bool lane = t < w + 2 * halo;
+    int c = lane ? x0 - halo + t : x0;
+    if (c < 0) c += ncol;
+    if (c >= ncol) c -= ncol;
+    const unsigned cl = (c == 0 ? ncol - 1 : c - 1) * sizeof(W), cc = c * sizeof(W),
+                   cr = (c == ncol - 1 ? 0 : c + 1) * sizeof(W);
+    // neighbouring threads' columns in shared memory, relative to the own one
+    const int dl = wrap && t == 0 ? w - 1 : (t == 0 ? 0 : -1);
+    const int dr = wrap && t == w - 1 ? 1 - w : (t == TB - 1 ? 0 : 1);
+    const bool mine = lane && t >= halo && t < halo + w;
+    // chunk 0 and the last one, which take the slower path with the walls, are shorter: edge rows
+    const int y0 = blockIdx.y == 0 ? 0 : edge + (blockIdx.y - 1) * chunk;
+    const int y1 = blockIdx.y == 0 ? min(edge, ny) : min(ny, y0 + chunk);
+
+    // ring slots of this row, the row before and the one before that: slot s of level k, entry v is
+    // base + ((k - 1) * 3 + s) * kRing * TB + v * TB
+    constexpr int kLevel = 3 * kRing * TB;
+    W* q0 = reinterpret_cast<W*>(rows_sm) + t;
+    W* q1 = q0 + kRing * TB;
+    W* q2 = q1 + kRing * TB;
+    Kept<W> kept[T - 1] = {};
+
+    // Row r: level 1 of row r, ..., level T of row r - (T - 1).  now / before: ring slots.
+    auto row = [&](auto walls, int r, W* now, W* before) {
+        // Without WALLS no level's row is beyond or at a wall; a level that is not on yet then computes
+        // something nobody uses.
+        constexpr bool WALLS = decltype(walls)::value;
+        V f[9], gx[5], gy[5];
+        W cur[9];  // words of the level just computed: f0 gx0 gy0, f2 gx2 gy2, f4 gx4 gy4
+#pragma unroll
+        for (int k = 1; k <= T; ++k) {
+            const int j = r - (k - 1);  // this level's row
+            const bool on = !WALLS || (j >= max(0, y0 - (T - k)) && j < min(ny, y1 + (T - k)));
+            const bool bottom = WALLS && j == 0, top = WALLS && j == ny - 1;
+            if (k == 1) {
+                if (on) {
+                    const unsigned rc = (unsigned)j * pitch, rs = rc - pitch, rn = rc + pitch;  // bytes
+                    auto word = [&](int a, unsigned at) -> W {
+                        return __ldg(reinterpret_cast<const W*>(io.in[a] + at));
+                    };
+                    auto same = [&](int a, unsigned row) -> V { return N::unpack(word(a, row + cc)); };
+                    auto left = [&](int a, unsigned row) -> V {
+                        return N::unpack(N::from_left(word(a, row + cl), N::kOwn ? word(a, row + cc) : W()));
+                    };
+                    auto right = [&](int a, unsigned row) -> V {
+                        return N::unpack(N::from_right(N::kOwn ? word(a, row + cc) : W(), word(a, row + cr)));
+                    };
+                    f[0] = same(0, rc);
+                    f[1] = left(1, rc);
+                    f[3] = right(3, rc);
+                    gx[0] = same(9, rc);
+                    gx[1] = left(10, rc);
+                    gx[3] = right(12, rc);
+                    gy[0] = same(14, rc);
+                    gy[1] = left(15, rc);
+                    gy[3] = right(17, rc);
+                    if (!bottom) {
+                        f[2] = same(2, rs);
+                        f[5] = left(5, rs);
+                        f[6] = right(6, rs);
+                        gx[2] = same(11, rs);
+                        gy[2] = same(16, rs);
+                    } else if (CLOSURE == 0) {  // the node's own outgoing populations
+                        f[2] = same(4, rc);
+                        f[5] = same(7, rc);
+                        f[6] = same(8, rc);
+                        gx[2] = same(13, rc);
+                        gy[2] = same(18, rc);
+                    }
+                    if (!top) {
+                        f[4] = same(4, rn);
+                        f[7] = right(7, rn);
+                        f[8] = left(8, rn);
+                        gx[4] = same(13, rn);
+                        gy[4] = same(18, rn);
+                    } else if (CLOSURE == 0) {
+                        f[4] = same(2, rc);
+                        f[7] = same(5, rc);
+                        f[8] = same(6, rc);
+                        gx[4] = same(11, rc);
+                        gy[4] = same(16, rc);
+                    }
+                }
+            } else {
+                // the level before: row j + 1 in `cur` and slot `now`, row j in `kept` and slot `before`
+                W *rn = now + (k - 2) * kLevel, *rb = before + (k - 2) * kLevel;
+                const W *rnl = rn + dl, *rnr = rn + dr, *rbl = rb + dl, *rbr = rb + dr;
+                auto left = [&](const W* q, const W* ql, int v) -> W {
+                    return N::from_left(ql[v * TB], N::kOwn ? q[v * TB] : W());
+                };
+                auto right = [&](const W* q, const W* qr, int v) -> W {
+                    return N::from_right(N::kOwn ? q[v * TB] : W(), qr[v * TB]);
+                };
+                Kept<W>& K = kept[k - 2];
+                if (on) {
+                    f[0] = N::unpack(K.a0[0]);
+                    gx[0] = N::unpack(K.a0[1]);
+                    gy[0] = N::unpack(K.a0[2]);
+                    f[1] = N::unpack(left(rb, rbl, 0));
+                    f[3] = N::unpack(right(rb, rbr, 1));
+                    gx[1] = N::unpack(left(rb, rbl, 2));
+                    gx[3] = N::unpack(right(rb, rbr, 3));
+                    gy[1] = N::unpack(left(rb, rbl, 4));
+                    gy[3] = N::unpack(right(rb, rbr, 5));
+                    if (!bottom) {
+                        f[2] = N::unpack(K.b2[0]);
+                        gx[2] = N::unpack(K.b2[1]);
+                        gy[2] = N::unpack(K.b2[2]);
+                        f[5] = N::unpack(K.b5);
+                        f[6] = N::unpack(K.b6);
+                    } else if (CLOSURE == 0) {
+                        f[2] = N::unpack(K.a4[0]);
+                        gx[2] = N::unpack(K.a4[1]);
+                        gy[2] = N::unpack(K.a4[2]);
+                        f[5] = N::unpack(rb[8 * TB]);
+                        f[6] = N::unpack(rb[9 * TB]);
+                    }
+                    if (!top) {
+                        f[4] = N::unpack(cur[6]);
+                        gx[4] = N::unpack(cur[7]);
+                        gy[4] = N::unpack(cur[8]);
+                        f[7] = N::unpack(right(rn, rnr, 8));
+                        f[8] = N::unpack(left(rn, rnl, 9));
+                    } else if (CLOSURE == 0) {
+                        f[4] = N::unpack(K.a2[0]);
+                        gx[4] = N::unpack(K.a2[1]);
+                        gy[4] = N::unpack(K.a2[2]);
+                        f[7] = N::unpack(rb[6 * TB]);
+                        f[8] = N::unpack(rb[7 * TB]);
+                    }
+                }
+                // the level before moves up one row
+#pragma unroll
+                for (int q = 0; q < 3; ++q) {
+                    K.b2[q] = K.a2[q];
+                    K.a0[q] = cur[q];
+                    K.a2[q] = cur[3 + q];
+                    if (CLOSURE == 0) K.a4[q] = cur[6 + q];
+                }
+                K.b5 = left(rb, rbl, 6);
+                K.b6 = right(rb, rbr, 7);
+            }
+            if (on) {
+                if (CLOSURE == 0) {
+                    if (bottom) {
+                        f[5] = f[5] + p.bot.du;
+                        f[6] = f[6] - p.bot.du;
+                        gx[2] = ffma(p.bot.r, gx[2], p.bot.kx);
+                        gy[2] = -gy[2];
+                    }
+                    if (top) {
+                        f[7] = f[7] - p.top.du;
+                        f[8] = f[8] + p.top.du;
+                        gx[4] = ffma(p.top.r, gx[4], p.top.kx);
+                        gy[4] = -gy[4];
+                    }
+                }
+                if constexpr (IsScaled<N>::value)
+                    close_collide_scaled<CLOSURE>(f, gx, gy, p, bottom, top);
+                else
+                    close_collide<CLOSURE, COUPLING>(f, gx, gy, p, bottom, top);
+                if (k < T) {
+                    W* ring = now + (k - 1) * kLevel;
+                    const V x[kRing] = {f[1], f[3], gx[1], gx[3], gy[1], gy[3], f[5], f[6], f[7], f[8]};
+#pragma unroll
+                    for (int v = 0; v < kRing; ++v) ring[v * TB] = N::pack(x[v]);
+                    const V own[9] = {f[0], gx[0], gy[0], f[2], gx[2], gy[2], f[4], gx[4], gy[4]};
+#pragma unroll
+                    for (int q = 0; q < 9; ++q) cur[q] = N::pack(own[q]);
+                } else if (mine && (WALLS || j >= y0)) {
+                    const unsigned n = (unsigned)j * pitch + cc;
+                    auto put = [&](int a, V v) {
+                        *reinterpret_cast<W*>(io.out[a] + n) = N::pack(v);
+                    };
+#pragma unroll
+                    for (int a = 0; a < 9; ++a) put(a, f[a]);
+#pragma unroll
+                    for (int a = 0; a < 5; ++a) put(9 + a, gx[a]);
+#pragma unroll
+                    for (int a = 0; a < 5; ++a) put(14 + a, gy[a]);
+                }
+            }
+            if (k < T) __syncthreads();
+        }
+    };
+
+    // The row that iteration r + kAhead will be the first to pull, brought into L2 (one line of one plane
+    // per thread).
+    const int lines = (w + 2 * halo) * (int)sizeof(W) / 128 + 1, pa = t / lines;
+    const int pey = pa < 9 ? ey9(pa) : ey5(pa < 14 ? pa - 9 : pa - 14);
+    const int px = x0 - halo < 0 ? 0 : x0 - halo;
+    const char* pf = io.in[min(pa, 18)] +
+                     min((px + (t % lines) * (128 / (int)sizeof(W))), ncol - 1) * (int)sizeof(W);
+    auto prefetch = [&](int r) {
+        const int y = r + kAhead - pey;
+        if (pa < 19 && y >= 0 && y < ny) asm volatile("prefetch.global.L2 [%0];" ::"l"(pf + (uint64_t)((unsigned)y * pitch)));
+    };
+    auto up = [&]() {  // the slots move up one row
+        W* q = q0;
+        q0 = q1;
+        q1 = q2;
+        q2 = q;
+    };
+    const int last = y1 - 1 + (T - 1);
+    if (y0 >= T && y1 <= ny - T) {
+#pragma unroll 1
+        for (int r = y0 - (T - 1); r <= last; ++r) {
+            prefetch(r);
+            row(std::false_type{}, r, q0, q2);
+            up();
+        }
+    } else {
+#pragma unroll 1
+        for (int r = max(0, y0 - (T - 1)); r <= last; ++r) {
+            row(std::true_type{}, r, q0, q2);
+            up();
+        }
+    }
+}
+
+template <typename S, typename N, int TB, int MINB>
+struct Rows {
+    static constexpr int kThreads = TB, kNodes = N::kNodes;
+    // the Maxwell coupling's form of the node type
+    static constexpr bool kScaled = std::is_same<N, TwoNodes<__half>>::value;
+    typedef typename std::conditional<kScaled, TwoNodesScaled<S>, N>::type M;
+    typedef void (*Fn)(const RowPlanes, const StepParams<float>, int, int, int);
+    static Fn kernel(int closure, int coupling) {
+        constexpr int T = kRowSteps;
+        if (coupling == 0)
+            return closure == 0 ? rows_kernel<S, M, 0, 0, T, TB, MINB> : rows_kernel<S, M, 1, 0, T, TB, MINB>;
+        return closure == 0 ? rows_kernel<S, N, 0, 1, T, TB, MINB> : rows_kernel<S, N, 1, 1, T, TB, MINB>;
+    }
+    static constexpr size_t smem() { return (size_t)(kRowSteps - 1) * 3 * kRing * TB * sizeof(typename N::W); }
+    static cudaError_t prepare(int closure, int coupling, int* blocks) {
+        Fn k = kernel(closure, coupling);
+        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem());
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, k, TB, smem());
+        return e;
+    }
+    static void launch(const void* fin, const void* gin, void* fout, void* gout, const StepParams<float>& p,
+                       int closure, const RowsPlan& rp, cudaStream_t st) {
+        const dim3 grid((p.nx / N::kNodes + rp.strip - 1) / rp.strip,
+                        rp.edge >= p.ny ? 1 : 1 + (p.ny - rp.edge + rp.chunk - 1) / rp.chunk);
+        RowPlanes io;
+        for (int a = 0; a < 19; ++a) {
+            io.in[a] = (const char*)(a < 9 ? (const S*)fin + a * p.N : (const S*)gin + (a - 9) * p.N);
+            io.out[a] = (char*)(a < 9 ? (S*)fout + a * p.N : (S*)gout + (a - 9) * p.N);
+        }
+        kernel(closure, p.coupling)<<<grid, TB, smem(), st>>>(
+            io, kScaled && p.coupling == 0 ? scaled_params(p, closure) : p, rp.strip, rp.chunk, rp.edge);
+    }
+};
+// Threads per block and blocks per SM, timed at 4096^2 (GLUPS, moment closure): FP32 128 x 5 98, 128 x 6 93,
+// 192 x 4 98, 256 x 3 91, 320 x 2 92; BF16 128 x 4 126, 96 x 5 118, 256 x 2 113, 128 x 5 98 (spills).  Small
+// blocks wait less at their barriers; the extra columns of narrow strips cost more below 128.
+#define F32S 128, 5
+#define H16S 128, 4
+typedef Rows<float, OneNode<float>, F32S> RowsF32;
+typedef Rows<__nv_bfloat16, TwoNodes<__nv_bfloat16>, H16S> RowsBf16;
+typedef Rows<__half, TwoNodes<__half>, H16S> RowsF16;
+
+}  // namespace
+
+// Strips and chunks of the kernel R: as many blocks as are resident at once.
+template <typename R>
+static cudaError_t plan_typed(int closure, int coupling, int nx, int ny, RowsPlan* rp) {
+    int dev = 0, sms = 0, blocks = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = R::prepare(closure, coupling, &blocks);
+    if (e != cudaSuccess) return e;
+    const int ncol = nx / R::kNodes;
+    const int most = R::kThreads - 2 * (kRowSteps - 1);
+    int strips = 1, strip = ncol;
+    if (ncol > R::kThreads) {
+        strips = (ncol + most - 1) / most;
+        strip = std::min(most, ((ncol + strips - 1) / strips + 7) / 8 * 8);
+        strips = (ncol + strip - 1) / strip;
+    }
+    const int slots = std::max(1, sms * blocks / strips);
+    // chunks of `chunk` rows and one of `edge` rows at each wall: 2 edge + (slots - 2) chunk >= ny
+    int chunk = (ny + slots - 1) / slots, edge = chunk;
+    if (slots >= 3) {
+        chunk = (int)((ny + slots - 2 * kEdgeShare) / (slots - 2 + 2 * kEdgeShare));
+        for (;; ++chunk) {
+            edge = std::max(kRowSteps, (int)(kEdgeShare * chunk));
+            if (2 * (int64_t)edge + (int64_t)(slots - 2) * chunk >= ny) break;
+        }
+    }
+    if (chunk < kRowMinChunk) return cudaSuccess;
+    rp->strip = strip;
+    rp->chunk = chunk;
+    rp->edge = edge;
+    return cudaSuccess;
+}
+
+cudaError_t plan_rows(int storage, int closure, int coupling, int nx, int ny, RowsPlan* rp) {
+    rp->strip = rp->chunk = rp->edge = 0;
+    if (storage == 0 || (storage >= 2 && nx % 2 != 0) || nx < 64) return cudaSuccess;
+    if (storage == 1) return plan_typed<RowsF32>(closure, coupling, nx, ny, rp);
+    if (storage == 2) return plan_typed<RowsBf16>(closure, coupling, nx, ny, rp);
+    return plan_typed<RowsF16>(closure, coupling, nx, ny, rp);
+}
+
+cudaError_t launch_rows(int storage, int closure, const void* fin, const void* gin, void* fout, void* gout,
+                        const StepParams<double>& pd, const RowsPlan& rp, cudaStream_t st) {
+    const StepParams<float> p = convert_params<float>(pd);
+    if (storage == 1) RowsF32::launch(fin, gin, fout, gout, p, closure, rp, st);
+    else if (storage == 2) RowsBf16::launch(fin, gin, fout, gout, p, closure, rp, st);
+    else RowsF16::launch(fin, gin, fout, gout, p, closure, rp, st);
+    return cudaGetLastError();
+}
+
+}  // namespace lks
