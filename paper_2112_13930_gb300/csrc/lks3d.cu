@@ -30,6 +30,7 @@
 #include "lks_bulk.cuh"
 #include "lks_internal.h"
 #include "lks_packed.cuh"
+#include "lks_pdl.cuh"
 #include "lks_vec.cuh"
 
 using lks::load_s;
@@ -480,8 +481,7 @@ __device__ __forceinline__ void collide3(const Params3<C>& p, In F, Out out) {
 // wall it crosses (no corner reconstruction); a link through both a y and a z wall (e_x = 0, f only)
 // is closed by the y wall, whose bounce-back adds no moving-wall term when e_x = 0.
 template <typename S, typename C, bool SIDE>
-__device__ __forceinline__ void step3_node(const S* __restrict__ fin, const S* __restrict__ gin,
-                                           S* __restrict__ fout, S* __restrict__ gout, const Params3<C>& p, int x,
+__device__ __forceinline__ void step3_node(const S* fin, const S* gin, S* fout, S* gout, const Params3<C>& p, int x,
                                            int y, int z) {
     const int nx = p.nx, ny = p.ny, nz = p.nz;
     const int64_t N = p.N;
@@ -504,16 +504,16 @@ __device__ __forceinline__ void step3_node(const S* __restrict__ fin, const S* _
     for (int a = 0; a < 19; ++a) {
         const int ey = EYa(a);
         if (cut(a)) continue;  // filled below
-        v[a] = load_s<S, C>(fin + a * N + src(EXa(a), ey, EZa(a)));
+        v[a] = lks::Loader<S, C, false>::ld(fin + a * N + src(EXa(a), ey, EZa(a)));
     }
 #pragma unroll
     for (int a = 0; a < 7; ++a) {
         const int ey = EYa(a);
         if (cut(a)) continue;
         const int64_t s = src(EXa(a), ey, EZa(a));
-        v[19 + a] = load_s<S, C>(gin + a * N + s);
-        v[26 + a] = load_s<S, C>(gin + (7 + a) * N + s);
-        v[33 + a] = load_s<S, C>(gin + (14 + a) * N + s);
+        v[19 + a] = lks::Loader<S, C, false>::ld(gin + a * N + s);
+        v[26 + a] = lks::Loader<S, C, false>::ld(gin + (7 + a) * N + s);
+        v[33 + a] = lks::Loader<S, C, false>::ld(gin + (14 + a) * N + s);
     }
     // wall rows: the node's own populations of the opposite directions, with the closure's terms
     if (bottom) {  // entering along e_y = +1: 3, 7, 10, 15, 17 (D3Q19); 3 (D3Q7)
@@ -521,7 +521,7 @@ __device__ __forceinline__ void step3_node(const S* __restrict__ fin, const S* _
         for (int k = 0; k < 40; ++k) {
             const int a = slot_dir3(k);
             if (EYa(a) != 1) continue;
-            v[k] = wall_in3<C, C>(p, true, false, k, load_s<S, C>((k < 19 ? fin : gin) + slot_plane3(k, opp(a)) * N + n));
+            v[k] = wall_in3<C, C>(p, true, false, k, lks::Loader<S, C, false>::ld((k < 19 ? fin : gin) + slot_plane3(k, opp(a)) * N + n));
         }
     }
     if (top) {  // entering along e_y = -1: 4, 8, 9, 16, 18; 4
@@ -529,7 +529,7 @@ __device__ __forceinline__ void step3_node(const S* __restrict__ fin, const S* _
         for (int k = 0; k < 40; ++k) {
             const int a = slot_dir3(k);
             if (EYa(a) != -1) continue;
-            v[k] = wall_in3<C, C>(p, false, true, k, load_s<S, C>((k < 19 ? fin : gin) + slot_plane3(k, opp(a)) * N + n));
+            v[k] = wall_in3<C, C>(p, false, true, k, lks::Loader<S, C, false>::ld((k < 19 ? fin : gin) + slot_plane3(k, opp(a)) * N + n));
         }
     }
     if (SIDE && (back || front)) {  // entering along e_z = +1 at z = 0, e_z = -1 at z = nz-1
@@ -538,7 +538,7 @@ __device__ __forceinline__ void step3_node(const S* __restrict__ fin, const S* _
             const int a = slot_dir3(k), ey = EYa(a), ez = EZa(a);
             if (!((ez == 1 && back) || (ez == -1 && front))) continue;
             if ((ey == 1 && bottom) || (ey == -1 && top)) continue;  // closed by the y wall above
-            v[k] = side_in3<C, C>(p, ez == 1, k, load_s<S, C>((k < 19 ? fin : gin) + slot_plane3(k, opp(a)) * N + n));
+            v[k] = side_in3<C, C>(p, ez == 1, k, lks::Loader<S, C, false>::ld((k < 19 ? fin : gin) + slot_plane3(k, opp(a)) * N + n));
         }
     }
     collide3<C, C>(p, [&](int k) -> C { return v[k]; },
@@ -547,8 +547,9 @@ __device__ __forceinline__ void step3_node(const S* __restrict__ fin, const S* _
 
 // One node per thread, x fastest (grid: x blocks, y, z).
 template <typename S, typename C>
-__global__ void __launch_bounds__(256) step3_kernel(const S* __restrict__ fin, const S* __restrict__ gin,
-                                                    S* __restrict__ fout, S* __restrict__ gout, const Params3<C> p) {
+__global__ void __launch_bounds__(256) step3_kernel(const S* fin, const S* gin, S* fout, S* gout,
+                                                    const Params3<C> p) {
+    lks::pdl_wait();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= p.nx) return;
     step3_node<S, C, false>(fin, gin, fout, gout, p, x, blockIdx.y, blockIdx.z);
@@ -558,9 +559,9 @@ __global__ void __launch_bounds__(256) step3_kernel(const S* __restrict__ fin, c
 // consecutive nodes (coalesced) whatever nx is: the duct (SIDE; a fully developed duct flow has
 // nx = 1), and the FP64 channel, whose blocks are small (lks::block_f64).
 template <typename S, typename C, bool SIDE>
-__global__ void __launch_bounds__(256) step3_flat_kernel(const S* __restrict__ fin, const S* __restrict__ gin,
-                                                         S* __restrict__ fout, S* __restrict__ gout,
+__global__ void __launch_bounds__(256) step3_flat_kernel(const S* fin, const S* gin, S* fout, S* gout,
                                                          const Params3<C> p) {
+    lks::pdl_wait();
     const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (n >= p.N) return;
     const int64_t t = n / p.nx;
@@ -617,6 +618,7 @@ __global__ void __launch_bounds__(kThreads3, 1) step3_staged_kernel(const S* __r
         }
         lks::mbar_init_fence();
     }
+    lks::pdl_wait();
     __syncthreads();
 
     if (warp == kConsumerWarps3) {  // producer: lane l fetches slots l and l + 32
@@ -936,6 +938,11 @@ Layout3 layout3(const lks3_params* p) {
 
 }  // namespace
 
+// Steps of the captured graphs (even: a graph returns the state to the buffer it started in), as in
+// lks_step: small lattices' steps cost less than a launch from the host.
+constexpr int kGraphSizes3 = 6;
+constexpr int64_t kGraphSteps3[kGraphSizes3] = {64, 32, 16, 8, 4, 2};
+
 struct lks3_handle {
     lks3_params p;
     Layout3 L;
@@ -955,6 +962,9 @@ struct lks3_handle {
     bool side = false;                 // duct: walls at the z planes (lks3_set_side_walls)
     double c_back = 0.0, c_front = 0.0;
     int64_t steps = 0;
+    cudaStream_t cap_stream = nullptr;
+    cudaGraphExec_t graph[kGraphSizes3][2] = {};  // by size and starting buffer, built on first use
+    bool graphs_disabled = false;
     std::string err;
 };
 
@@ -1007,13 +1017,13 @@ unsigned grid_for(int64_t N) { return (unsigned)std::min<int64_t>((N + 255) / 25
     } while (0)
 
 template <typename S>
-void launch_staged3(lks3_handle* h, int src) {
+void launch_staged3(lks3_handle* h, int src, cudaStream_t st) {
     const lks3_params& p = h->p;
     const int R = rows_per_task3(p.nx, p.ny);
     const int64_t ntask = (int64_t)p.nz * ((p.ny + R - 1) / R);
     const unsigned grid = (unsigned)std::min<int64_t>(ntask, h->staged_grid);
     const Params3<float> q = make_params3<float>(p, h->c_bot, h->c_top, h->u_bot, h->u_top);
-    step3_staged_kernel<S><<<grid, kThreads3, staged_smem3(), h->stream>>>(
+    lks::launch_pdl(step3_staged_kernel<S>, grid, kThreads3, staged_smem3(), st, 
         (const S*)h->f[src], (const S*)h->g[src], (S*)h->f[src ^ 1], (S*)h->g[src ^ 1], q, R, h->flag);
 }
 
@@ -1041,25 +1051,24 @@ cudaError_t prepare_staged3(lks3_handle* h) {
     return e;
 }
 
-cudaError_t launch_step3(lks3_handle* h) {
+cudaError_t launch_step3(lks3_handle* h, int src, cudaStream_t st) {
     const lks3_params& p = h->p;
     const dim3 grid((p.nx + 255) / 256, p.ny, p.nz);
-    const int src = h->cur;
     if (h->side) {
         const int64_t N = (int64_t)p.nx * p.ny * p.nz;
         LKS3_DISPATCH(p.storage, {
             const Params3<C> q = make_params3<C>(p, h->c_bot, h->c_top, h->u_bot, h->u_top, h->c_back, h->c_front);
             const unsigned block = sizeof(C) == 8 ? lks::block_f64(N) : 256;
-            step3_flat_kernel<S, C, true><<<(unsigned)((N + block - 1) / block), block, 0, h->stream>>>(
+            lks::launch_pdl(step3_flat_kernel<S, C, true>, dim3((unsigned)((N + block - 1) / block)), block, 0, st, 
                 (const S*)h->f[src], (const S*)h->g[src], (S*)h->f[src ^ 1], (S*)h->g[src ^ 1], q);
         });
         return cudaGetLastError();
     }
     if (h->staged) {
         if (p.storage == LKS_BF16_DEV)
-            launch_staged3<__nv_bfloat16>(h, src);
+            launch_staged3<__nv_bfloat16>(h, src, st);
         else
-            launch_staged3<__half>(h, src);
+            launch_staged3<__half>(h, src, st);
         return cudaGetLastError();
     }
     LKS3_DISPATCH(p.storage, {
@@ -1070,13 +1079,36 @@ cudaError_t launch_step3(lks3_handle* h) {
         S* go = (S*)h->g[src ^ 1];
         if constexpr (sizeof(C) == 8) {
             const unsigned block = lks::block_f64(q.N);
-            step3_flat_kernel<S, C, false><<<(unsigned)((q.N + block - 1) / block), block, 0, h->stream>>>(fi, gi, fo,
+            lks::launch_pdl(step3_flat_kernel<S, C, false>, dim3((unsigned)((q.N + block - 1) / block)), block, 0, st, fi, gi, fo,
                                                                                                            go, q);
         } else {
-            step3_kernel<S, C><<<grid, 256, 0, h->stream>>>(fi, gi, fo, go, q);
+            lks::launch_pdl(step3_kernel<S, C>, grid, 256, 0, st, fi, gi, fo, go, q);
         }
     });
     return cudaGetLastError();
+}
+
+void drop_graphs3(lks3_handle* h) {
+    for (auto& pair : h->graph)
+        for (cudaGraphExec_t& g : pair)
+            if (g) {
+                cudaGraphExecDestroy(g);
+                g = nullptr;
+            }
+}
+
+// Capture kGraphSteps3[size] steps starting from buffer `start` into an executable graph.
+cudaError_t build_graph3(lks3_handle* h, int size, int start) {
+    cudaGraph_t graph = nullptr;
+    cudaError_t e = cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal);
+    if (e != cudaSuccess) return e;
+    cudaError_t le = cudaSuccess;
+    for (int64_t k = 0; k < kGraphSteps3[size] && le == cudaSuccess; ++k)
+        le = launch_step3(h, (start + (int)k) & 1, h->cap_stream);
+    e = cudaStreamEndCapture(h->cap_stream, &graph);
+    if (le == cudaSuccess && e == cudaSuccess) e = cudaGraphInstantiate(&h->graph[size][start], graph, 0);
+    if (graph) cudaGraphDestroy(graph);
+    return le != cudaSuccess ? le : e;
 }
 
 cudaError_t launch_snapshot3(lks3_handle* h) {
@@ -1135,6 +1167,7 @@ lks_status lks3_create(const lks3_params* p, lks3_handle** out) {
     double rest[19];
     for (int a = 0; a < 19; ++a) rest[a] = f_rest(a, p->B0);
     e = cudaHostAlloc((void**)&h->host4, 4 * sizeof(double), cudaHostAllocDefault);
+    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking);
     // rest state: all deviations zero
     if (e == cudaSuccess) e = cudaMemsetAsync(h->f[0], 0, h->L.f_bytes, h->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(h->g[0], 0, h->L.g_bytes, h->stream);
@@ -1159,6 +1192,7 @@ lks_status lks3_set_walls(lks3_handle* h, double c_bottom, double c_top, double 
     h->c_top = c_top;
     h->u_bot = u_bottom;
     h->u_top = u_top;
+    drop_graphs3(h);
     return LKS_OK;
 }
 
@@ -1170,14 +1204,28 @@ lks_status lks3_set_side_walls(lks3_handle* h, int32_t enable, double c_back, do
     h->side = enable != 0;
     h->c_back = c_back;
     h->c_front = c_front;
+    drop_graphs3(h);
     return LKS_OK;
 }
 
 lks_status lks3_step(lks3_handle* h, int64_t n) {
     if (!h) return fail3(nullptr, LKS_EINVAL, "handle is NULL");
     if (n < 0) return fail3(h, LKS_EINVAL, "n must be >= 0");
+    for (int g = 0; g < kGraphSizes3 && !h->graphs_disabled; ++g) {
+        while (n >= kGraphSteps3[g]) {
+            if (!h->graph[g][h->cur] && build_graph3(h, g, h->cur) != cudaSuccess) {
+                cudaGetLastError();
+                h->graphs_disabled = true;  // fall back to direct launches
+                break;
+            }
+            cudaError_t e = cudaGraphLaunch(h->graph[g][h->cur], h->stream);
+            if (e != cudaSuccess) return cuda3(h, e, "cudaGraphLaunch");
+            n -= kGraphSteps3[g];
+            h->steps += kGraphSteps3[g];
+        }
+    }
     for (int64_t k = 0; k < n; ++k) {
-        cudaError_t e = launch_step3(h);
+        cudaError_t e = launch_step3(h, h->cur, h->stream);
         if (e != cudaSuccess) return cuda3(h, e, "3D step kernel launch");
         h->cur ^= 1;
         h->steps += 1;
@@ -1399,6 +1447,8 @@ lks_status lks3_sync(lks3_handle* h) {
 lks_status lks3_destroy(lks3_handle* h) {
     if (!h) return LKS_OK;
     if (h->stream || h->base) cudaStreamSynchronize(h->stream);
+    drop_graphs3(h);
+    if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
     if (h->state_stage) cudaFree(h->state_stage);
     if (h->owns && h->base) cudaFree(h->base);
     if (h->host4) cudaFreeHost(h->host4);

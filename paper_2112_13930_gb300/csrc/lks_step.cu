@@ -12,15 +12,16 @@
 #include "lks_device.cuh"
 #include "lks_internal.h"
 #include "lks_packed.cuh"
+#include "lks_pdl.cuh"
 
 namespace lks {
 
 // ROWS2D: grid (ceil(nx/256), ny), the column and row come from the block indices; otherwise a
 // 1D grid over n = y*nx + x (narrow lattices), split with one 32-bit division.
 template <typename S, typename C, int CLOSURE, int COUPLING, bool ROWS2D>
-__global__ void __launch_bounds__(256) step_kernel(const S* __restrict__ fin, const S* __restrict__ gin,
-                                                   S* __restrict__ fout, S* __restrict__ gout,
+__global__ void __launch_bounds__(256) step_kernel(const S* fin, const S* gin, S* fout, S* gout,
                                                    const StepParams<C> p) {
+    pdl_wait();
     int i, j;
     if (ROWS2D) {
         i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -33,7 +34,7 @@ __global__ void __launch_bounds__(256) step_kernel(const S* __restrict__ fin, co
         i = (int)(n32 - (unsigned)j * (unsigned)p.nx);
     }
     const int64_t n = (int64_t)j * p.nx + i;
-    step_node<S, C, CLOSURE, true, COUPLING>(fin, gin, fout, gout, p, n, i, j);
+    step_node<S, C, CLOSURE, false, COUPLING>(fin, gin, fout, gout, p, n, i, j);
 }
 
 // 16-bit storage moves 2 bytes per population, so the one-node kernel issues twice the load/store
@@ -215,11 +216,11 @@ template <typename S, typename C, bool R2>
 static void launch_typed_grid(const S* fi, const S* gi, S* fo, S* go, const StepParams<C>& p, int closure,
                               dim3 grid, unsigned block, cudaStream_t st) {
     if (p.coupling == 0) {
-        if (closure == 0) step_kernel<S, C, 0, 0, R2><<<grid, block, 0, st>>>(fi, gi, fo, go, p);
-        else step_kernel<S, C, 1, 0, R2><<<grid, block, 0, st>>>(fi, gi, fo, go, p);
+        if (closure == 0) launch_pdl(step_kernel<S, C, 0, 0, R2>, grid, block, 0, st, fi, gi, fo, go, p);
+        else launch_pdl(step_kernel<S, C, 1, 0, R2>, grid, block, 0, st, fi, gi, fo, go, p);
     } else {
-        if (closure == 0) step_kernel<S, C, 0, 1, R2><<<grid, block, 0, st>>>(fi, gi, fo, go, p);
-        else step_kernel<S, C, 1, 1, R2><<<grid, block, 0, st>>>(fi, gi, fo, go, p);
+        if (closure == 0) launch_pdl(step_kernel<S, C, 0, 1, R2>, grid, block, 0, st, fi, gi, fo, go, p);
+        else launch_pdl(step_kernel<S, C, 1, 1, R2>, grid, block, 0, st, fi, gi, fo, go, p);
     }
 }
 

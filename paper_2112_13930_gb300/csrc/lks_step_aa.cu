@@ -5,11 +5,13 @@
 #include "lks_aa.cuh"
 #include "lks_internal.h"
 #include "lks_packed.cuh"
+#include "lks_pdl.cuh"
 
 namespace lks {
 
 template <typename S, typename C, int CLOSURE, int COUPLING, int PHASE, bool ROWS2D>
 __global__ void __launch_bounds__(256) step_kernel_aa(S* fb, S* gb, const StepParams<C> p) {
+    pdl_wait();
     int i, j;
     if (ROWS2D) {
         i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -39,6 +41,7 @@ __global__ void __launch_bounds__(256) step_kernel_aa(S* fb, S* gb, const StepPa
 template <typename S, int CLOSURE, int COUPLING, int PHASE, bool ROWS2D>
 __global__ void __launch_bounds__(256, (CLOSURE == 0 || PHASE == 0) ? 3 : 4) step_kernel_aa_pair(S* fb, S* gb, const StepParams<float> p) {
     typedef Packed<S> P;
+    pdl_wait();
     const int H = p.nx >> 1;
     const int64_t NP = p.N >> 1;
     int j, w;
@@ -230,11 +233,11 @@ template <typename S, typename C, int PHASE, bool R2>
 static void launch_aa_grid(S* f, S* g, const StepParams<C>& p, int closure, dim3 grid, unsigned block,
                            cudaStream_t st) {
     if (p.coupling == 0) {
-        if (closure == 0) step_kernel_aa<S, C, 0, 0, PHASE, R2><<<grid, block, 0, st>>>(f, g, p);
-        else step_kernel_aa<S, C, 1, 0, PHASE, R2><<<grid, block, 0, st>>>(f, g, p);
+        if (closure == 0) launch_pdl(step_kernel_aa<S, C, 0, 0, PHASE, R2>, grid, block, 0, st, f, g, p);
+        else launch_pdl(step_kernel_aa<S, C, 1, 0, PHASE, R2>, grid, block, 0, st, f, g, p);
     } else {
-        if (closure == 0) step_kernel_aa<S, C, 0, 1, PHASE, R2><<<grid, block, 0, st>>>(f, g, p);
-        else step_kernel_aa<S, C, 1, 1, PHASE, R2><<<grid, block, 0, st>>>(f, g, p);
+        if (closure == 0) launch_pdl(step_kernel_aa<S, C, 0, 1, PHASE, R2>, grid, block, 0, st, f, g, p);
+        else launch_pdl(step_kernel_aa<S, C, 1, 1, PHASE, R2>, grid, block, 0, st, f, g, p);
     }
 }
 
@@ -256,11 +259,11 @@ static cudaError_t launch_aa_typed(void* f, void* g, const StepParams<C>& p, int
 template <typename S, int PHASE, bool R2>
 static void launch_aa_pair_grid(S* f, S* g, const StepParams<float>& p, int closure, dim3 grid, cudaStream_t st) {
     if (p.coupling == 0) {
-        if (closure == 0) step_kernel_aa_pair<S, 0, 0, PHASE, R2><<<grid, 256, 0, st>>>(f, g, p);
-        else step_kernel_aa_pair<S, 1, 0, PHASE, R2><<<grid, 256, 0, st>>>(f, g, p);
+        if (closure == 0) launch_pdl(step_kernel_aa_pair<S, 0, 0, PHASE, R2>, grid, 256, 0, st, f, g, p);
+        else launch_pdl(step_kernel_aa_pair<S, 1, 0, PHASE, R2>, grid, 256, 0, st, f, g, p);
     } else {
-        if (closure == 0) step_kernel_aa_pair<S, 0, 1, PHASE, R2><<<grid, 256, 0, st>>>(f, g, p);
-        else step_kernel_aa_pair<S, 1, 1, PHASE, R2><<<grid, 256, 0, st>>>(f, g, p);
+        if (closure == 0) launch_pdl(step_kernel_aa_pair<S, 0, 1, PHASE, R2>, grid, 256, 0, st, f, g, p);
+        else launch_pdl(step_kernel_aa_pair<S, 1, 1, PHASE, R2>, grid, 256, 0, st, f, g, p);
     }
 }
 

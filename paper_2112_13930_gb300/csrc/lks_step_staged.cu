@@ -35,6 +35,7 @@
 #include "lks_internal.h"
 #include "lks_packed.cuh"
 #include "lks_pair.cuh"
+#include "lks_pdl.cuh"
 
 namespace lks {
 namespace {
@@ -87,6 +88,7 @@ __global__ void __launch_bounds__(kThreads, 1) step_kernel_staged(const S* __res
         }
         mbar_init_fence();
     }
+    pdl_wait();
     __syncthreads();
 
     if (warp == kConsumerWarps) {  // producer: lane k < 19 fetches slot k
@@ -279,6 +281,7 @@ __global__ void __launch_bounds__(kThreads, 1) step_kernel_aa_staged(S* __restri
         }
         mbar_init_fence();
     }
+    pdl_wait();
     __syncthreads();
 
     if (warp == kConsumerWarps) {  // producer: lane k < 19 fetches slot k
@@ -508,11 +511,11 @@ void launch_typed_aa_staged(void* f, void* g, const StepParams<float>& p, int cl
     S* fb = (S*)f;
     S* gb = (S*)g;
     if (p.coupling == 0) {
-        if (closure == 0) step_kernel_aa_staged<S, 0, 0><<<grid, kThreads, kSmemTB, st>>>(fb, gb, p, ss.err);
-        else step_kernel_aa_staged<S, 1, 0><<<grid, kThreads, kSmemTB, st>>>(fb, gb, p, ss.err);
+        if (closure == 0) launch_pdl(step_kernel_aa_staged<S, 0, 0>, grid, kThreads, kSmemTB, st, fb, gb, p, ss.err);
+        else launch_pdl(step_kernel_aa_staged<S, 1, 0>, grid, kThreads, kSmemTB, st, fb, gb, p, ss.err);
     } else {
-        if (closure == 0) step_kernel_aa_staged<S, 0, 1><<<grid, kThreads, kSmemTB, st>>>(fb, gb, p, ss.err);
-        else step_kernel_aa_staged<S, 1, 1><<<grid, kThreads, kSmemTB, st>>>(fb, gb, p, ss.err);
+        if (closure == 0) launch_pdl(step_kernel_aa_staged<S, 0, 1>, grid, kThreads, kSmemTB, st, fb, gb, p, ss.err);
+        else launch_pdl(step_kernel_aa_staged<S, 1, 1>, grid, kThreads, kSmemTB, st, fb, gb, p, ss.err);
     }
 }
 
@@ -526,11 +529,11 @@ void launch_typed_staged(const void* fin, const void* gin, void* fout, void* gou
     S* fo = (S*)fout;
     S* go = (S*)gout;
     if (p.coupling == 0) {
-        if (closure == 0) step_kernel_staged<S, 0, 0><<<grid, kThreads, kSmemTB, st>>>(fi, gi, fo, go, p, ss.err);
-        else step_kernel_staged<S, 1, 0><<<grid, kThreads, kSmemTB, st>>>(fi, gi, fo, go, p, ss.err);
+        if (closure == 0) launch_pdl(step_kernel_staged<S, 0, 0>, grid, kThreads, kSmemTB, st, fi, gi, fo, go, p, ss.err);
+        else launch_pdl(step_kernel_staged<S, 1, 0>, grid, kThreads, kSmemTB, st, fi, gi, fo, go, p, ss.err);
     } else {
-        if (closure == 0) step_kernel_staged<S, 0, 1><<<grid, kThreads, kSmemTB, st>>>(fi, gi, fo, go, p, ss.err);
-        else step_kernel_staged<S, 1, 1><<<grid, kThreads, kSmemTB, st>>>(fi, gi, fo, go, p, ss.err);
+        if (closure == 0) launch_pdl(step_kernel_staged<S, 0, 1>, grid, kThreads, kSmemTB, st, fi, gi, fo, go, p, ss.err);
+        else launch_pdl(step_kernel_staged<S, 1, 1>, grid, kThreads, kSmemTB, st, fi, gi, fo, go, p, ss.err);
     }
 }
 
