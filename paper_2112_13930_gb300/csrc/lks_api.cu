@@ -28,6 +28,9 @@ thread_local std::string g_last_error = "";
 // fused kernel applies (the n % kRowSteps steps left over are then launched one by one).
 constexpr int kGraphSizes = 6;
 constexpr int64_t kGraphLaunches[kGraphSizes] = {64, 32, 16, 8, 4, 2};
+// Most steps of one launch of a resident lattice (even, so that it returns to the buffer it started in): a
+// tenth of a second at the most.
+constexpr int64_t kResidentSteps = 16384;
 constexpr size_t kAlign = 256;
 
 inline size_t align_up(size_t x) { return (x + kAlign - 1) & ~(kAlign - 1); }
@@ -203,6 +206,7 @@ struct lks_handle {
     int* flag = nullptr;
     bool staged = false;              // 16-bit, nx % 8 == 0, nx >= 1024: the staged kernels
     lks::StagedStep ss = {nullptr, 0};
+    lks::ResidentPlan resident = {0, 0, 0, 0, 0};  // ctas > 0: all steps of a call in one launch
     lks::RowsPlan rows = {0, 0, 0};     // strip > 0: kRowSteps steps per launch
     double c_bot = 0.0, c_top = 0.0, u_bot = 0.0, u_top = 0.0;
     StepParams<double> sp;
@@ -424,7 +428,8 @@ lks_status lks_create(const lks_params* p, lks_handle** out) {
         h->ss.err = h->flag;
         h->staged = e == cudaSuccess;
     }
-    if (e == cudaSuccess && !p->inplace)
+    if (e == cudaSuccess) e = lks::plan_resident(p->storage, p->closure, p->coupling, p->nx, p->ny, &h->resident);
+    if (e == cudaSuccess && !p->inplace && !h->resident.ctas)
         e = lks::plan_rows(p->storage, p->closure, p->coupling, p->nx, p->ny, &h->rows);
     if (e != cudaSuccess) {
         lks_destroy(h);
@@ -462,6 +467,17 @@ lks_status lks_step(lks_handle* h, int64_t n) {
     if (!h) return fail(nullptr, LKS_EINVAL, "handle is NULL");
     if (n < 0) return fail(h, LKS_EINVAL, "n must be >= 0");
     if (h->p.inplace && (n & 1)) return fail(h, LKS_EINVAL, "an in-place handle steps in pairs: n must be even");
+    while (h->resident.ctas && n > 1) {
+        const int64_t k = n < kResidentSteps ? n : kResidentSteps;
+        const int to = h->p.inplace ? 0 : (int)(h->cur ^ (k & 1));
+        const int from = h->p.inplace ? 0 : h->cur;
+        cudaError_t e = lks::launch_resident(h->p.storage, h->p.closure, h->f[from], h->g[from], h->f[to], h->g[to],
+                                             h->sp, h->resident, ilv_of(h), (int)k, h->stream);
+        if (e != cudaSuccess) return cuda_fail(h, e, "step kernel launch");
+        h->cur ^= (int)(k & 1);
+        h->steps += k;
+        n -= k;
+    }
     const int64_t per = launch_steps(h);
     int64_t left = n / per;  // launches of `per` steps
     for (int g = 0; g < kGraphSizes && !h->graphs_disabled; ++g) {

@@ -110,6 +110,23 @@ cudaError_t plan_rows(int storage, int closure, int coupling, int nx, int ny, Ro
 cudaError_t launch_rows(int storage, int closure, const void* fin, const void* gin, void* fout, void* gout,
                         const StepParams<double>& pd, const RowsPlan& rp, cudaStream_t st);
 
+// Small lattices held in one cluster's shared memory for all steps of a call (lks_resident.cu).  ctas: 0
+// where it does not apply.  fin / fout: the buffers before and after `steps` steps (they may be the same);
+// ilv as interleave_row.
+constexpr int kResidentThreads = 512;
+// Most nodes: the lattice then has 16 SMs, so that above these single steps on all SMs are faster (us a step,
+// resident against single: FP32 64 x 128 1.36 / 1.41, 64 x 190 1.81 / 1.46; FP16 100 x 100 1.99 / 2.53; FP64 from
+// 129 nodes a CTA on two warps share a sub-partition).
+constexpr int64_t kResidentNodesF64 = 2048, kResidentNodesF32 = 8192, kResidentNodes16 = 12288;
+constexpr int kResidentQuads = 2;  // groups of 32 nodes a CTA, four warps each (FP64, Maxwell coupling)
+struct ResidentPlan {
+    int ctas, threads, rows_max, quads;
+    size_t smem;
+};
+cudaError_t plan_resident(int storage, int closure, int coupling, int nx, int ny, ResidentPlan* rp);
+cudaError_t launch_resident(int storage, int closure, const void* fin, const void* gin, void* fout, void* gout,
+                            const StepParams<double>& pd, const ResidentPlan& rp, int ilv, int steps, cudaStream_t st);
+
 // Initial equilibrium state (deviation form) with the counter-based perturbation.
 cudaError_t launch_init(int storage, void* f, void* g, int nx, int ny, double B0, uint64_t seed, double amp,
                         cudaStream_t st, int ilv = 0);
