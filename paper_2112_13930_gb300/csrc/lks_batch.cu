@@ -13,6 +13,7 @@
 #include <math.h>
 #include <string.h>
 
+#include <algorithm>
 #include <map>
 #include <new>
 #include <string>
@@ -23,12 +24,14 @@
 #include "../../include/lks_batch.h"
 #include "lks_aa.cuh"
 #include "lks_internal.h"
+#include "lks_resident.cuh"
 
 using lks::StepParams;
 
 namespace {
 
 constexpr size_t kAlign = 256;
+constexpr size_t kMaxBand = 208 * 1024;  // most dynamic shared memory of a resident kernel's CTA
 constexpr int kMaxGroups = 15;  // named barriers 1..15 (0 is __syncthreads)
 // An instance is declared STALLED when its residual has not reached a new minimum for kStallChecks
 // checks in a row while already below the rounding floor of the storage type (lks::stall_floor), or
@@ -279,6 +282,85 @@ template <> struct CgLoader<__half, float> {
     }
 };
 
+// What the CTAs of a cluster share: work pick, status, residual partials.
+struct ClusterShared {
+    int32_t pick, flag;
+    double cpart[4 * 8];
+};
+
+// The residual check of an instance in cluster mode: thread t < T of CTA r takes nodes r*T + t,
+// r*T + t + CS*T, ... of the state in global memory; r, best and stall live in CTA 0's
+// thread 0.  Returns the instance's status.
+template <typename S, typename C, int COUPLING>
+__device__ __forceinline__ int cluster_check(InstDev* I, int64_t N, int cur, int64_t steps, double* red,
+                                             ClusterShared* sh, int T, double& r, double& best, int& stall) {
+    cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+    const int CS = (int)cl.num_blocks(), rank = (int)cl.block_rank(), lt = threadIdx.x;
+    const int64_t first = (int64_t)rank * T + lt, stride = (int64_t)CS * T, max_steps = I->max_steps;
+    int32_t& flag = sh->flag;
+    double* cpart = sh->cpart;
+    int32_t* flag0 = cl.map_shared_rank(&sh->flag, 0);
+    double* cpart0 = cl.map_shared_rank(sh->cpart, 0);
+    double acc[4] = {0.0, 0.0, 0.0, 0.0};
+    const S* fc = (const S*)I->f[cur];
+    const S* gc = (const S*)I->g[cur];
+    double* snap = I->snap;
+    for (int64_t n = first; n < N && lt < T; n += stride) {
+        double ux, bx;
+        stored_ux_bx<S, C, CgLoader<S, C>, COUPLING>(fc, gc, N, n, I, ux, bx);
+        const double du = ux - snap[n], db = bx - snap[N + n];
+        acc[0] = lks::ffma(du, du, acc[0]);
+        acc[1] = lks::ffma(ux, ux, acc[1]);
+        acc[2] = lks::ffma(db, db, acc[2]);
+        acc[3] = lks::ffma(bx, bx, acc[3]);
+        snap[n] = ux;
+        snap[N + n] = bx;
+    }
+    lks::warp_sum<4>(acc);
+    const int W = T >> 5;
+    if ((lt & 31) == 0 && lt < T)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) red[k * W + (lt >> 5)] = acc[k];
+    __syncthreads();
+    if (lt == 0)
+        for (int k = 0; k < 4; ++k) {
+            double t = red[k * W];
+            for (int q = 1; q < W; ++q) t += red[k * W + q];
+            cpart0[4 * rank + k] = t;
+        }
+    cl.sync();
+    if (rank == 0 && lt == 0) {
+        double t[4] = {0.0, 0.0, 0.0, 0.0};
+        for (int q = 0; q < CS; ++q)
+            for (int k = 0; k < 4; ++k) t[k] += cpart[4 * q + k];
+        const double ru = t[1] > 1e-60 ? sqrt(t[0] / t[1]) : 0.0;
+        const double rb = t[3] > 1e-60 ? sqrt(t[2] / t[3]) : 0.0;
+        r = ru > rb ? ru : rb;
+        int st = LKS_INST_RUNNING;
+        if (!isfinite(r) || !isfinite(t[1]) || !isfinite(t[3])) {
+            st = LKS_INST_UNSTABLE;
+        } else if (r == 0.0 && sizeof(S) < 8 &&
+                   (I->pd.Fx != 0.0 || I->pd.bot.U != 0.0 || I->pd.top.U != 0.0)) {
+            st = LKS_INST_STALLED;  // a driven channel that stopped changing (zero_residual_is_stall)
+        } else if (r < I->tol) {
+            st = LKS_INST_CONVERGED;
+        } else {
+            if (r < best) {
+                best = r;
+                stall = 0;
+            } else if (++stall >= kStallChecks && best < I->stall_below) {
+                st = LKS_INST_STALLED;
+            }
+            if (st == LKS_INST_RUNNING && steps >= max_steps) st = LKS_INST_MAX_STEPS;
+        }
+        flag = st;
+    }
+    cl.sync();
+    // CTA 0 writes `flag` again only at the next check, after at least one more
+    // cluster barrier, and leaves the kernel only after the next pick's barriers.
+    return *flag0;
+}
+
 // Cluster mode: the CS CTAs of one thread-block cluster (on CS SMs) work on one instance together,
 // CTA r updating nodes r*T + t, r*T + t + CS*T, ...; one cluster barrier (release/acquire at cluster
 // scope) separates the steps, and the residual partials of the CTAs are summed by CTA 0 in rank
@@ -290,20 +372,17 @@ __global__ void __launch_bounds__(512) batch_cluster_kernel(InstDev* tab, const 
     namespace cg = cooperative_groups;
     cg::cluster_group cl = cg::this_cluster();
     extern __shared__ double red[];
-    __shared__ int32_t pick;
-    __shared__ int32_t flag;
-    __shared__ double cpart[4 * 8];
+    __shared__ ClusterShared shared;
+    ClusterShared* sh = &shared;
     const int CS = (int)cl.num_blocks();
     const int rank = (int)cl.block_rank();
     const int lt = threadIdx.x;
     const int nwork = ctl->nwork;
     const int64_t quantum = ctl->quantum;
-    int32_t* pick0 = cl.map_shared_rank(&pick, 0);
-    int32_t* flag0 = cl.map_shared_rank(&flag, 0);
-    double* cpart0 = cl.map_shared_rank(cpart, 0);
+    int32_t* pick0 = cl.map_shared_rank(&sh->pick, 0);
     const int64_t stride = (int64_t)CS * T;
     for (;;) {
-        if (rank == 0 && lt == 0) pick = atomicAdd(counter, 1);
+        if (rank == 0 && lt == 0) sh->pick = atomicAdd(counter, 1);
         cl.sync();
         const int w = *pick0;
         // Every CTA must have read CTA 0's shared `pick` before CTA 0 can overwrite it or exit
@@ -360,67 +439,101 @@ __global__ void __launch_bounds__(512) batch_cluster_kernel(InstDev* tab, const 
             ++steps;
             cl.sync();
             if (steps % check_every == 0 || steps >= max_steps) {
-                double acc[4] = {0.0, 0.0, 0.0, 0.0};
-                const S* fc = (const S*)I->f[cur];
-                const S* gc = (const S*)I->g[cur];
-                double* snap = I->snap;
-                for (int64_t n = first; n < N; n += stride) {
-                    double ux, bx;
-                    stored_ux_bx<S, C, CgLoader<S, C>, COUPLING>(fc, gc, N, n, I, ux, bx);
-                    const double du = ux - snap[n], db = bx - snap[N + n];
-                    acc[0] = lks::ffma(du, du, acc[0]);
-                    acc[1] = lks::ffma(ux, ux, acc[1]);
-                    acc[2] = lks::ffma(db, db, acc[2]);
-                    acc[3] = lks::ffma(bx, bx, acc[3]);
-                    snap[n] = ux;
-                    snap[N + n] = bx;
-                }
-                lks::warp_sum<4>(acc);
-                const int W = T >> 5;
-                if ((lt & 31) == 0)
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) red[k * W + (lt >> 5)] = acc[k];
-                __syncthreads();
-                if (lt == 0)
-                    for (int k = 0; k < 4; ++k) {
-                        double t = red[k * W];
-                        for (int q = 1; q < W; ++q) t += red[k * W + q];
-                        cpart0[4 * rank + k] = t;
-                    }
-                cl.sync();
-                if (rank == 0 && lt == 0) {
-                    double t[4] = {0.0, 0.0, 0.0, 0.0};
-                    for (int q = 0; q < CS; ++q)
-                        for (int k = 0; k < 4; ++k) t[k] += cpart[4 * q + k];
-                    const double ru = t[1] > 1e-60 ? sqrt(t[0] / t[1]) : 0.0;
-                    const double rb = t[3] > 1e-60 ? sqrt(t[2] / t[3]) : 0.0;
-                    r = ru > rb ? ru : rb;
-                    int st = LKS_INST_RUNNING;
-                    if (!isfinite(r) || !isfinite(t[1]) || !isfinite(t[3])) {
-                        st = LKS_INST_UNSTABLE;
-                    } else if (r == 0.0 && sizeof(S) < 8 &&
-                               (I->pd.Fx != 0.0 || I->pd.bot.U != 0.0 || I->pd.top.U != 0.0)) {
-                        st = LKS_INST_STALLED;  // a driven channel that stopped changing (zero_residual_is_stall)
-                    } else if (r < I->tol) {
-                        st = LKS_INST_CONVERGED;
-                    } else {
-                        if (r < best) {
-                            best = r;
-                            stall = 0;
-                        } else if (++stall >= kStallChecks && best < I->stall_below) {
-                            st = LKS_INST_STALLED;
-                        }
-                        if (st == LKS_INST_RUNNING && steps >= max_steps) st = LKS_INST_MAX_STEPS;
-                    }
-                    flag = st;
-                }
-                cl.sync();
-                // CTA 0 writes `flag` again only at the next check, after at least one more
-                // cluster barrier, and leaves the kernel only after the next pick's barriers.
-                state = *flag0;
+                state = cluster_check<S, C, COUPLING>(I, N, cur, steps, red, sh, T, r, best, stall);
                 if (state != LKS_INST_RUNNING) break;
             }
         }
+        if (rank == 0 && lt == 0) {
+            I->cur = cur;
+            I->steps = steps;
+            I->state = state;
+            I->residual = r;
+            I->best_r = best;
+            I->stall = stall;
+            res[slot].state = state;
+            res[slot].cur = cur;
+            res[slot].steps = steps;
+            res[slot].residual = r;
+        }
+        cl.sync();
+    }
+}
+
+// Shared memory of a resident cluster kernel's CTA: the residual's warp sums, then the instance's band.
+inline size_t red_bytes(int T) { return (size_t)4 * (T / 32) * sizeof(double); }
+// Bytes a CTA needs to hold its band of an nx x ny instance on a cluster of CS; 0: some CTA would have no row.
+inline size_t band_bytes(int nx, int ny, size_t sb, int CS) {
+    return ny < CS ? 0 : 2 * 19 * (size_t)nx * ((ny + CS - 1) / CS + 2) * sb;
+}
+
+// Cluster mode with every instance of the work list held in its cluster's shared memory for the launch
+// (lks_resident.cuh; FP32 and 16-bit storage): a step then costs a cluster barrier and shared-memory
+// latency instead of L2 round trips (forty FP32 instances of 4 x 33 .. 257 on clusters of 8: 2.4 -> 1.4 us a
+// step).  A check stores the bands first and reads the state as the other
+// cluster kernel does, so that the residual's summation order, and with it every bit, is the same.
+// The instance's parameters stay in shared memory: as 27 registers a thread they spilled.
+template <typename S, typename C, int COUPLING, bool INPLACE>
+__global__ void __launch_bounds__(512) batch_resident_kernel(InstDev* tab, const int32_t* work, const Ctl* ctl,
+                                                              int32_t* counter, ResultDev* res, int T) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    extern __shared__ double red[];
+    __shared__ ClusterShared shared;
+    __shared__ StepParams<C> q;
+    ClusterShared* sh = &shared;
+    const int CS = (int)cl.num_blocks();
+    const int rank = (int)cl.block_rank();
+    const int lt = threadIdx.x;
+    const int nwork = ctl->nwork;
+    const int64_t quantum = ctl->quantum;
+    int32_t* pick0 = cl.map_shared_rank(&sh->pick, 0);
+    for (;;) {
+        if (rank == 0 && lt == 0) sh->pick = atomicAdd(counter, 1);
+        cl.sync();
+        const int w = *pick0;
+        cl.sync();  // as in batch_cluster_kernel
+        if (w >= nwork) break;
+        const int slot = work[w];
+        InstDev* I = tab + slot;
+        const int64_t N = I->pd.N;
+        const int closure = I->closure, nx = I->pd.nx, ny = I->pd.ny;
+        const int64_t check_every = I->check_every, max_steps = I->max_steps;
+        int cur = I->cur;
+        int64_t steps = I->steps;
+        int state = LKS_INST_RUNNING;
+        double r = I->residual, best = I->best_r;
+        int stall = I->stall;
+        lks::Band<S> band;
+        band.set(reinterpret_cast<S*>(red + 4 * (T >> 5)), nx, ny, (ny + CS - 1) / CS);
+        band.load((const S*)I->f[cur], (const S*)I->g[cur], N, ny, 0);
+        if (lt == 0) {
+            q = to_compute<C>(I->pd);
+            q.N = band.plane;
+        }
+        cl.sync();
+        int b = 0;
+        bool stored = true;  // the state in global memory is the current one
+        int64_t to_check = check_every - steps % check_every;
+        for (int64_t s = 0; s < quantum; ++s) {
+            if (closure == 0)
+                lks::band_step<S, C, 0, COUPLING>(band, b, q);
+            else
+                lks::band_step<S, C, 1, COUPLING>(band, b, q);
+            b ^= 1;
+            if (!INPLACE) cur ^= 1;
+            ++steps;
+            stored = false;
+            cl.sync();
+            if (--to_check == 0 || steps >= max_steps) {
+                if (to_check == 0) to_check = check_every;
+                band.store(b, (S*)I->f[cur], (S*)I->g[cur], N, 0);
+                stored = true;
+                cl.sync();
+                state = cluster_check<S, C, COUPLING>(I, N, cur, steps, red, sh, T, r, best, stall);
+                if (state != LKS_INST_RUNNING) break;
+            }
+        }
+        if (!stored) band.store(b, (S*)I->f[cur], (S*)I->g[cur], N, 0);
         if (rank == 0 && lt == 0) {
             I->cur = cur;
             I->steps = steps;
@@ -449,7 +562,22 @@ BatchClusterFn cluster_kernel_typed(int storage) {
     }
 }
 
-BatchClusterFn cluster_kernel_for(const lks_batch_config& c) {
+template <int COUPLING, bool INPLACE>
+BatchClusterFn resident_kernel_typed(int storage) {
+    switch (storage) {
+        case 1: return batch_resident_kernel<float, float, COUPLING, INPLACE>;
+        case 2: return batch_resident_kernel<__nv_bfloat16, float, COUPLING, INPLACE>;
+        default: return batch_resident_kernel<__half, float, COUPLING, INPLACE>;
+    }
+}
+
+// band_cap > 0: the kernel that keeps the instances in shared memory (not for FP64 storage).
+BatchClusterFn cluster_kernel_for(const lks_batch_config& c, size_t band_cap) {
+    if (band_cap) {
+        if (c.coupling == 1)
+            return c.inplace ? resident_kernel_typed<1, true>(c.storage) : resident_kernel_typed<1, false>(c.storage);
+        return c.inplace ? resident_kernel_typed<0, true>(c.storage) : resident_kernel_typed<0, false>(c.storage);
+    }
     if (c.coupling == 1) return c.inplace ? cluster_kernel_typed<1, true>(c.storage) : cluster_kernel_typed<1, false>(c.storage);
     return c.inplace ? cluster_kernel_typed<0, true>(c.storage) : cluster_kernel_typed<0, false>(c.storage);
 }
@@ -535,6 +663,8 @@ struct lks_batch {
     int T = 256, G = 1, CS = 1;
     cudaGraphExec_t graph = nullptr;
     int graph_T = 0, graph_G = 0, graph_CS = 0;
+    size_t band_cap = 0, graph_band_cap = 0;  // shared memory for a resident instance's band; 0: not resident
+    int band_threads = 0, graph_band_threads = 0;
     std::string err;
 };
 
@@ -597,7 +727,7 @@ int blocks_per_sm(lks_batch* b, int T, int G) {
 
 cudaError_t enqueue_launch(lks_batch* b, cudaStream_t st) {
     const int T = b->T, G = b->G, CS = b->CS;
-    const size_t smem = (size_t)G * 4 * (T / 32) * sizeof(double);
+    const size_t smem = G * red_bytes(T) + b->band_cap;
     cudaError_t e = cudaMemsetAsync(b->d_counter, 0, sizeof(int32_t), st);
     if (e != cudaSuccess) return e;
     if (CS == 1) {
@@ -611,18 +741,18 @@ cudaError_t enqueue_launch(lks_batch* b, cudaStream_t st) {
         attr[0].val.clusterDim.x = CS;
         attr[0].val.clusterDim.y = 1;
         attr[0].val.clusterDim.z = 1;
-        lc.blockDim = dim3(T);
+        lc.blockDim = dim3(b->band_cap ? b->band_threads : T);
         lc.dynamicSmemBytes = smem;
         lc.stream = st;
         lc.attrs = attr;
         lc.numAttrs = 1;
         lc.gridDim = dim3(CS * b->nsm);
         int clusters = 0;
-        e = cudaOccupancyMaxActiveClusters(&clusters, cluster_kernel_for(b->cfg), &lc);
+        e = cudaOccupancyMaxActiveClusters(&clusters, cluster_kernel_for(b->cfg, b->band_cap), &lc);
         if (e != cudaSuccess) return e;
         if (clusters < 1) clusters = 1;
         lc.gridDim = dim3(clusters * CS);
-        e = cudaLaunchKernelEx(&lc, cluster_kernel_for(b->cfg), b->d_tab, (const int32_t*)b->d_work,
+        e = cudaLaunchKernelEx(&lc, cluster_kernel_for(b->cfg, b->band_cap), b->d_tab, (const int32_t*)b->d_work,
                                (const Ctl*)b->d_ctl, b->d_counter, b->d_res, T);
         if (e != cudaSuccess) return e;
     }
@@ -632,7 +762,9 @@ cudaError_t enqueue_launch(lks_batch* b, cudaStream_t st) {
 }
 
 cudaError_t ensure_graph(lks_batch* b) {
-    if (b->graph && b->graph_T == b->T && b->graph_G == b->G && b->graph_CS == b->CS) return cudaSuccess;
+    if (b->graph && b->graph_T == b->T && b->graph_G == b->G && b->graph_CS == b->CS &&
+        b->graph_band_cap == b->band_cap && b->graph_band_threads == b->band_threads)
+        return cudaSuccess;
     if (b->graph) {
         cudaGraphExecDestroy(b->graph);
         b->graph = nullptr;
@@ -641,6 +773,11 @@ cudaError_t ensure_graph(lks_batch* b) {
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(kernel_for(b->cfg), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)smem);
+        if (e != cudaSuccess) return e;
+    }
+    if (b->band_cap) {  // the limit is the function's, shared by every batch: always the same value
+        cudaError_t e = cudaFuncSetAttribute(cluster_kernel_for(b->cfg, b->band_cap),
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxBand);
         if (e != cudaSuccess) return e;
     }
     cudaGraph_t g = nullptr;
@@ -659,8 +796,36 @@ cudaError_t ensure_graph(lks_batch* b) {
         b->graph_T = b->T;
         b->graph_G = b->G;
         b->graph_CS = b->CS;
+        b->graph_band_cap = b->band_cap;
+        b->graph_band_threads = b->band_threads;
     }
     return e;
+}
+
+// Shared memory per CTA for the resident kernel: what the largest instance of the work list needs, if that
+// leaves all its clusters running at once (an SM has 227 KB for its CTAs); 0 otherwise, for one CTA per
+// instance and for FP64, which the FP64 pipe bounds either way.  Rounded up, so that few graphs are built.
+// Threads: one per node of the largest band while the blocks that share an SM fit its registers, at least
+// the T that a check uses.
+void choose_band(lks_batch* b, int nwork) {
+    b->band_cap = 0;
+    b->band_threads = 0;
+    if (b->CS == 1 || b->cfg.storage == 0) return;
+    const size_t sb = lks::storage_bytes(b->cfg.storage);
+    const size_t per_sm = ((size_t)nwork * b->CS + b->nsm - 1) / b->nsm;
+    size_t most = 0;
+    int nodes = 0;
+    for (int k = 0; k < nwork; ++k) {
+        const Slot& s = b->slots[b->h_work[k]];
+        const size_t need = band_bytes(s.nx, s.ny, sb, b->CS);
+        if (need == 0) return;
+        most = std::max(most, need);
+        nodes = std::max(nodes, (s.ny + b->CS - 1) / b->CS * s.nx);
+    }
+    most = (most + 8191) / 8192 * 8192;
+    if (red_bytes(b->T) + most > kMaxBand || per_sm * (most + red_bytes(b->T) + 2048) > 226 * 1024) return;
+    b->band_cap = most;
+    b->band_threads = std::max(b->T, (std::min(nodes, (int)(512 / per_sm)) + 31) / 32 * 32);
 }
 
 }  // namespace
@@ -841,6 +1006,7 @@ lks_status lks_batch_run(lks_batch* b, int64_t quantum, int32_t* n_running) {
         b->h_ctl->nwork = nwork;
         b->h_ctl->pad = 0;
         b->h_ctl->quantum = quantum;
+        choose_band(b, nwork);
         cudaError_t e = ensure_graph(b);
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(b->d_work, b->h_work, nwork * sizeof(int32_t), cudaMemcpyHostToDevice, b->stream);
