@@ -557,7 +557,8 @@ __global__ void __launch_bounds__(256) step3_kernel(const S* fin, const S* gin, 
 
 // One node per thread over the flattened node index n = (z ny + y) nx + x, so that a warp covers
 // consecutive nodes (coalesced) whatever nx is: the duct (SIDE; a fully developed duct flow has
-// nx = 1), and the FP64 channel, whose blocks are small (lks::block_f64).
+// nx = 1), channels whose rows would leave a third of their threads idle, and the FP64 channel, whose
+// blocks are small (lks::block_f64).
 template <typename S, typename C, bool SIDE>
 __global__ void __launch_bounds__(256) step3_flat_kernel(const S* fin, const S* gin, S* fout, S* gout,
                                                          const Params3<C> p) {
@@ -1023,7 +1024,7 @@ void launch_staged3(lks3_handle* h, int src, cudaStream_t st) {
     const int64_t ntask = (int64_t)p.nz * ((p.ny + R - 1) / R);
     const unsigned grid = (unsigned)std::min<int64_t>(ntask, h->staged_grid);
     const Params3<float> q = make_params3<float>(p, h->c_bot, h->c_top, h->u_bot, h->u_top);
-    lks::launch_pdl(step3_staged_kernel<S>, grid, kThreads3, staged_smem3(), st, 
+    lks::launch_pdl(step3_staged_kernel<S>, grid, kThreads3, staged_smem3(), st,
         (const S*)h->f[src], (const S*)h->g[src], (S*)h->f[src ^ 1], (S*)h->g[src ^ 1], q, R, h->flag);
 }
 
@@ -1053,14 +1054,13 @@ cudaError_t prepare_staged3(lks3_handle* h) {
 
 cudaError_t launch_step3(lks3_handle* h, int src, cudaStream_t st) {
     const lks3_params& p = h->p;
-    const dim3 grid((p.nx + 255) / 256, p.ny, p.nz);
     if (h->side) {
         const int64_t N = (int64_t)p.nx * p.ny * p.nz;
         LKS3_DISPATCH(p.storage, {
             const Params3<C> q = make_params3<C>(p, h->c_bot, h->c_top, h->u_bot, h->u_top, h->c_back, h->c_front);
-            const unsigned block = sizeof(C) == 8 ? lks::block_f64(N) : 256;
-            lks::launch_pdl(step3_flat_kernel<S, C, true>, dim3((unsigned)((N + block - 1) / block)), block, 0, st, 
-                (const S*)h->f[src], (const S*)h->g[src], (S*)h->f[src ^ 1], (S*)h->g[src ^ 1], q);
+            const unsigned block = sizeof(C) == 8 ? lks::block_f64(N) : lks::block_f32(N, 1);
+            lks::launch_pdl(step3_flat_kernel<S, C, true>, dim3((unsigned)((N + block - 1) / block)), block, 0, st,
+                            (const S*)h->f[src], (const S*)h->g[src], (S*)h->f[src ^ 1], (S*)h->g[src ^ 1], q);
         });
         return cudaGetLastError();
     }
@@ -1077,12 +1077,19 @@ cudaError_t launch_step3(lks3_handle* h, int src, cudaStream_t st) {
         const S* gi = (const S*)h->g[src];
         S* fo = (S*)h->f[src ^ 1];
         S* go = (S*)h->g[src ^ 1];
-        if constexpr (sizeof(C) == 8) {
-            const unsigned block = lks::block_f64(q.N);
-            lks::launch_pdl(step3_flat_kernel<S, C, false>, dim3((unsigned)((q.N + block - 1) / block)), block, 0, st, fi, gi, fo,
-                                                                                                           go, q);
+        const bool flat = sizeof(C) == 8 || (p.nx + 63) / 64 * 64 * 2 > 3 * p.nx;  // else a grid row per row
+        const unsigned block = sizeof(C) == 8 ? lks::block_f64(q.N)
+                               : flat ? lks::block_f32(q.N, 1)
+                               // large channels run at the HBM rate, idle lanes or not (160 x 129 x 200: 194 us a step
+                               // with 256 threads, 196 with 64)
+                               : q.N >= (int64_t)1 << 21 ? 256u : lks::block_f32(p.nx, (int64_t)p.ny * p.nz);
+        if (flat) {
+            lks::launch_pdl(step3_flat_kernel<S, C, false>, dim3((unsigned)((q.N + block - 1) / block)), block, 0, st, fi,
+                            gi, fo, go, q);
         } else {
-            lks::launch_pdl(step3_kernel<S, C>, grid, 256, 0, st, fi, gi, fo, go, q);
+            if constexpr (sizeof(C) == 4)
+                lks::launch_pdl(step3_kernel<S, C>, dim3((p.nx + block - 1) / block, p.ny, p.nz), block, 0, st, fi, gi, fo,
+                                go, q);
         }
     });
     return cudaGetLastError();

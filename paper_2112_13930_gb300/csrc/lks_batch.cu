@@ -506,10 +506,7 @@ __global__ void __launch_bounds__(512) batch_resident_kernel(InstDev* tab, const
         lks::Band<S> band;
         band.set(reinterpret_cast<S*>(red + 4 * (T >> 5)), nx, ny, (ny + CS - 1) / CS);
         band.load((const S*)I->f[cur], (const S*)I->g[cur], N, ny, 0);
-        if (lt == 0) {
-            q = to_compute<C>(I->pd);
-            q.N = band.plane;
-        }
+        if (lt == 0) q = to_compute<C>(I->pd);
         cl.sync();
         int b = 0;
         bool stored = true;  // the state in global memory is the current one

@@ -57,6 +57,18 @@ StepParams<double> make_step_params(int nx, int ny, int closure, double tau_f, d
 // large lattices take the same time with blocks of 64, 128 and 256.
 inline unsigned block_f64(int64_t N) { return N <= 152 * 64 ? 64 : 128; }
 
+// Threads per block of the FP32 and 16-bit step kernels, for `items` (nodes, or words of two nodes) a row with a
+// grid row to each, or for `items` in one flat row.  256 for large lattices; smaller blocks where they pad a row
+// less, or where 256 would leave SMs without a block (us a step, 256 / 128 / 64 threads: FP16 280 x 447 4.15 / 4.33 /
+// 3.69, 300 x 1200 8.93 / 8.88 / 7.08, BF16 85 x 798 3.75 / 2.63 / 2.82, 126 x 287 2.54 / 2.20 / 2.25, FP32
+// 360 x 360 3.56 / 3.29 / 3.19, 1000 x 513 8.18 / 8.16 / 8.26).
+inline unsigned block_f32(int64_t items, int64_t rows) {
+    auto padded = [&](int64_t b) { return (items + b - 1) / b * b; };
+    const int64_t best = padded(64);
+    if (rows * items >= (int64_t)1 << 21 && padded(256) * 16 <= best * 17) return 256;
+    return padded(128) * 16 > best * 17 || rows * padded(128) / 128 < 4 * 152 ? 64 : 128;
+}
+
 // Bytes per stored population for each lks_storage value.
 inline size_t storage_bytes(int storage) { return storage == 0 ? 8 : (storage == 1 ? 4 : 2); }
 
@@ -113,11 +125,11 @@ cudaError_t launch_rows(int storage, int closure, const void* fin, const void* g
 // Small lattices held in one cluster's shared memory for all steps of a call (lks_resident.cu).  ctas: 0
 // where it does not apply.  fin / fout: the buffers before and after `steps` steps (they may be the same);
 // ilv as interleave_row.
-constexpr int kResidentThreads = 512;
+constexpr int kResidentThreads = 1024;  // FP64: half
 // Most nodes: the lattice then has 16 SMs, so that above these single steps on all SMs are faster (us a step,
-// resident against single: FP32 64 x 128 1.36 / 1.41, 64 x 190 1.81 / 1.46; FP16 100 x 100 1.99 / 2.53; FP64 from
+// resident against single: FP32 64 x 120 1.17 / 1.41, 64 x 190 1.44 / 1.40; BF16 96 x 96 1.41 / 2.2; FP64 from
 // 129 nodes a CTA on two warps share a sub-partition).
-constexpr int64_t kResidentNodesF64 = 2048, kResidentNodesF32 = 8192, kResidentNodes16 = 12288;
+constexpr int64_t kResidentNodesF64 = 2048, kResidentNodesF32 = 10240, kResidentNodes16 = 12288;
 constexpr int kResidentQuads = 2;  // groups of 32 nodes a CTA, four warps each (FP64, Maxwell coupling)
 struct ResidentPlan {
     int ctas, threads, rows_max, quads;

@@ -11,7 +11,7 @@ namespace {
 constexpr size_t kResidentSmem = 200 * 1024;  // most dynamic shared memory of a CTA
 
 template <typename S, typename C, int CLOSURE, int COUPLING>
-__global__ void __launch_bounds__(kResidentThreads) resident_kernel(const S* fin, const S* gin, S* fout, S* gout,
+__global__ void __launch_bounds__(sizeof(C) == 8 ? kResidentThreads / 2 : kResidentThreads) resident_kernel(const S* fin, const S* gin, S* fout, S* gout,
                                                                     const StepParams<C> p, int rows_max, int ilv,
                                                                     int steps) {
     extern __shared__ __align__(16) unsigned char res_sm[];
@@ -19,12 +19,10 @@ __global__ void __launch_bounds__(kResidentThreads) resident_kernel(const S* fin
     Band<S> band;
     band.set(reinterpret_cast<S*>(res_sm), p.nx, p.ny, rows_max);
     band.load(fin, gin, p.N, p.ny, ilv);
-    StepParams<C> q = p;
-    q.N = band.plane;
     cl.sync();  // every band is loaded before anyone stores, and every CTA runs before its memory is written
     int b = 0;
     for (int s = 0; s < steps; ++s, b ^= 1) {
-        band_step<S, C, CLOSURE, COUPLING>(band, b, q);
+        band_step<S, C, CLOSURE, COUPLING>(band, b, p);
         cl.sync();
     }
     band.store(b, fout, gout, p.N, ilv);
@@ -113,7 +111,7 @@ cudaError_t plan_resident(int storage, int closure, int coupling, int nx, int ny
     while (ctas > ny) ctas /= 2;
     rp->rows_max = (ny + ctas - 1) / ctas;
     const int nodes = rp->rows_max * nx;
-    rp->threads = std::min(kResidentThreads, (nodes + 31) / 32 * 32);
+    rp->threads = std::min(storage == 0 ? kResidentThreads / 2 : kResidentThreads, (nodes + 31) / 32 * 32);
     rp->smem = (size_t)2 * 19 * nx * (rp->rows_max + 2) * storage_bytes(storage);
     if (storage == 0 && coupling == 0 && nodes <= 32 * kResidentQuads) {
         rp->quads = (nodes + 31) / 32;

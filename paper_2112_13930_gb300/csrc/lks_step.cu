@@ -189,13 +189,13 @@ static bool rows2d(int row_items, int ny) { return row_items >= 64 && ny <= 6553
 
 template <typename S, bool R2>
 static void launch_pair_grid(const S* fi, const S* gi, S* fo, S* go, const StepParams<float>& p, int closure,
-                             dim3 grid, cudaStream_t st) {
+                             dim3 grid, unsigned block, cudaStream_t st) {
     if (p.coupling == 0) {
-        if (closure == 0) step_kernel_pair<S, 0, 0, R2><<<grid, 256, 0, st>>>(fi, gi, fo, go, p);
-        else step_kernel_pair<S, 1, 0, R2><<<grid, 256, 0, st>>>(fi, gi, fo, go, p);
+        if (closure == 0) step_kernel_pair<S, 0, 0, R2><<<grid, block, 0, st>>>(fi, gi, fo, go, p);
+        else step_kernel_pair<S, 1, 0, R2><<<grid, block, 0, st>>>(fi, gi, fo, go, p);
     } else {
-        if (closure == 0) step_kernel_pair<S, 0, 1, R2><<<grid, 256, 0, st>>>(fi, gi, fo, go, p);
-        else step_kernel_pair<S, 1, 1, R2><<<grid, 256, 0, st>>>(fi, gi, fo, go, p);
+        if (closure == 0) step_kernel_pair<S, 0, 1, R2><<<grid, block, 0, st>>>(fi, gi, fo, go, p);
+        else step_kernel_pair<S, 1, 1, R2><<<grid, block, 0, st>>>(fi, gi, fo, go, p);
     }
 }
 
@@ -203,12 +203,14 @@ template <typename S>
 static cudaError_t launch_pair(const void* fin, const void* gin, void* fout, void* gout, const StepParams<float>& p,
                                int closure, cudaStream_t st) {
     const int npr = p.nx / 2;
-    if (rows2d(npr, p.ny))
+    const bool flat = !rows2d(npr, p.ny);
+    const unsigned block = block_f32(flat ? p.N / 2 : npr, flat ? 1 : p.ny);
+    if (!flat)
         launch_pair_grid<S, true>((const S*)fin, (const S*)gin, (S*)fout, (S*)gout, p, closure,
-                                  dim3((npr + 255) / 256, p.ny), st);
+                                  dim3((npr + block - 1) / block, p.ny), block, st);
     else
         launch_pair_grid<S, false>((const S*)fin, (const S*)gin, (S*)fout, (S*)gout, p, closure,
-                                   dim3((unsigned)((p.N / 2 + 255) / 256)), st);
+                                   dim3((unsigned)((p.N / 2 + block - 1) / block)), block, st);
     return cudaGetLastError();
 }
 
@@ -232,12 +234,13 @@ static cudaError_t launch_typed(const void* fin, const void* gin, void* fout, vo
     // small (block_f64), so that small lattices use as many SMs as they can
     if constexpr (sizeof(C) == 4) {
         if (rows2d(p.nx, p.ny)) {
+            const unsigned block = block_f32(p.nx, p.ny);
             launch_typed_grid<S, C, true>((const S*)fin, (const S*)gin, (S*)fout, (S*)gout, p, closure,
-                                          dim3((p.nx + 255) / 256, p.ny), 256, st);
+                                          dim3((p.nx + block - 1) / block, p.ny), block, st);
             return cudaGetLastError();
         }
     }
-    const unsigned block = sizeof(C) == 8 ? block_f64(p.N) : 256;
+    const unsigned block = sizeof(C) == 8 ? block_f64(p.N) : block_f32(p.N, 1);
     launch_typed_grid<S, C, false>((const S*)fin, (const S*)gin, (S*)fout, (S*)gout, p, closure,
                                    dim3((unsigned)((p.N + block - 1) / block)), block, st);
     return cudaGetLastError();

@@ -246,34 +246,39 @@ static cudaError_t launch_aa_typed(void* f, void* g, const StepParams<C>& p, int
     // as in the two-buffer step: FP64 is FP64-pipe-bound and keeps the 1D grid of small blocks
     if constexpr (sizeof(C) == 4) {
         if (p.nx >= 64 && p.ny <= 65535) {
-            launch_aa_grid<S, C, PHASE, true>((S*)f, (S*)g, p, closure, dim3((p.nx + 255) / 256, p.ny), 256, st);
+            const unsigned block = block_f32(p.nx, p.ny);
+            launch_aa_grid<S, C, PHASE, true>((S*)f, (S*)g, p, closure, dim3((p.nx + block - 1) / block, p.ny), block, st);
             return cudaGetLastError();
         }
     }
-    const unsigned block = sizeof(C) == 8 ? block_f64(p.N) : 256;
+    const unsigned block = sizeof(C) == 8 ? block_f64(p.N) : block_f32(p.N, 1);
     launch_aa_grid<S, C, PHASE, false>((S*)f, (S*)g, p, closure, dim3((unsigned)((p.N + block - 1) / block)), block,
                                        st);
     return cudaGetLastError();
 }
 
 template <typename S, int PHASE, bool R2>
-static void launch_aa_pair_grid(S* f, S* g, const StepParams<float>& p, int closure, dim3 grid, cudaStream_t st) {
+static void launch_aa_pair_grid(S* f, S* g, const StepParams<float>& p, int closure, dim3 grid, unsigned block,
+                                cudaStream_t st) {
     if (p.coupling == 0) {
-        if (closure == 0) launch_pdl(step_kernel_aa_pair<S, 0, 0, PHASE, R2>, grid, 256, 0, st, f, g, p);
-        else launch_pdl(step_kernel_aa_pair<S, 1, 0, PHASE, R2>, grid, 256, 0, st, f, g, p);
+        if (closure == 0) launch_pdl(step_kernel_aa_pair<S, 0, 0, PHASE, R2>, grid, block, 0, st, f, g, p);
+        else launch_pdl(step_kernel_aa_pair<S, 1, 0, PHASE, R2>, grid, block, 0, st, f, g, p);
     } else {
-        if (closure == 0) launch_pdl(step_kernel_aa_pair<S, 0, 1, PHASE, R2>, grid, 256, 0, st, f, g, p);
-        else launch_pdl(step_kernel_aa_pair<S, 1, 1, PHASE, R2>, grid, 256, 0, st, f, g, p);
+        if (closure == 0) launch_pdl(step_kernel_aa_pair<S, 0, 1, PHASE, R2>, grid, block, 0, st, f, g, p);
+        else launch_pdl(step_kernel_aa_pair<S, 1, 1, PHASE, R2>, grid, block, 0, st, f, g, p);
     }
 }
 
 template <typename S, int PHASE>
 static cudaError_t launch_aa_pair(void* f, void* g, const StepParams<float>& p, int closure, cudaStream_t st) {
     const int npr = p.nx / 2;
-    if (npr >= 64 && p.ny <= 65535)
-        launch_aa_pair_grid<S, PHASE, true>((S*)f, (S*)g, p, closure, dim3((npr + 255) / 256, p.ny), st);
+    const bool flat = !(npr >= 64 && p.ny <= 65535);
+    const unsigned block = block_f32(flat ? p.N / 2 : npr, flat ? 1 : p.ny);
+    if (!flat)
+        launch_aa_pair_grid<S, PHASE, true>((S*)f, (S*)g, p, closure, dim3((npr + block - 1) / block, p.ny), block, st);
     else
-        launch_aa_pair_grid<S, PHASE, false>((S*)f, (S*)g, p, closure, dim3((unsigned)((p.N / 2 + 255) / 256)), st);
+        launch_aa_pair_grid<S, PHASE, false>((S*)f, (S*)g, p, closure,
+                                             dim3((unsigned)((p.N / 2 + block - 1) / block)), block, st);
     return cudaGetLastError();
 }
 
