@@ -120,7 +120,10 @@ typedef struct lks_params {
                               the second reads and writes only the node's own slots), half
                               the population memory at the same bytes per step and the
                               same results bit for bit; lks_step and lks_run_to_steady then
-                              take even step counts (LKS_EINVAL otherwise).  With 16-bit
+                              take even step counts (LKS_EINVAL otherwise).  A large FP32
+                              in-place handle also allocates a workspace for the edges of
+                              its kernel's blocks (8 % of the populations at 4096 x 4096)
+                              when it is created; where that fails it steps without.  With 16-bit
                               storage and even nx the in-place buffer keeps each row
                               interleaved (32-bit word w holds nodes x = w and x = w + nx/2);
                               lks_moments, lks_get_state and lks_set_state present and take
@@ -153,9 +156,12 @@ lks_status lks_create(const lks_params* p, lks_handle** out);
 lks_status lks_set_walls(lks_handle* h, double c_bottom, double c_top, double u_bottom, double u_top);
 
 /* Enqueue n >= 0 fused collide-stream steps (pull-stream, wall closures, moments, equilibria,
- * collision and store in one kernel per step).  Asynchronous; n runs as captured CUDA graphs of
- * 64, 32, ..., 2 steps (built on first use, rebuilt after lks_set_walls) plus at most one direct
- * launch.  n must be even for an in-place handle (LKS_EINVAL). */
+ * collision and store in one kernel).  Asynchronous.  Small lattices (up to about 1e4 nodes) take
+ * the whole call in one launch of one thread-block cluster; large FP32 and 16-bit ones take three
+ * steps per pass over memory, the n % 3 left over one by one; all others a kernel per step.  The
+ * result has the same bits either way.  Launches run as captured CUDA graphs of 64, 32, ..., 2 of
+ * them (built on first use, rebuilt after lks_set_walls) plus at most one direct launch.  n must be
+ * even for an in-place handle (LKS_EINVAL). */
 lks_status lks_step(lks_handle* h, int64_t n);
 
 /* Steps taken since lks_create / lks_set_state. */

@@ -207,6 +207,7 @@ struct lks_handle {
     bool staged = false;              // 16-bit, nx % 8 == 0, nx >= 1024: the staged kernels
     lks::StagedStep ss = {nullptr, 0};
     lks::ResidentPlan resident = {0, 0, 0, 0, 0};  // ctas > 0: all steps of a call in one launch
+    void* rows_work = nullptr;        // in-place handles: the fused steps' workspace
     lks::RowsPlan rows = {0, 0, 0};     // strip > 0: kRowSteps steps per launch
     double c_bot = 0.0, c_top = 0.0, u_bot = 0.0, u_top = 0.0;
     StepParams<double> sp;
@@ -271,7 +272,7 @@ int launch_steps(const lks_handle* h) { return h->rows.strip ? lks::kRowSteps : 
 cudaError_t launch_once(lks_handle* h, int src, cudaStream_t st) {
     if (h->rows.strip)
         return lks::launch_rows(h->p.storage, h->p.closure, h->f[src], h->g[src], h->f[src ^ 1], h->g[src ^ 1], h->sp,
-                                h->rows, st);
+                                h->rows, h->rows_work, st);
     return step_once(h, src, st);
 }
 
@@ -429,8 +430,14 @@ lks_status lks_create(const lks_params* p, lks_handle** out) {
         h->staged = e == cudaSuccess;
     }
     if (e == cudaSuccess) e = lks::plan_resident(p->storage, p->closure, p->coupling, p->nx, p->ny, &h->resident);
-    if (e == cudaSuccess && !p->inplace && !h->resident.ctas)
-        e = lks::plan_rows(p->storage, p->closure, p->coupling, p->nx, p->ny, &h->rows);
+    if (e == cudaSuccess && !h->resident.ctas)
+        e = lks::plan_rows(p->storage, p->closure, p->coupling, p->inplace, p->nx, p->ny, &h->rows);
+    if (e == cudaSuccess && p->inplace && h->rows.strip &&
+        cudaMalloc(&h->rows_work, lks::rows_workspace(p->nx, p->ny, h->rows)) != cudaSuccess) {
+        cudaGetLastError();  // no room for it: pairs of single steps
+        h->rows_work = nullptr;
+        h->rows.strip = 0;
+    }
     if (e != cudaSuccess) {
         lks_destroy(h);
         return cuda_fail(nullptr, e, "lks_create");
@@ -480,6 +487,8 @@ lks_status lks_step(lks_handle* h, int64_t n) {
     }
     const int64_t per = launch_steps(h);
     int64_t left = n / per;  // launches of `per` steps
+    if (h->rows_work) left &= ~(int64_t)1;  // in place the rest is taken in pairs of steps
+    n -= left * per;
     for (int g = 0; g < kGraphSizes && !h->graphs_disabled; ++g) {
         while (left >= kGraphLaunches[g] && !h->graphs_disabled) {
             if (!h->graph[g][h->cur]) {
@@ -499,10 +508,10 @@ lks_status lks_step(lks_handle* h, int64_t n) {
     for (; left > 0; --left) {
         cudaError_t e = launch_once(h, h->cur, h->stream);
         if (e != cudaSuccess) return cuda_fail(h, e, "step kernel launch");
-        h->cur ^= 1;
+        if (!h->rows_work) h->cur ^= 1;
         h->steps += per;
     }
-    for (n %= per; n > 0; --n) {
+    for (; n > 0; --n) {
         cudaError_t e = step_once(h, h->cur, h->stream);
         if (e != cudaSuccess) return cuda_fail(h, e, "step kernel launch");
         h->cur ^= 1;
@@ -720,6 +729,7 @@ lks_status lks_destroy(lks_handle* h) {
     if (h->stream || h->base) cudaStreamSynchronize(h->stream);
     drop_graphs(h);
     if (h->state_stage) cudaFree(h->state_stage);
+    if (h->rows_work) cudaFree(h->rows_work);
     if (h->owns && h->base) cudaFree(h->base);
     if (h->host_small) cudaFreeHost(h->host_small);
     if (h->cap_stream) cudaStreamDestroy(h->cap_stream);

@@ -109,18 +109,19 @@ cudaError_t launch_step(int storage, int closure, const void* fin, const void* g
 cudaError_t launch_step_aa(int storage, int closure, int phase, void* f, void* g, const StepParams<double>& pd,
                            cudaStream_t st, const StagedStep* ss = nullptr);
 
-// kRowSteps fused steps per pass over memory (lks_step_rows.cu): two-buffer handles with FP32 or 16-bit
-// storage.  kRowSteps is odd, so that a fused pass moves the state to the other buffer as that many
-// single steps do.  strip: columns per block (words of two nodes for 16-bit storage), 0 where the
+// kRowSteps fused steps per pass over memory (lks_step_rows.cu): FP32 and 16-bit storage.  kRowSteps is odd,
+// so that a fused pass of a two-buffer handle moves the state to the other buffer as that many single steps do.  strip: columns per block (words of two nodes for 16-bit storage), 0 where the
 // kernel does not apply; chunk: rows per block; edge: rows of the blocks at the bottom wall (at the top
 // wall: what is left).
 constexpr int kRowSteps = 3;
 struct RowsPlan {
     int strip, chunk, edge;
 };
-cudaError_t plan_rows(int storage, int closure, int coupling, int nx, int ny, RowsPlan* rp);
+cudaError_t plan_rows(int storage, int closure, int coupling, int inplace, int nx, int ny, RowsPlan* rp);
+// In place (fin = fout; FP32): `work` holds rows_workspace() bytes; null for two buffers.
+size_t rows_workspace(int nx, int ny, const RowsPlan& rp);
 cudaError_t launch_rows(int storage, int closure, const void* fin, const void* gin, void* fout, void* gout,
-                        const StepParams<double>& pd, const RowsPlan& rp, cudaStream_t st);
+                        const StepParams<double>& pd, const RowsPlan& rp, void* work, cudaStream_t st);
 
 // Small lattices held in one cluster's shared memory for all steps of a call (lks_resident.cu).  ctas: 0
 // where it does not apply.  fin / fout: the buffers before and after `steps` steps (they may be the same);

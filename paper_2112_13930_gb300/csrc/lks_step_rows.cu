@@ -1,5 +1,4 @@
-// lks_step_rows.cu -- kRowSteps steps of one lattice per pass over memory (two-buffer handles, FP32
-// and 16-bit storage).
+// lks_step_rows.cu -- kRowSteps steps of one lattice per pass over memory (FP32 and 16-bit storage).
 //
 // A single FP32 step moves 152 bytes a node and runs at the HBM rate, so more steps per second need
 // fewer bytes per step: a block takes a strip of columns and marches up its rows, computing
@@ -17,6 +16,13 @@
 // A strip carries kRowSteps - 1 extra columns on each side, and a chunk of rows as many extra rows
 // at each end, recomputed by the neighbouring block; a row that fits one block wraps around
 // instead.
+//
+// In place (one population buffer) a block overwrites rows and columns that its neighbours still have to
+// pull from.  A copy kernel therefore saves kRowSteps rows or columns on either side of every block
+// boundary first, and pulls that leave the block's own area read the copies.  Inside the area a row is
+// stored two rows after its last pull.  The pass leaves the natural layout, as a pair of AA steps does.  FP32
+// 4096^2 in place: 45.0 -> 68.4 GLUPS, 2056 x 1500: 43.1 -> 55.7 (two buffers: 98 and 95): the copies take 7 %, and
+// the warp with the block's edges holds up the others at the barriers.
 #include <algorithm>
 #include <type_traits>
 
@@ -185,12 +191,27 @@ __device__ __forceinline__ int ey5(int a) { return a == 2 ? 1 : (a == 4 ? -1 : 0
 struct RowPlanes {
     const char* in[19];
     char* out[19];
+    // in place: what a block pulls from rows and columns of other blocks, saved before the pass
+    const void *rows, *cols;
+};
+
+// Words of the in-place workspace: for each chunk boundary 2 T rows around it, [boundary][plane][2 T][ncol], then for
+// each strip boundary 2 T columns, [strip][plane][ny][2 T].
+struct RowHalos {
+    int chunks, strips;
+    int64_t rows, cols;
+    __host__ __device__ RowHalos(int ncol, int ny, const RowsPlan& rp) {
+        strips = (ncol + rp.strip - 1) / rp.strip;
+        chunks = rp.edge >= ny ? 1 : 1 + (ny - rp.edge + rp.chunk - 1) / rp.chunk;
+        rows = (int64_t)(chunks - 1) * 19 * (2 * kRowSteps) * ncol;
+        cols = (int64_t)strips * 19 * (2 * kRowSteps) * ny;
+    }
 };
 
 // Ring entries of a level: f1 f3 gx1 gx3 gy1 gy3 f5 f6 f7 f8 (the populations with e_x != 0).
 constexpr int kRing = 10;
 
-template <typename S, typename N, int CLOSURE, int COUPLING, int T, int TB, int MINB>
+template <typename S, typename N, int CLOSURE, int COUPLING, bool INPLACE, int T, int TB, int MINB>
 __global__ void __launch_bounds__(TB, MINB) rows_kernel(const __grid_constant__ RowPlanes io,
                                                         const __grid_constant__ StepParams<float> p, int strip,
                                                         int chunk, int edge) {
@@ -201,18 +222,23 @@ __global__ void __launch_bounds__(TB, MINB) rows_kernel(const __grid_constant__ 
     const int ncol = p.nx / N::kNodes, ny = p.ny;   // columns of words
     const unsigned pitch = (unsigned)ncol * (unsigned)sizeof(W);  // bytes of a row
     const int x0 = blockIdx.x * strip, w = min(strip, ncol - x0);
-    const bool wrap = strip >= ncol;                // the whole row in one block
+    const bool wrap = !INPLACE && strip >= ncol;    // the whole row in one block
     const int halo = wrap ? 0 : T - 1;
-    const bool lane = t < w + 2 * halo;
-    int c = lane ? x0 - halo + t : x0;
+    // The thread's slot among the block's columns.  In place the columns that pull from other blocks, three at each
+    // end, go to the first warp, so that one warp takes the longer way to its words.
+    const int slots = w + 2 * halo;
+    const int sl = !INPLACE || slots <= 32 ? t : (t < 29 || t >= slots ? t : (t < 32 ? slots - 32 + t : t - 3));
+    const bool lane = t < slots;
+    const int u = lane ? x0 - halo + sl : x0;  // the thread's column, beyond the periodic edge in a halo
+    int c = u;
     if (c < 0) c += ncol;
     if (c >= ncol) c -= ncol;
     const unsigned cl = (c == 0 ? ncol - 1 : c - 1) * sizeof(W), cc = c * sizeof(W),
                    cr = (c == ncol - 1 ? 0 : c + 1) * sizeof(W);
-    // neighbouring threads' columns in shared memory, relative to the own one
-    const int dl = wrap && t == 0 ? w - 1 : (t == 0 ? 0 : -1);
-    const int dr = wrap && t == w - 1 ? 1 - w : (t == TB - 1 ? 0 : 1);
-    const bool mine = lane && t >= halo && t < halo + w;
+    // the neighbouring columns' slots in shared memory, relative to the own one
+    const int dl = wrap && t == 0 ? w - 1 : (sl == 0 ? 0 : -1);
+    const int dr = wrap && t == w - 1 ? 1 - w : (sl == TB - 1 ? 0 : 1);
+    const bool mine = lane && sl >= halo && sl < halo + w;
     // chunk 0 and the last one, which take the slower path with the walls, are shorter: edge rows
     const int y0 = blockIdx.y == 0 ? 0 : edge + (blockIdx.y - 1) * chunk;
     const int y1 = blockIdx.y == 0 ? min(edge, ny) : min(ny, y0 + chunk);
@@ -220,11 +246,40 @@ __global__ void __launch_bounds__(TB, MINB) rows_kernel(const __grid_constant__ 
     // ring slots of this row, the row before and the one before that: slot s of level k, entry v is
     // base + ((k - 1) * 3 + s) * kRing * TB + v * TB
     constexpr int kLevel = 3 * kRing * TB;
-    W* q0 = reinterpret_cast<W*>(rows_sm) + t;
+    W* q0 = reinterpret_cast<W*>(rows_sm) + sl;
     W* q1 = q0 + kRing * TB;
     W* q2 = q1 + kRing * TB;
     Kept<W> kept[T - 1] = {};
 
+    // In place, near a block's edge: where the planes' words of column v (beyond the periodic edge or not) of row y
+    // are, in the saved copy if the row or the column is another block's: plane a < 9 at f + a ps, 9 + a at g + a ps.
+    // Selects rather than a branch per load, which would wait for each load.
+    struct Planes {
+        const char *f, *g;
+        unsigned ps;
+    };
+    auto planes_at = [&](int y, int v) -> Planes {
+        Planes q;
+        if (y < y0 || y >= y1) {  // the same for the whole block
+            const int vm = v < 0 ? v + ncol : (v >= ncol ? v - ncol : v);
+            const int b = (int)blockIdx.y - (y < y0 ? 1 : 0), k = y - (y < y0 ? y0 : y1) + T;
+            q.ps = 2 * T * pitch;
+            q.f = (const char*)io.rows + ((uint64_t)(unsigned)(b * 19) * q.ps + (unsigned)k * pitch + vm * (unsigned)sizeof(W));
+            q.g = q.f + 9 * (uint64_t)q.ps;
+            return q;
+        }
+        const bool left = v < x0, out = left || v >= x0 + w;
+        const int b = left ? blockIdx.x : (blockIdx.x + 1 == gridDim.x ? 0 : blockIdx.x + 1);
+        const unsigned saved = 2 * T * sizeof(W) * ny, plane = pitch * ny;
+        const unsigned at_out = (unsigned)y * (2 * T * sizeof(W)) + (v - (left ? x0 : x0 + w) + T) * (unsigned)sizeof(W);
+        const unsigned at_own = (unsigned)y * pitch + v * (unsigned)sizeof(W);
+        const char* base = (const char*)io.cols + (uint64_t)(unsigned)(b * 19) * saved;
+        const unsigned at = out ? at_out : at_own;
+        q.ps = out ? saved : plane;
+        q.f = (out ? base : io.in[0]) + at;
+        q.g = (out ? base + 9 * (uint64_t)saved : io.in[9]) + at;
+        return q;
+    };
     // Row r: level 1 of row r, ..., level T of row r - (T - 1).  now / before: ring slots.
     auto row = [&](auto walls, int r, W* now, W* before) {
         // Without WALLS no level's row is beyond or at a wall; a level that is not on yet then computes
@@ -239,51 +294,68 @@ __global__ void __launch_bounds__(TB, MINB) rows_kernel(const __grid_constant__ 
             const bool bottom = WALLS && j == 0, top = WALLS && j == ny - 1;
             if (k == 1) {
                 if (on) {
+                    // get(plane, dy, dx): the word of the own column + dx in row j + dy
+                    auto load = [&](auto get) {
+                        auto same = [&](int a, int dy) -> V { return N::unpack(get(a, dy, 0)); };
+                        auto left = [&](int a, int dy) -> V {
+                            return N::unpack(N::from_left(get(a, dy, -1), N::kOwn ? get(a, dy, 0) : W()));
+                        };
+                        auto right = [&](int a, int dy) -> V {
+                            return N::unpack(N::from_right(N::kOwn ? get(a, dy, 0) : W(), get(a, dy, 1)));
+                        };
+                        f[0] = same(0, 0);
+                        f[1] = left(1, 0);
+                        f[3] = right(3, 0);
+                        gx[0] = same(9, 0);
+                        gx[1] = left(10, 0);
+                        gx[3] = right(12, 0);
+                        gy[0] = same(14, 0);
+                        gy[1] = left(15, 0);
+                        gy[3] = right(17, 0);
+                        if (!bottom) {
+                            f[2] = same(2, -1);
+                            f[5] = left(5, -1);
+                            f[6] = right(6, -1);
+                            gx[2] = same(11, -1);
+                            gy[2] = same(16, -1);
+                        } else if (CLOSURE == 0) {  // the node's own outgoing populations
+                            f[2] = same(4, 0);
+                            f[5] = same(7, 0);
+                            f[6] = same(8, 0);
+                            gx[2] = same(13, 0);
+                            gy[2] = same(18, 0);
+                        }
+                        if (!top) {
+                            f[4] = same(4, 1);
+                            f[7] = right(7, 1);
+                            f[8] = left(8, 1);
+                            gx[4] = same(13, 1);
+                            gy[4] = same(18, 1);
+                        } else if (CLOSURE == 0) {
+                            f[4] = same(2, 0);
+                            f[7] = same(5, 0);
+                            f[8] = same(6, 0);
+                            gx[4] = same(11, 0);
+                            gy[4] = same(16, 0);
+                        }
+                    };
                     const unsigned rc = (unsigned)j * pitch, rs = rc - pitch, rn = rc + pitch;  // bytes
-                    auto word = [&](int a, unsigned at) -> W {
-                        return __ldg(reinterpret_cast<const W*>(io.in[a] + at));
+                    auto near = [&](int a, int dy, int dx) -> W {
+                        const W* q = reinterpret_cast<const W*>(io.in[a] + ((dy == 0 ? rc : (dy < 0 ? rs : rn)) +
+                                                                             (dx == 0 ? cc : (dx < 0 ? cl : cr))));
+                        return INPLACE ? *q : __ldg(q);
                     };
-                    auto same = [&](int a, unsigned row) -> V { return N::unpack(word(a, row + cc)); };
-                    auto left = [&](int a, unsigned row) -> V {
-                        return N::unpack(N::from_left(word(a, row + cl), N::kOwn ? word(a, row + cc) : W()));
-                    };
-                    auto right = [&](int a, unsigned row) -> V {
-                        return N::unpack(N::from_right(N::kOwn ? word(a, row + cc) : W(), word(a, row + cr)));
-                    };
-                    f[0] = same(0, rc);
-                    f[1] = left(1, rc);
-                    f[3] = right(3, rc);
-                    gx[0] = same(9, rc);
-                    gx[1] = left(10, rc);
-                    gx[3] = right(12, rc);
-                    gy[0] = same(14, rc);
-                    gy[1] = left(15, rc);
-                    gy[3] = right(17, rc);
-                    if (!bottom) {
-                        f[2] = same(2, rs);
-                        f[5] = left(5, rs);
-                        f[6] = right(6, rs);
-                        gx[2] = same(11, rs);
-                        gy[2] = same(16, rs);
-                    } else if (CLOSURE == 0) {  // the node's own outgoing populations
-                        f[2] = same(4, rc);
-                        f[5] = same(7, rc);
-                        f[6] = same(8, rc);
-                        gx[2] = same(13, rc);
-                        gy[2] = same(18, rc);
-                    }
-                    if (!top) {
-                        f[4] = same(4, rn);
-                        f[7] = right(7, rn);
-                        f[8] = left(8, rn);
-                        gx[4] = same(13, rn);
-                        gy[4] = same(18, rn);
-                    } else if (CLOSURE == 0) {
-                        f[4] = same(2, rc);
-                        f[7] = same(5, rc);
-                        f[8] = same(6, rc);
-                        gx[4] = same(11, rc);
-                        gy[4] = same(16, rc);
+                    if constexpr (INPLACE) {
+                        if (__all_sync(0xffffffffu, u > x0 && u + 1 < x0 + w && j > y0 && j + 1 < y1))
+                            load(near);
+                        else
+                            load([&](int a, int dy, int dx) -> W {
+                                const Planes q = planes_at(j + dy, u + dx);
+                                return *reinterpret_cast<const W*>((a < 9 ? q.f : q.g) +
+                                                                   (uint64_t)q.ps * (a < 9 ? a : a - 9));
+                            });
+                    } else {
+                        load(near);
                     }
                 }
             } else {
@@ -423,18 +495,44 @@ __global__ void __launch_bounds__(TB, MINB) rows_kernel(const __grid_constant__ 
     }
 }
 
-template <typename S, typename N, int TB, int MINB>
+// Copies the rows and columns around the blocks' boundaries (RowHalos) before an in-place pass overwrites them.
+// blockIdx.x: boundary and plane; blockIdx.y: a part of it.
+template <typename W>
+__global__ void __launch_bounds__(256) rows_save_kernel(const __grid_constant__ RowPlanes io, int ncol, int ny,
+                                                        const __grid_constant__ RowsPlan rp, W* rows, W* cols) {
+    constexpr int D = 2 * kRowSteps;
+    const RowHalos h(ncol, ny, rp);
+    const int a = blockIdx.x % 19, b = blockIdx.x / 19;
+    const int first = blockIdx.y * blockDim.x + threadIdx.x, stride = gridDim.y * blockDim.x;
+    const W* in = reinterpret_cast<const W*>(io.in[a]);
+    if (b < h.chunks - 1) {
+        const int y = rp.edge + b * rp.chunk - kRowSteps, n = min(D, ny - y);  // a last chunk may be shorter
+        const W* src = in + (int64_t)y * ncol;
+        W* dst = rows + (int64_t)(b * 19 + a) * D * ncol;
+        for (int k = first; k < n * ncol; k += stride) dst[k] = src[k];
+    } else {
+        const int s = b - (h.chunks - 1);
+        W* dst = cols + (int64_t)(s * 19 + a) * ny * D;
+        for (int k = first; k < D * ny; k += stride) {
+            const int y = k / D, v = s * rp.strip - kRowSteps + (k - y * D);
+            dst[k] = in[(int64_t)y * ncol + (v < 0 ? v + ncol : (v >= ncol ? v - ncol : v))];
+        }
+    }
+}
+
+template <typename S, typename N, bool INPLACE, int TB, int MINB>
 struct Rows {
     static constexpr int kThreads = TB, kNodes = N::kNodes;
     // the Maxwell coupling's form of the node type
     static constexpr bool kScaled = std::is_same<N, TwoNodes<__half>>::value;
     typedef typename std::conditional<kScaled, TwoNodesScaled<S>, N>::type M;
+    static constexpr bool kInplace = INPLACE;
     typedef void (*Fn)(const RowPlanes, const StepParams<float>, int, int, int);
     static Fn kernel(int closure, int coupling) {
         constexpr int T = kRowSteps;
         if (coupling == 0)
-            return closure == 0 ? rows_kernel<S, M, 0, 0, T, TB, MINB> : rows_kernel<S, M, 1, 0, T, TB, MINB>;
-        return closure == 0 ? rows_kernel<S, N, 0, 1, T, TB, MINB> : rows_kernel<S, N, 1, 1, T, TB, MINB>;
+            return closure == 0 ? rows_kernel<S, M, 0, 0, INPLACE, T, TB, MINB> : rows_kernel<S, M, 1, 0, INPLACE, T, TB, MINB>;
+        return closure == 0 ? rows_kernel<S, N, 0, 1, INPLACE, T, TB, MINB> : rows_kernel<S, N, 1, 1, INPLACE, T, TB, MINB>;
     }
     static constexpr size_t smem() { return (size_t)(kRowSteps - 1) * 3 * kRing * TB * sizeof(typename N::W); }
     static cudaError_t prepare(int closure, int coupling, int* blocks) {
@@ -444,13 +542,22 @@ struct Rows {
         return e;
     }
     static void launch(const void* fin, const void* gin, void* fout, void* gout, const StepParams<float>& p,
-                       int closure, const RowsPlan& rp, cudaStream_t st) {
-        const dim3 grid((p.nx / N::kNodes + rp.strip - 1) / rp.strip,
-                        rp.edge >= p.ny ? 1 : 1 + (p.ny - rp.edge + rp.chunk - 1) / rp.chunk);
+                       int closure, const RowsPlan& rp, void* work, cudaStream_t st) {
+        const int ncol = p.nx / N::kNodes;
+        const RowHalos halos(ncol, p.ny, rp);
+        const dim3 grid(halos.strips, halos.chunks);
         RowPlanes io;
         for (int a = 0; a < 19; ++a) {
             io.in[a] = (const char*)(a < 9 ? (const S*)fin + a * p.N : (const S*)gin + (a - 9) * p.N);
             io.out[a] = (char*)(a < 9 ? (S*)fout + a * p.N : (S*)gout + (a - 9) * p.N);
+        }
+        io.rows = io.cols = nullptr;
+        if (INPLACE) {
+            typedef typename N::W W;
+            W *rows = (W*)work, *cols = rows + halos.rows;
+            rows_save_kernel<W><<<dim3(19 * (halos.chunks - 1 + halos.strips), 8), 256, 0, st>>>(io, ncol, p.ny, rp, rows, cols);
+            io.rows = rows;
+            io.cols = cols;
         }
         kernel(closure, p.coupling)<<<grid, TB, smem(), st>>>(
             io, kScaled && p.coupling == 0 ? scaled_params(p, closure) : p, rp.strip, rp.chunk, rp.edge);
@@ -461,9 +568,10 @@ struct Rows {
 // blocks wait less at their barriers; the extra columns of narrow strips cost more below 128.
 #define F32S 128, 5
 #define H16S 128, 4
-typedef Rows<float, OneNode<float>, F32S> RowsF32;
-typedef Rows<__nv_bfloat16, TwoNodes<__nv_bfloat16>, H16S> RowsBf16;
-typedef Rows<__half, TwoNodes<__half>, H16S> RowsF16;
+typedef Rows<float, OneNode<float>, false, F32S> RowsF32;
+typedef Rows<__nv_bfloat16, TwoNodes<__nv_bfloat16>, false, H16S> RowsBf16;
+typedef Rows<__half, TwoNodes<__half>, false, H16S> RowsF16;
+typedef Rows<float, OneNode<float>, true, F32S> InplaceF32;
 
 }  // namespace
 
@@ -478,7 +586,7 @@ static cudaError_t plan_typed(int closure, int coupling, int nx, int ny, RowsPla
     const int ncol = nx / R::kNodes;
     const int most = R::kThreads - 2 * (kRowSteps - 1);
     int strips = 1, strip = ncol;
-    if (ncol > R::kThreads) {
+    if (ncol > (R::kInplace ? most : R::kThreads)) {
         strips = (ncol + most - 1) / most;
         strip = std::min(most, ((ncol + strips - 1) / strips + 7) / 8 * 8);
         strips = (ncol + strip - 1) / strip;
@@ -500,20 +608,32 @@ static cudaError_t plan_typed(int closure, int coupling, int nx, int ny, RowsPla
     return cudaSuccess;
 }
 
-cudaError_t plan_rows(int storage, int closure, int coupling, int nx, int ny, RowsPlan* rp) {
+cudaError_t plan_rows(int storage, int closure, int coupling, int inplace, int nx, int ny, RowsPlan* rp) {
     rp->strip = rp->chunk = rp->edge = 0;
     if (storage == 0 || (storage >= 2 && nx % 2 != 0) || nx < 64) return cudaSuccess;
+    if (inplace) {
+        // FP32 only: the interleaved rows of 16-bit storage ran at 64 (BF16) and 58 (FP16) GLUPS against 67 and 83 in AA
+        // pairs (2056 x 1500).  Plane strides are 32-bit.
+        if (storage != 1 || (int64_t)nx * ny * 4 >= (int64_t)1 << 32) return cudaSuccess;
+        return plan_typed<InplaceF32>(closure, coupling, nx, ny, rp);
+    }
     if (storage == 1) return plan_typed<RowsF32>(closure, coupling, nx, ny, rp);
     if (storage == 2) return plan_typed<RowsBf16>(closure, coupling, nx, ny, rp);
     return plan_typed<RowsF16>(closure, coupling, nx, ny, rp);
 }
 
+size_t rows_workspace(int nx, int ny, const RowsPlan& rp) {
+    const RowHalos h(nx, ny, rp);
+    return (size_t)(h.rows + h.cols) * sizeof(float);
+}
+
 cudaError_t launch_rows(int storage, int closure, const void* fin, const void* gin, void* fout, void* gout,
-                        const StepParams<double>& pd, const RowsPlan& rp, cudaStream_t st) {
+                        const StepParams<double>& pd, const RowsPlan& rp, void* work, cudaStream_t st) {
     const StepParams<float> p = convert_params<float>(pd);
-    if (storage == 1) RowsF32::launch(fin, gin, fout, gout, p, closure, rp, st);
-    else if (storage == 2) RowsBf16::launch(fin, gin, fout, gout, p, closure, rp, st);
-    else RowsF16::launch(fin, gin, fout, gout, p, closure, rp, st);
+    if (work) InplaceF32::launch(fin, gin, fout, gout, p, closure, rp, work, st);
+    else if (storage == 1) RowsF32::launch(fin, gin, fout, gout, p, closure, rp, nullptr, st);
+    else if (storage == 2) RowsBf16::launch(fin, gin, fout, gout, p, closure, rp, nullptr, st);
+    else RowsF16::launch(fin, gin, fout, gout, p, closure, rp, nullptr, st);
     return cudaGetLastError();
 }
 

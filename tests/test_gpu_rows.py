@@ -42,3 +42,28 @@ def test_fused_steps_equal_single_steps_bitwise(lks, storage, closure, coupling)
             assert np.array_equal(a.get_state_raw(), b.get_state_raw()), (nx, ny, n)
         a.close()
         b.close()
+
+
+@pytest.mark.parametrize("closure", ["link", "moment"])
+@pytest.mark.parametrize("coupling", ["maxwell", "lorentz"])
+def test_fused_steps_in_place_equal_two_buffer_single_steps_bitwise(lks, closure, coupling):
+    """One buffer (FP32): fused passes come in twos (6 steps), the rest in AA pairs.  (124, 6000) is one strip whose
+    halo columns wrap onto itself, (125, 3100) a second strip of one column's width, (1001, 1307) a last chunk of
+    one row."""
+    storage = "f32"
+    for nx, ny in SIZES[storage] + [(124, 6000), (125, 3100), (1001, 1307)]:
+        kw = dict(closure=closure, storage=storage, coupling=coupling, seed=5, perturb_amp=1e-2)
+        a = lks.Lattice(nx, ny, 0.7, 0.9, 0.02, 2e-5, inplace=True, **kw)
+        b = lks.Lattice(nx, ny, 0.7, 0.9, 0.02, 2e-5, **kw)
+        for lat in (a, b):
+            lat.set_walls(0.4, 3.0, 0.02, -0.04)
+        for n in (6, 14):      # one graph of two passes; two of them and a pair
+            a.step(n)
+            for _ in range(n):
+                b.step(1)
+            assert a.steps == b.steps
+            fa, ga = a.get_state()
+            fb, gb = b.get_state()
+            assert np.array_equal(fa, fb) and np.array_equal(ga, gb), (nx, ny, n)
+        a.close()
+        b.close()
