@@ -429,9 +429,10 @@ lks_status lks_create(const lks_params* p, lks_handle** out) {
         h->ss.err = h->flag;
         h->staged = e == cudaSuccess;
     }
+    refresh_params(h);
     if (e == cudaSuccess) e = lks::plan_resident(p->storage, p->closure, p->coupling, p->nx, p->ny, &h->resident);
     if (e == cudaSuccess && !h->resident.ctas)
-        e = lks::plan_rows(p->storage, p->closure, p->coupling, p->inplace, p->nx, p->ny, &h->rows);
+        e = lks::plan_rows(p->storage, p->closure, h->sp, p->inplace, &h->rows);
     if (e == cudaSuccess && p->inplace && h->rows.strip &&
         cudaMalloc(&h->rows_work, lks::rows_workspace(p->nx, p->ny, h->rows)) != cudaSuccess) {
         cudaGetLastError();  // no room for it: pairs of single steps
@@ -442,7 +443,6 @@ lks_status lks_create(const lks_params* p, lks_handle** out) {
         lks_destroy(h);
         return cuda_fail(nullptr, e, "lks_create");
     }
-    refresh_params(h);
     const int ilv = lks::interleave_row(p->storage, p->nx, p->inplace);
     e = lks::launch_init(p->storage, h->f[0], h->g[0], p->nx, p->ny, p->B0, p->seed, p->perturb_amp, h->stream, ilv);
     if (e == cudaSuccess)

@@ -117,7 +117,7 @@ constexpr int kRowSteps = 3;
 struct RowsPlan {
     int strip, chunk, edge;
 };
-cudaError_t plan_rows(int storage, int closure, int coupling, int inplace, int nx, int ny, RowsPlan* rp);
+cudaError_t plan_rows(int storage, int closure, const StepParams<double>& p, int inplace, RowsPlan* rp);
 // In place (fin = fout; FP32): `work` holds rows_workspace() bytes; null for two buffers.
 size_t rows_workspace(int nx, int ny, const RowsPlan& rp);
 cudaError_t launch_rows(int storage, int closure, const void* fin, const void* gin, void* fout, void* gout,

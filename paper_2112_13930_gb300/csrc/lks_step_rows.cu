@@ -101,33 +101,46 @@ StepParams<float> scaled_params(StepParams<float> p, int closure) {
     return p;
 }
 
-// collide_node and collide_g on scaled populations with scaled_params: the same operations in the same
-// order, the moments unscaled.
-__device__ __forceinline__ void collide_scaled(float2 f[9], float2 gx[5], float2 gy[5], const StepParams<float>& p) {
-    const float un = kHalfUnscale, half = 0.5f, three = 3.0f, four5 = 4.5f, one5 = 1.5f;
-    const auto drho = fmul(un, ((f[0] + f[1]) + (f[2] + f[3])) + ((f[4] + f[5]) + (f[6] + f[7])) + f[8]);
+// collide_node and collide_g, the same operations in the same order, with two things it leaves to its caller:
+// SCALED populations with scaled_params, whose moments are brought back here, and no body force (FORCE false:
+// the source terms are zeros then, a sixth of the arithmetic; 4096^2 without a force, GLUPS: BF16 125 -> 141,
+// FP16 117 -> 132, FP32, near the HBM rate, 97.8 -> 100.5).
+template <bool FORCE, bool SCALED, typename V>
+__device__ __forceinline__ void collide_rows(V f[9], V gx[5], V gy[5], const StepParams<float>& p) {
+    const float half = 0.5f, three = 3.0f, four5 = 4.5f, one5 = 1.5f;
+    auto back = [&](V x) -> V {
+        if constexpr (SCALED) return fmul(kHalfUnscale, x);
+        return x;
+    };
+    const auto drho = back(((f[0] + f[1]) + (f[2] + f[3])) + ((f[4] + f[5]) + (f[6] + f[7])) + f[8]);
     const auto rho = 1.0f + drho;
-    const auto jx = fmul(un, (f[1] - f[3]) + (f[5] - f[6]) + (f[8] - f[7]));
-    const auto jy = fmul(un, (f[2] - f[4]) + (f[5] + f[6]) - (f[7] + f[8]));
+    const auto jx = back((f[1] - f[3]) + (f[5] - f[6]) + (f[8] - f[7]));
+    const auto jy = back((f[2] - f[4]) + (f[5] + f[6]) - (f[7] + f[8]));
     const auto inv_rho = recip(rho);
-    const auto ux = fmul(ffma(half, p.Fx, jx), inv_rho);
+    const auto ux = fmul(FORCE ? ffma(half, p.Fx, jx) : jx, inv_rho);
     const auto uy = fmul(jy, inv_rho);
-    const auto bx = fmul(un, ((gx[0] + gx[1]) + (gx[2] + gx[3])) + gx[4]);
-    const auto dby = fmul(un, ((gy[0] + gy[1]) + (gy[2] + gy[3])) + gy[4]);
+    const auto bx = back(((gx[0] + gx[1]) + (gx[2] + gx[3])) + gx[4]);
+    const auto dby = back(((gy[0] + gy[1]) + (gy[2] + gy[3])) + gy[4]);
     const auto by = p.B0 + dby;
     const auto q = fmul(dby, p.B0 + by);
     const auto om13 = fmul(p.owf1, fmul(2.25f, ffma(-bx, bx, q)));
     const auto omxy = fmul(p.owf5, fmul(fmul(9.0f, bx), by));
     const auto usq = fmul(one5, ffma(ux, ux, fmul(uy, uy)));
-    const auto s0 = fmul(p.sw0, -ux);
-    const auto s1p = fmul(p.sw1, 1.0f - ux), s1z = fmul(p.sw1, -ux), s1m = fmul(p.sw1, -1.0f - ux);
-    const auto s5p = fmul(p.sw5, 1.0f - ux), s5m = fmul(p.sw5, -1.0f - ux);
-    auto dir = [&](int a, float2 eu, float ow, float2 omag, float2 sa) {
+    V s0 = zero_of<V>(), s1p = s0, s1z = s0, s1m = s0, s5p = s0, s5m = s0;  // source prefactors
+    if constexpr (FORCE) {
+        s0 = fmul(p.sw0, -ux);
+        s1p = fmul(p.sw1, 1.0f - ux), s1z = fmul(p.sw1, -ux), s1m = fmul(p.sw1, -1.0f - ux);
+        s5p = fmul(p.sw5, 1.0f - ux), s5m = fmul(p.sw5, -1.0f - ux);
+    }
+    auto dir = [&](int a, V eu, float ow, V omag, V sa) {
         const auto bm1 = ffma(ffma(four5, eu, three), eu, -usq);
         const auto ofeq = ffma(ow, ffma(rho, bm1, drho), omag);
-        f[a] = ffma(p.om1f, f[a], ofeq + ffma(sa, bm1, sa));
+        if constexpr (FORCE)
+            f[a] = ffma(p.om1f, f[a], ofeq + ffma(sa, bm1, sa));
+        else
+            f[a] = ffma(p.om1f, f[a], ofeq);
     };
-    const float2 zero = make_float2(0.0f, 0.0f);
+    const V zero = zero_of<V>();
     dir(0, zero, p.owf0, zero, s0);
     dir(1, ux, p.owf1, om13, s1p);
     dir(2, uy, p.owf1, -om13, s1z);
@@ -140,38 +153,33 @@ __device__ __forceinline__ void collide_scaled(float2 f[9], float2 gx[5], float2
     collide_g<float>(gx, gy, ux, uy, bx, by, dby, p);
 }
 
-// The wall closure of a scaled moment-closed row, unscaled, and the scaled collision.
-template <int CLOSURE>
-__device__ __forceinline__ void close_collide_scaled(float2 f[9], float2 gx[5], float2 gy[5],
-                                                     const StepParams<float>& p, bool bottom, bool top) {
-    if (CLOSURE == 1 && (bottom || top)) {
-        auto all = [&](float c) {
+// Moment closure and collision of a thread's node or nodes.  A scaled row is closed unscaled.
+template <int CLOSURE, int COUPLING, bool FORCE, bool SCALED, typename V>
+__device__ __forceinline__ void close_collide(V f[9], V gx[5], V gy[5], const StepParams<float>& p, bool bottom,
+                                              bool top) {
+    if constexpr (COUPLING == 1) {
+        if constexpr (std::is_same<V, float>::value) {
+            if (CLOSURE == 1 && bottom) moment_closure_bottom<float, 1>(f, gx, gy, p.bot, p);
+            if (CLOSURE == 1 && top) moment_closure_top<float, 1>(f, gx, gy, p.top, p);
+            collide<float, 1>(f, gx, gy, p);
+        } else {
+            close_collide_pair<CLOSURE, 1, true>(f, gx, gy, p, bottom, top);
+        }
+    } else {
+        if (CLOSURE == 1 && (bottom || top)) {
+            auto all = [&](float c) {
 #pragma unroll
-            for (int a = 0; a < 9; ++a) f[a] = fmul(c, f[a]);
+                for (int a = 0; a < 9; ++a) f[a] = fmul(c, f[a]);
 #pragma unroll
-            for (int a = 0; a < 5; ++a) gx[a] = fmul(c, gx[a]), gy[a] = fmul(c, gy[a]);
-        };
-        all(kHalfUnscale);
-        if (bottom) moment_closure_bottom<float, 0>(f, gx, gy, p.bot, p);
-        if (top) moment_closure_top<float, 0>(f, gx, gy, p.top, p);
-        all(kHalfScale);
+                for (int a = 0; a < 5; ++a) gx[a] = fmul(c, gx[a]), gy[a] = fmul(c, gy[a]);
+            };
+            if (SCALED) all(kHalfUnscale);
+            if (bottom) moment_closure_bottom<float, 0>(f, gx, gy, p.bot, p);
+            if (top) moment_closure_top<float, 0>(f, gx, gy, p.top, p);
+            if (SCALED) all(kHalfScale);
+        }
+        collide_rows<FORCE, SCALED>(f, gx, gy, p);
     }
-    collide_scaled(f, gx, gy, p);
-}
-
-template <int CLOSURE, int COUPLING>
-__device__ __forceinline__ void close_collide(float f[9], float gx[5], float gy[5], const StepParams<float>& p,
-                                              bool bottom, bool top) {
-    if (CLOSURE == 1) {
-        if (bottom) moment_closure_bottom<float, COUPLING>(f, gx, gy, p.bot, p);
-        if (top) moment_closure_top<float, COUPLING>(f, gx, gy, p.top, p);
-    }
-    collide<float, COUPLING>(f, gx, gy, p);
-}
-template <int CLOSURE, int COUPLING>
-__device__ __forceinline__ void close_collide(float2 f[9], float2 gx[5], float2 gy[5], const StepParams<float>& p,
-                                              bool bottom, bool top) {
-    close_collide_pair<CLOSURE, COUPLING, true>(f, gx, gy, p, bottom, top);
 }
 
 // What a thread keeps of a level for the next one, as storage words: of the row before, the e_x = 0
@@ -211,7 +219,7 @@ struct RowHalos {
 // Ring entries of a level: f1 f3 gx1 gx3 gy1 gy3 f5 f6 f7 f8 (the populations with e_x != 0).
 constexpr int kRing = 10;
 
-template <typename S, typename N, int CLOSURE, int COUPLING, bool INPLACE, int T, int TB, int MINB>
+template <typename S, typename N, int CLOSURE, int COUPLING, bool FORCE, bool INPLACE, int T, int TB, int MINB>
 __global__ void __launch_bounds__(TB, MINB) rows_kernel(const __grid_constant__ RowPlanes io,
                                                         const __grid_constant__ StepParams<float> p, int strip,
                                                         int chunk, int edge) {
@@ -432,10 +440,7 @@ __global__ void __launch_bounds__(TB, MINB) rows_kernel(const __grid_constant__ 
                         gy[4] = -gy[4];
                     }
                 }
-                if constexpr (IsScaled<N>::value)
-                    close_collide_scaled<CLOSURE>(f, gx, gy, p, bottom, top);
-                else
-                    close_collide<CLOSURE, COUPLING>(f, gx, gy, p, bottom, top);
+                close_collide<CLOSURE, COUPLING, FORCE, IsScaled<N>::value>(f, gx, gy, p, bottom, top);
                 if (k < T) {
                     W* ring = now + (k - 1) * kLevel;
                     const V x[kRing] = {f[1], f[3], gx[1], gx[3], gy[1], gy[3], f[5], f[6], f[7], f[8]};
@@ -528,15 +533,20 @@ struct Rows {
     typedef typename std::conditional<kScaled, TwoNodesScaled<S>, N>::type M;
     static constexpr bool kInplace = INPLACE;
     typedef void (*Fn)(const RowPlanes, const StepParams<float>, int, int, int);
-    static Fn kernel(int closure, int coupling) {
-        constexpr int T = kRowSteps;
-        if (coupling == 0)
-            return closure == 0 ? rows_kernel<S, M, 0, 0, INPLACE, T, TB, MINB> : rows_kernel<S, M, 1, 0, INPLACE, T, TB, MINB>;
-        return closure == 0 ? rows_kernel<S, N, 0, 1, INPLACE, T, TB, MINB> : rows_kernel<S, N, 1, 1, INPLACE, T, TB, MINB>;
+    template <int CLOSURE, int COUPLING>
+    static Fn typed(bool force) {
+        typedef typename std::conditional<COUPLING == 0, M, N>::type K;
+        if constexpr (COUPLING == 0)
+            if (!force) return rows_kernel<S, K, CLOSURE, 0, false, INPLACE, kRowSteps, TB, MINB>;
+        return rows_kernel<S, K, CLOSURE, COUPLING, true, INPLACE, kRowSteps, TB, MINB>;
+    }
+    static Fn kernel(int closure, int coupling, bool force) {
+        if (coupling == 0) return closure == 0 ? typed<0, 0>(force) : typed<1, 0>(force);
+        return closure == 0 ? typed<0, 1>(force) : typed<1, 1>(force);
     }
     static constexpr size_t smem() { return (size_t)(kRowSteps - 1) * 3 * kRing * TB * sizeof(typename N::W); }
-    static cudaError_t prepare(int closure, int coupling, int* blocks) {
-        Fn k = kernel(closure, coupling);
+    static cudaError_t prepare(int closure, int coupling, bool force, int* blocks) {
+        Fn k = kernel(closure, coupling, force);
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem());
         if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, k, TB, smem());
         return e;
@@ -559,7 +569,7 @@ struct Rows {
             io.rows = rows;
             io.cols = cols;
         }
-        kernel(closure, p.coupling)<<<grid, TB, smem(), st>>>(
+        kernel(closure, p.coupling, p.Fx != 0.0f)<<<grid, TB, smem(), st>>>(
             io, kScaled && p.coupling == 0 ? scaled_params(p, closure) : p, rp.strip, rp.chunk, rp.edge);
     }
 };
@@ -577,11 +587,11 @@ typedef Rows<float, OneNode<float>, true, F32S> InplaceF32;
 
 // Strips and chunks of the kernel R: as many blocks as are resident at once.
 template <typename R>
-static cudaError_t plan_typed(int closure, int coupling, int nx, int ny, RowsPlan* rp) {
+static cudaError_t plan_typed(int closure, int coupling, bool force, int nx, int ny, RowsPlan* rp) {
     int dev = 0, sms = 0, blocks = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) e = R::prepare(closure, coupling, &blocks);
+    if (e == cudaSuccess) e = R::prepare(closure, coupling, force, &blocks);
     if (e != cudaSuccess) return e;
     const int ncol = nx / R::kNodes;
     const int most = R::kThreads - 2 * (kRowSteps - 1);
@@ -608,18 +618,20 @@ static cudaError_t plan_typed(int closure, int coupling, int nx, int ny, RowsPla
     return cudaSuccess;
 }
 
-cudaError_t plan_rows(int storage, int closure, int coupling, int inplace, int nx, int ny, RowsPlan* rp) {
+cudaError_t plan_rows(int storage, int closure, const StepParams<double>& p, int inplace, RowsPlan* rp) {
+    const int nx = p.nx, ny = p.ny, coupling = p.coupling;
+    const bool force = (float)p.Fx != 0.0f;
     rp->strip = rp->chunk = rp->edge = 0;
     if (storage == 0 || (storage >= 2 && nx % 2 != 0) || nx < 64) return cudaSuccess;
     if (inplace) {
         // FP32 only: the interleaved rows of 16-bit storage ran at 64 (BF16) and 58 (FP16) GLUPS against 67 and 83 in AA
         // pairs (2056 x 1500).  Plane strides are 32-bit.
         if (storage != 1 || (int64_t)nx * ny * 4 >= (int64_t)1 << 32) return cudaSuccess;
-        return plan_typed<InplaceF32>(closure, coupling, nx, ny, rp);
+        return plan_typed<InplaceF32>(closure, coupling, force, nx, ny, rp);
     }
-    if (storage == 1) return plan_typed<RowsF32>(closure, coupling, nx, ny, rp);
-    if (storage == 2) return plan_typed<RowsBf16>(closure, coupling, nx, ny, rp);
-    return plan_typed<RowsF16>(closure, coupling, nx, ny, rp);
+    if (storage == 1) return plan_typed<RowsF32>(closure, coupling, force, nx, ny, rp);
+    if (storage == 2) return plan_typed<RowsBf16>(closure, coupling, force, nx, ny, rp);
+    return plan_typed<RowsF16>(closure, coupling, force, nx, ny, rp);
 }
 
 size_t rows_workspace(int nx, int ny, const RowsPlan& rp) {
