@@ -823,6 +823,7 @@ __global__ void residual3_partial(const S* f, const S* g, int64_t N, double B0, 
                                   double* partial) {
     __shared__ double red[4 * 32];
     double acc[4] = {0, 0, 0, 0};
+    lks::pdl_wait();
     for (int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; n < N; n += (int64_t)gridDim.x * blockDim.x) {
         double m[7];
         node_moments3<S>(f, g, N, n, B0, Fx, m);
@@ -842,6 +843,7 @@ __global__ void residual3_partial(const S* f, const S* g, int64_t N, double B0, 
 __global__ void residual3_final(const double* partial, int nb, double* out) {
     __shared__ double red[4 * 32];
     double acc[4];
+    lks::pdl_wait();
     for (int c = 0; c < 4; ++c) acc[c] = (int)threadIdx.x < nb ? partial[c * nb + threadIdx.x] : 0.0;
     lks::block_sum<4>(acc, red);
     if (threadIdx.x == 0)
@@ -905,7 +907,7 @@ const char* validate3(const lks3_params* p) {
 }
 
 struct Layout3 {
-    size_t f_bytes, g_bytes, off_f[2], off_g[2], off_snap, off_partial, off_out, off_prof, off_rest, off_flag, total;
+    size_t f_bytes, g_bytes, off_f[2], off_g[2], off_snap, off_partial, off_prof, off_rest, off_flag, total;
 };
 
 Layout3 layout3(const lks3_params* p) {
@@ -925,8 +927,6 @@ Layout3 layout3(const lks3_params* p) {
     o += align3(2 * N * sizeof(double));
     L.off_partial = o;
     o += align3(4 * kRedBlocks * sizeof(double));
-    L.off_out = o;
-    o += align3(4 * sizeof(double));
     L.off_prof = o;
     o += align3(7 * (size_t)p->ny * sizeof(double));
     L.off_rest = o;
@@ -953,7 +953,7 @@ struct lks3_handle {
     void* f[2] = {nullptr, nullptr};
     void* g[2] = {nullptr, nullptr};
     int cur = 0;
-    double *snap = nullptr, *partial = nullptr, *dout = nullptr, *prof = nullptr, *rest = nullptr;
+    double *snap = nullptr, *partial = nullptr, *prof = nullptr, *rest = nullptr;
     int* flag = nullptr;
     bool staged = false;       // 16-bit storage with nx % 8 == 0: step3_staged_kernel
     unsigned staged_grid = 0;  // resident blocks of it on the device
@@ -1121,8 +1121,8 @@ cudaError_t build_graph3(lks3_handle* h, int size, int start) {
 cudaError_t launch_snapshot3(lks3_handle* h) {
     const int64_t N = (int64_t)h->p.nx * h->p.ny * h->p.nz;
     LKS3_DISPATCH(h->p.storage,
-                  (residual3_partial<S><<<kRedBlocks, 256, 0, h->stream>>>((const S*)h->f[h->cur], (const S*)h->g[h->cur],
-                                                                           N, h->p.B0, h->p.Fx, h->snap, h->partial)));
+                  lks::launch_pdl(residual3_partial<S>, dim3(kRedBlocks), 256, 0, h->stream, (const S*)h->f[h->cur],
+                                  (const S*)h->g[h->cur], N, h->p.B0, h->p.Fx, h->snap, h->partial));
     return cudaGetLastError();
 }
 
@@ -1166,7 +1166,6 @@ lks_status lks3_create(const lks3_params* p, lks3_handle** out) {
     }
     h->snap = (double*)(h->base + h->L.off_snap);
     h->partial = (double*)(h->base + h->L.off_partial);
-    h->dout = (double*)(h->base + h->L.off_out);
     h->prof = (double*)(h->base + h->L.off_prof);
     h->rest = (double*)(h->base + h->L.off_rest);
     h->flag = (int*)(h->base + h->L.off_flag);
@@ -1303,10 +1302,9 @@ lks_status lks3_residual(lks3_handle* h, double* r_u, double* r_b) {
     if (!h) return fail3(nullptr, LKS_EINVAL, "handle is NULL");
     cudaError_t e = launch_snapshot3(h);
     if (e == cudaSuccess) {
-        residual3_final<<<1, 1024, 0, h->stream>>>(h->partial, kRedBlocks, h->dout);
+        lks::launch_pdl(residual3_final, dim3(1), 1024, 0, h->stream, (const double*)h->partial, kRedBlocks, h->host4);
         e = cudaGetLastError();
     }
-    if (e == cudaSuccess) e = cudaMemcpyAsync(h->host4, h->dout, 4 * sizeof(double), cudaMemcpyDeviceToHost, h->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess) return cuda3(h, e, "lks3_residual");
     if (lks_status fs = flag_check3(h, "lks3_residual")) return fs;

@@ -42,7 +42,7 @@ struct NvtxRange {
 };
 
 struct Layout {
-    size_t f_bytes, g_bytes, off_fa, off_ga, off_fb, off_gb, off_snap, off_partial, off_out, off_prof, off_flag, total;
+    size_t f_bytes, g_bytes, off_fa, off_ga, off_fb, off_gb, off_snap, off_partial, off_prof, off_flag, total;
 };
 
 Layout make_layout(const lks_params* p) {
@@ -63,7 +63,6 @@ Layout make_layout(const lks_params* p) {
     }
     L.off_snap = o; o += align_up(2 * N * sizeof(double));
     L.off_partial = o; o += align_up(4 * (size_t)lks::residual_blocks((int64_t)N) * sizeof(double));
-    L.off_out = o; o += align_up(8 * sizeof(double));
     L.off_prof = o; o += align_up(5 * (size_t)p->ny * sizeof(double));
     L.off_flag = o; o += align_up(sizeof(int));  // set by a staged step whose bounded wait ran out
     L.total = o;
@@ -199,10 +198,9 @@ struct lks_handle {
     int cur = 0;
     double* snap = nullptr;
     double* partial = nullptr;
-    double* dout = nullptr;
     double* prof = nullptr;
     double* state_stage = nullptr;  // 19 * min(N, 2^20) doubles for state and moment transfers, on first use
-    double* host_small = nullptr;  // pinned 8 doubles
+    double* host_small = nullptr;  // pinned (and so mapped: kernels write it) 8 doubles
     int* flag = nullptr;
     bool staged = false;              // 16-bit, nx % 8 == 0, nx >= 1024: the staged kernels
     lks::StagedStep ss = {nullptr, 0};
@@ -418,7 +416,6 @@ lks_status lks_create(const lks_params* p, lks_handle** out) {
     h->g[1] = h->base + h->L.off_gb;
     h->snap = (double*)(h->base + h->L.off_snap);
     h->partial = (double*)(h->base + h->L.off_partial);
-    h->dout = (double*)(h->base + h->L.off_out);
     h->prof = (double*)(h->base + h->L.off_prof);
     h->flag = (int*)(h->base + h->L.off_flag);
     e = cudaHostAlloc((void**)&h->host_small, 8 * sizeof(double), cudaHostAllocDefault);
@@ -561,10 +558,8 @@ lks_status lks_residual(lks_handle* h, double* r_u, double* r_b) {
     NvtxRange nvtx_range("lks_residual");
     if (!h) return fail(nullptr, LKS_EINVAL, "handle is NULL");
     cudaError_t e = lks::launch_residual(h->p.storage, h->f[h->cur], h->g[h->cur], h->p.nx, h->p.ny, h->p.B0,
-                                         h->p.Fx, h->snap, h->partial, h->dout, h->stream, h->p.coupling,
+                                         h->p.Fx, h->snap, h->partial, h->host_small, h->stream, h->p.coupling,
                                          h->p.tau_m, lks::interleave_row(h->p.storage, h->p.nx, h->p.inplace));
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(h->host_small, h->dout, 4 * sizeof(double), cudaMemcpyDeviceToHost, h->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "lks_residual");
     if (lks_status fs = staged_check(h, "lks_residual")) return fs;

@@ -161,7 +161,7 @@ cudaError_t launch_node_moments(int storage, const void* f, const void* g, int64
 
 // Residual partial sums: nblk blocks write partial[4*blk + k] = (sum du^2, sum u^2, sum db^2, sum b^2)
 // and refresh the snapshot snap[0..N) = u_x, snap[N..2N) = B_x; then one block reduces in fixed order
-// into out[0..4).  residual_blocks(N) never exceeds kResidualMaxBlocks (8 blocks per SM on 152 SMs).
+// into out[0..4), device or page-locked host memory.  residual_blocks(N) never exceeds kResidualMaxBlocks (8 blocks per SM on 152 SMs).
 constexpr int kResidualMaxBlocks = 1216;
 int residual_blocks(int64_t N);
 
