@@ -578,18 +578,25 @@ __global__ void __launch_bounds__(256) step3_flat_kernel(const S* fin, const S* 
 // each slot with one bulk copy of R' nx elements (two where the task holds a wall row and e_y != 0:
 // that row takes the node's own row of the opposite plane), one slot per lane, into one of
 // kStages3 shared-memory stages, completing on the stage's `full` barrier.  The periodic x pull is
-// an index wrap within the staged row.  Eight consumer warps take the task's nodes: 40 values from
-// shared memory, collide3, 40 stores; each warp then arrives on the stage's `empty` barrier,
-// which the producer waits for before it refills the stage, so kStages3 - 1 tasks' reads are in
-// flight while one is computed.  Each consumer thread takes two x-adjacent nodes (x even) as one
-// float2 (packed FP32 arithmetic), reading 32-bit words of the staged rows and storing one word
-// per plane.  Each slot takes a fixed kTaskNodes3 elements of a stage, so the slot offsets are
-// constants.  Rows must be 16-byte aligned: nx a multiple of 8, and nx <= kTaskNodes3.  A wait
-// that runs out (kWaitNs) sets *err and ends that warp's loop; the producer then waits, within the
-// same limit, for the last copies it issued to each stage before it returns.
+// an index wrap within the staged row.  The consumer warps take the tasks' nodes 64 at a time: a lane
+// reads its slots into registers (two x-adjacent nodes, x even, so one 32-bit word of a staged row per
+// slot), arrives on the stage's `empty` barrier, which the producer waits for before it refills the
+// stage, and then computes both nodes as one float2 (packed FP32 arithmetic), storing one word per
+// plane.  Each slot takes a fixed kTaskNodes3 elements of a stage, so the slot offsets are constants.
+// Rows must be 16-byte aligned: nx a multiple of 8, and nx <= kTaskNodes3.  A wait that runs out
+// (kWaitNs) sets *err and ends that warp's loop; the producer then waits, within the same limit, for
+// the last copies it issued to each stage before it returns.
+//
+// Bound by HBM (the copies and stores alone run at 6.44 TB/s) with 960 instructions per 64 nodes to hide
+// behind it.  Eleven consumer warps and the producer fill the SM at the 168 registers a thread that nine
+// warps are given anyway; warps held to one task's eight shares, with the stage kept until the stores,
+// left two of five stages out of flight.  256 x 128 x 96 BF16, us a step: 91.1 with eight warps a task, 91.4
+// with eleven on shares, 88.7 with stages given back early, 86.3 with the destination planes as parameters
+// (FP16 87.0).
 constexpr int kTaskNodes3 = 512;                 // nodes of a task: consumer threads x 2
-constexpr int kConsumerWarps3 = kTaskNodes3 / 64;
-constexpr int kThreads3 = kTaskNodes3 / 2 + 32;  // consumers + the producer warp
+constexpr int kItems3 = kTaskNodes3 / 64;        // a consumer warp takes 64 nodes at a time
+constexpr int kConsumerWarps3 = 11;
+constexpr int kThreads3 = (kConsumerWarps3 + 1) * 32;  // consumers + the producer warp
 constexpr int kStages3 = 5;
 constexpr int kStageElems3 = 40 * kTaskNodes3;   // a slot takes kTaskNodes3 elements of a stage
 constexpr uint64_t kWaitNs = 1000000000ull;  // 1 s
@@ -597,10 +604,14 @@ constexpr uint64_t kWaitNs = 1000000000ull;  // 1 s
 inline int rows_per_task3(int nx, int ny) { return std::max(1, std::min(ny, kTaskNodes3 / nx)); }
 inline size_t staged_smem3() { return 128 + (size_t)kStages3 * kStageElems3 * 2; }
 
+struct Planes3 {
+    void* slot[40];  // the destination planes: a store adds one 32-bit offset to a uniform base
+};
+
 template <typename S>
 __global__ void __launch_bounds__(kThreads3, 1) step3_staged_kernel(const S* __restrict__ fin, const S* __restrict__ gin,
-                                                                    S* __restrict__ fout, S* __restrict__ gout,
-                                                                    const Params3<float> p, int R, int* err) {
+                                                                    const Planes3 dst, const Params3<float> p, int R,
+                                                                    int* err) {
     extern __shared__ __align__(128) unsigned char sm3[];
     uint64_t* full = reinterpret_cast<uint64_t*>(sm3);
     uint64_t* empty = full + kStages3;
@@ -615,7 +626,7 @@ __global__ void __launch_bounds__(kThreads3, 1) step3_staged_kernel(const S* __r
     if (tid == 0) {
         for (int s = 0; s < kStages3; ++s) {
             lks::mbar_init(&full[s], 1);
-            lks::mbar_init(&empty[s], kConsumerWarps3);
+            lks::mbar_init(&empty[s], kItems3);
         }
         lks::mbar_init_fence();
     }
@@ -659,15 +670,15 @@ __global__ void __launch_bounds__(kThreads3, 1) step3_staged_kernel(const S* __r
                 const int ey = ey2[i], ez = ez2[i];
                 const int zsrc = ez == 1 ? (z == 0 ? nz - 1 : z - 1) : ez == -1 ? (z == nz - 1 ? 0 : z + 1) : z;
                 const int64_t rsrc = (int64_t)zsrc * ny, rown = (int64_t)z * ny;
-                S* dst = stage0 + s * kStageElems3 + k * kTaskNodes3;
+                S* row = stage0 + s * kStageElems3 + k * kTaskNodes3;
                 if (ey == 1 && y0 == 0) {  // row 0 is a wall row: own row 0, opposite plane
-                    lks::bulk_g2s(dst, bw[i] + rown * nx, row_bytes, &full[s]);
-                    if (Rt > 1) lks::bulk_g2s(dst + nx, bn[i] + rsrc * nx, (uint32_t)(Rt - 1) * row_bytes, &full[s]);
+                    lks::bulk_g2s(row, bw[i] + rown * nx, row_bytes, &full[s]);
+                    if (Rt > 1) lks::bulk_g2s(row + nx, bn[i] + rsrc * nx, (uint32_t)(Rt - 1) * row_bytes, &full[s]);
                 } else if (ey == -1 && y0 + Rt == ny) {  // row ny - 1 is a wall row
-                    if (Rt > 1) lks::bulk_g2s(dst, bn[i] + (rsrc + y0 + 1) * nx, (uint32_t)(Rt - 1) * row_bytes, &full[s]);
-                    lks::bulk_g2s(dst + (size_t)(Rt - 1) * nx, bw[i] + (rown + ny - 1) * nx, row_bytes, &full[s]);
+                    if (Rt > 1) lks::bulk_g2s(row, bn[i] + (rsrc + y0 + 1) * nx, (uint32_t)(Rt - 1) * row_bytes, &full[s]);
+                    lks::bulk_g2s(row + (size_t)(Rt - 1) * nx, bw[i] + (rown + ny - 1) * nx, row_bytes, &full[s]);
                 } else {
-                    lks::bulk_g2s(dst, bn[i] + (rsrc + y0 - ey) * nx, (uint32_t)Rt * row_bytes, &full[s]);
+                    lks::bulk_g2s(row, bn[i] + (rsrc + y0 - ey) * nx, (uint32_t)Rt * row_bytes, &full[s]);
                 }
             }
         }
@@ -681,46 +692,55 @@ __global__ void __launch_bounds__(kThreads3, 1) step3_staged_kernel(const S* __r
         return;
     }
 
-    // consumers: thread tid holds nodes x, x + 1 (x = 2 tid mod nx, even) of task row j = 2 tid / nx
+    // consumers: of item c of a task (nodes 64 c ..), a lane holds nodes x, x + 1 (x even) of task row j
     typedef lks::Packed<S> P;
-    const int j = (2 * tid) / nx, x = 2 * tid - j * nx;
-    const int nw = nx / 2, xw = x / 2;                        // words per row, the pair's word
-    const int xwm = xw == 0 ? nw - 1 : xw - 1, xwp = xw == nw - 1 ? 0 : xw + 1;
-    for (int64_t it = 0; it < nmine; ++it) {
-        const int s = (int)(it % kStages3);
-        if (!lks::mbar_wait_bounded(&full[s], (uint32_t)(it / kStages3) & 1u, kWaitNs)) {
+    const int nw = nx / 2;  // words per row
+    const uint32_t nitem = (uint32_t)nmine * kItems3;  // a block's share of at most 2^31 nodes' rows
+    for (uint32_t q = warp; q < nitem; q += kConsumerWarps3) {
+        const uint32_t it = q / kItems3, s = it % kStages3;
+        if (!lks::mbar_wait_bounded(&full[s], (it / kStages3) & 1u, kWaitNs)) {
             atomicExch(err, 1);
             break;
         }
-        const int64_t t = t0 + it * G;
-        const int z = (int)(t / tpp), y0 = (int)(t % tpp) * R;
-        const int y = y0 + j;
-        if (j < R && y < ny) {
-            const bool bottom = (y == 0), top = (y == ny - 1);
+        const int i = (int)(q % kItems3) * 64 + 2 * lane;
+        const int j = i / nx, x = i - j * nx;
+        const int xw = x / 2, xwm = xw == 0 ? nw - 1 : xw - 1, xwp = xw == nw - 1 ? 0 : xw + 1;
+        const uint32_t t = (uint32_t)t0 + it * (uint32_t)G;
+        const int z = (int)(t / (uint32_t)tpp), y = (int)(t % (uint32_t)tpp) * R + j;
+        const bool live = j < R && y < ny, bottom = y == 0, top = y == ny - 1;
+        // The stage is read into registers (a word holds a slot of both nodes) and given back before the
+        // arithmetic, so that the copies in flight are kStages3 tasks deep whatever that takes.
+        uint32_t w[40];
+        if (live) {
             const uint32_t* st = reinterpret_cast<const uint32_t*>(stage0 + s * kStageElems3 + j * nx);
-            const int64_t n = ((int64_t)z * ny + y) * nx + x;
-            uint32_t* fo = reinterpret_cast<uint32_t*>(fout + n);
-            uint32_t* go = reinterpret_cast<uint32_t*>(gout + n);
+#pragma unroll
+            for (int k = 0; k < 40; ++k) {
+                const int a = slot_dir3(k), ex = EXa(a), ey = EYa(a);
+                const bool wall = (ey == 1 && bottom) || (ey == -1 && top);
+                const uint32_t* row = st + k * (kTaskNodes3 / 2);
+                const uint32_t own = row[xw];
+                if (ex == 0)
+                    w[k] = own;
+                else if (ex == 1)  // x <- x - 1 (high half of the word before), x + 1 <- x
+                    w[k] = __byte_perm(row[xwm], own, 0x5432);
+                else  // x <- x + 1, x + 1 <- x + 2 (low half of the word after)
+                    w[k] = __byte_perm(own, row[xwp], 0x5432);
+                if (ex != 0 && ey != 0 && wall) w[k] = own;
+            }
+        }
+        __syncwarp();
+        if (lane == 0) lks::mbar_arrive(&empty[s]);
+        if (live) {
+            const uint32_t off = 2u * (((uint32_t)z * ny + y) * nx + x);  // bytes: at most 2^30 nodes
             // rows without a wall (all but two per z plane) take a path with no wall logic
             auto body = [&](auto walls) {
                 constexpr bool W = decltype(walls)::value;
                 auto in = [&](int k) -> float2 {
-                    const int a = slot_dir3(k), ex = EXa(a), ey = EYa(a);
-                    const bool wall = W && ((ey == 1 && bottom) || (ey == -1 && top));
-                    const uint32_t* row = st + k * (kTaskNodes3 / 2);
-                    uint32_t w;
-                    if (wall || ex == 0)
-                        w = row[xw];
-                    else if (ex == 1)  // x <- x - 1 (high half of the word before), x + 1 <- x
-                        w = __byte_perm(row[xwm], row[xw], 0x5432);
-                    else  // x <- x + 1, x + 1 <- x + 2 (low half of the word after)
-                        w = __byte_perm(row[xw], row[xwp], 0x5432);
-                    const float2 v = P::pair(w);
+                    const float2 v = P::pair(w[k]);
                     return W ? wall_in3<float2, float>(p, bottom, top, k, v) : v;
                 };
                 collide3<float2, float>(p, in, [&](int k, float2 v) {
-                    const size_t off = (size_t)slot_plane3(k, slot_dir3(k)) * (size_t)N / 2;
-                    (k < 19 ? fo : go)[off] = P::pack(v.x, v.y);
+                    *reinterpret_cast<uint32_t*>(static_cast<char*>(dst.slot[k]) + off) = P::pack(v.x, v.y);
                 });
             };
             if (bottom || top)
@@ -728,8 +748,6 @@ __global__ void __launch_bounds__(kThreads3, 1) step3_staged_kernel(const S* __r
             else
                 body(std::false_type{});
         }
-        __syncwarp();
-        if (lane == 0) lks::mbar_arrive(&empty[s]);
     }
 }
 
@@ -1024,8 +1042,11 @@ void launch_staged3(lks3_handle* h, int src, cudaStream_t st) {
     const int64_t ntask = (int64_t)p.nz * ((p.ny + R - 1) / R);
     const unsigned grid = (unsigned)std::min<int64_t>(ntask, h->staged_grid);
     const Params3<float> q = make_params3<float>(p, h->c_bot, h->c_top, h->u_bot, h->u_top);
-    lks::launch_pdl(step3_staged_kernel<S>, grid, kThreads3, staged_smem3(), st,
-        (const S*)h->f[src], (const S*)h->g[src], (S*)h->f[src ^ 1], (S*)h->g[src ^ 1], q, R, h->flag);
+    Planes3 out;
+    for (int k = 0; k < 40; ++k)
+        out.slot[k] = (S*)(k < 19 ? h->f : h->g)[src ^ 1] + slot_plane3(k, slot_dir3(k)) * q.N;
+    lks::launch_pdl(step3_staged_kernel<S>, grid, kThreads3, staged_smem3(), st, (const S*)h->f[src],
+                    (const S*)h->g[src], out, q, R, h->flag);
 }
 
 // Opt the staged kernel of the handle's storage into its shared memory and size its grid.
