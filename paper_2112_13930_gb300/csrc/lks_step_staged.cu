@@ -3,28 +3,26 @@
 // kSegX).  The pull, wall closures, collision and store as in step_node_with (lks_device.cuh), with the same per-node
 // arithmetic: the results agree bit for bit with the one- and two-node kernels.
 //
-// A task is a row segment of up to kSegX nodes (x0 .. x0 + T - 1 of row y).  For each of the 19
-// population slots (f_0..8, g_x0..4, g_y0..4) a producer warp copies, one slot per lane, the segment
-// of the row the slot pulls from (y - e_y; a link-closure wall row takes its own row of the opposite
-// plane; a moment-closure wall row fetches nothing for the slots it reconstructs) into one of the
-// shared-memory stages, with a 16-byte halo on each side for the x-shifted slots (periodic in x:
-// wrapped copies at the row ends), completing on the stage's `full` mbarrier.  Sixteen consumer
-// warps take two x-adjacent nodes per thread as one float2 (packed FP32x2 arithmetic): 19 words of
-// the staged rows (byte_perm for the x shift), the wall closure, the collision, 19 packed words
-// stored.  Each lane first copies its 19 words into its column of the warp's private scratch and
-// the warp arrives on the stage's `empty` mbarrier at once, so the producer refills the stage while
-// the warp computes from the scratch.  Every wait is bounded (kWaitNs); one that runs out sets *err and
-// ends that warp's loop, and the producer waits, within the same limit, for its last copies to each
-// stage before it returns.
+// A task is a row segment of up to kSegX nodes (x0 .. x0 + T - 1 of row y), the segments of a row of equal
+// length.  For each of the 19 population slots (f_0..8, g_x0..4, g_y0..4) a producer warp copies, one slot
+// per lane, the segment of the row the slot pulls from (y - e_y; a link-closure wall row takes its own row
+// of the opposite plane; a moment-closure wall row fetches nothing for the slots it reconstructs) into one
+// of the shared-memory stages, with a 16-byte halo on each side for the x-shifted slots (periodic in x:
+// wrapped copies at the row ends), completing on the stage's `full` mbarrier.  The consumer warps take
+// the tasks' nodes 64 at a time: a lane reads 19 words (two x-adjacent nodes; byte_perm for the x shift)
+// into registers, the warp arrives on the stage's `empty` mbarrier, so that the producer refills it
+// while the warp computes, and then come the wall closure, the collision as one float2 (packed FP32x2
+// arithmetic) and 19 packed words stored.  Rows without a wall run a path with no closure code.  Every
+// wait is bounded (kWaitNs); one that runs out sets *err and ends that warp's loop, and the producer
+// waits, within the same limit, for its last copies to each stage before it returns.
 //
-// One block of 16 consumer warps per SM with 1024-node tasks (2 KB copies) beat two blocks of 8
-// warps with 512-node tasks at 4096^2: 76-80 against 71-72 GLUPS (the copies per byte halve).  Rows
-// without a wall run a compile-time path without the closure code (BF16, moment closure: 79.8
-// against 76.1 GLUPS).  Releasing the stage as soon as the words are read, through the per-warp
-// scratch (four stages instead of five): BF16 82.8, FP16 80.0 GLUPS against 79.4 and 78.8 with the
-// release after the stores.  Holding the words in registers across the release instead spilled at
-// the 96 registers a thread of this block has (BF16 78.0, FP16 78.7); a whole producer warpgroup
-// that moved registers to the consumers with setmaxnreg (32 / 112) ran at 73.4.
+// Bound by memory (76 bytes a node and step) and by how evenly the block's warps are kept at it.  With
+// sixteen warps tied to the sixteen 64-node shares of a task, a row of 2056 nodes left a third of the
+// tasks four words long; and 17 warps have 96 registers, too few to hold the words, so they went through
+// a scratch area.  Fifteen warps and the producer have 128.  Three stages: two starve the warps, four and
+// five put more reads among the writes than DRAM likes.  us a step, before -> after: BF16 in place
+// 2056 x 1500 46.2 -> 42.7, 4096^2 205.5 -> 204.0 (two stages 223, five 214.5), 3000^2 113.8 -> 113.0
+// (126, 118); two buffers 1024 x 1000 16.1 -> 14.3, 4096 x 150 10.7 -> 9.8, 2056 x 400 FP16 16.7 -> 14.3.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -40,23 +38,51 @@
 namespace lks {
 namespace {
 
-constexpr int kSegX = 1024;                      // nodes of a task: consumer threads x 2
+constexpr int kSegX = 1024;                      // nodes of a task, at most
 constexpr int kHaloW = 4;                        // halo words (8 elements = 16 bytes) per side
 constexpr int kSlotW = kSegX / 2 + 2 * kHaloW;   // words of a staged slot row
 constexpr int kSlots = 19;
-constexpr int kStages = 5;
+constexpr int kStages = 3;
 constexpr int kStageW = kSlots * kSlotW;
-constexpr int kConsumerWarps = kSegX / 64;
-constexpr int kThreads = kSegX / 2 + 32;         // consumers + the producer warp
+constexpr int kConsumerWarps = 15;
+constexpr int kThreads = (kConsumerWarps + 1) * 32;  // consumers + the producer warp
 constexpr uint64_t kWaitNs = 1000000000ull;      // 1 s
 constexpr size_t kSmem = 128 + (size_t)kStages * kStageW * 4;
-// Both kernels: four stages, and behind them a private scratch area per consumer warp into which each
-// lane copies its 19 staged words, so that the warp can hand its stage back at once (the in-place
-// phase 0 with it: BF16 81.8, FP16 83.0 GLUPS per pair of steps against 80.9 and 80.5).
-constexpr int kStagesTB = 4;
-constexpr int kScratchW = kSlots * 32;  // words per consumer warp
-constexpr size_t kSmemTB = 128 + (size_t)kStagesTB * kStageW * 4 + (size_t)kConsumerWarps * kScratchW * 4;
-static_assert(kSmemTB <= 227 * 1024, "shared memory per block");
+static_assert(kSmem <= 227 * 1024, "shared memory per block");
+
+// The destination planes: a store adds one 32-bit offset to a uniform base.
+struct SlotPlanes {
+    void* slot[kSlots];
+};
+__device__ __forceinline__ void put_word(const SlotPlanes& d, int k, uint32_t byte, uint32_t v) {
+    *reinterpret_cast<uint32_t*>(static_cast<char*>(d.slot[k]) + byte) = v;
+}
+
+// Segments of a row: as few as kSegX allows, of equal length in items (64 nodes, or 32 words).
+struct Segments {
+    int n, items;  // segments per row, items per segment
+};
+inline Segments segments_of(int nx) {
+    const int n = (nx + kSegX - 1) / kSegX;
+    return {n, ((nx + n - 1) / n + 63) / 64};
+}
+
+// A consumer warp's walk over the items of its block's tasks t0, t0 + G, ...: every kConsumerWarps-th item.
+struct ItemWalk {
+    uint32_t it;  // task of the block
+    int c, y, g;  // item of the task, the task's row and segment
+    __device__ __forceinline__ ItemWalk(int warp, int nseg) : it(0), c(warp), y(blockIdx.x / nseg), g(blockIdx.x % nseg) {}
+    __device__ __forceinline__ bool next(uint32_t ntask, const Segments& sg, int dy, int dg) {
+        while (c >= sg.items) {
+            c -= sg.items;
+            ++it;
+            y += dy;
+            g += dg;
+            if (g >= sg.n) g -= sg.n, ++y;
+        }
+        return it < ntask;
+    }
+};
 
 // D2Q9 (f) and D2Q5 (g) directions of slot k: k < 9 is f_k, 9..13 is g_x,k-9, 14..18 is g_y,k-14.
 __host__ __device__ constexpr int dir_of(int k) { return k < 9 ? k : (k < 14 ? k - 9 : k - 14); }
@@ -68,23 +94,23 @@ __host__ __device__ constexpr int plane_of(int k, int a) { return k < 9 ? a : (k
 
 template <typename S, int CLOSURE, int COUPLING>
 __global__ void __launch_bounds__(kThreads, 1) step_kernel_staged(const S* __restrict__ fin, const S* __restrict__ gin,
-                                                                   S* __restrict__ fout, S* __restrict__ gout,
-                                                                   const StepParams<float> p, int* err) {
+                                                                   const SlotPlanes out, const StepParams<float> p,
+                                                                   const Segments sg, int* err) {
     extern __shared__ __align__(128) unsigned char sm[];
     uint64_t* full = reinterpret_cast<uint64_t*>(sm);
-    uint64_t* empty = full + kStagesTB;
+    uint64_t* empty = full + kStages;
     uint32_t* stage0 = reinterpret_cast<uint32_t*>(sm + 128);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int nx = p.nx, ny = p.ny;
     const int64_t N = p.N;
-    const int nseg = (nx + kSegX - 1) / kSegX;
+    const int nseg = sg.n, seg = 64 * sg.items;
     const int64_t ntask = (int64_t)ny * nseg;
     const int64_t G = gridDim.x, t0 = blockIdx.x;
     const int64_t nmine = t0 < ntask ? (ntask - 1 - t0) / G + 1 : 0;  // tasks t0, t0 + G, ...
     if (tid == 0) {
-        for (int s = 0; s < kStagesTB; ++s) {
+        for (int s = 0; s < kStages; ++s) {
             mbar_init(&full[s], 1);
-            mbar_init(&empty[s], kConsumerWarps);
+            mbar_init(&empty[s], sg.items);
         }
         mbar_init_fence();
     }
@@ -99,15 +125,15 @@ __global__ void __launch_bounds__(kThreads, 1) step_kernel_staged(const S* __res
         const S* bw = base + (int64_t)plane_of(k, opp9(a)) * N;  // the opposite one (link walls)
         int64_t it = 0;
         for (; it < nmine; ++it) {
-            const int s = (int)(it % kStagesTB);
-            const int64_t u = it / kStagesTB;
+            const int s = (int)(it % kStages);
+            const int64_t u = it / kStages;
             if (u > 0 && !mbar_wait_bounded(&empty[s], (uint32_t)(u - 1) & 1u, kWaitNs)) {
                 if (lane == 0) atomicExch(err, 1);
                 break;
             }
             const int64_t t = t0 + it * G;
-            const int y = (int)(t / nseg), x0 = (int)(t % nseg) * kSegX;
-            const int T = min(kSegX, nx - x0);
+            const int y = (int)(t / nseg), x0 = (int)(t % nseg) * seg;
+            const int T = min(seg, nx - x0);
             const bool wall = (ey == 1 && y == 0) || (ey == -1 && y == ny - 1);
             uint32_t* dst = stage0 + s * kStageW + k * kSlotW;
             // this lane's copies: (global element offset, shared word offset, elements)
@@ -144,61 +170,55 @@ __global__ void __launch_bounds__(kThreads, 1) step_kernel_staged(const S* __res
         }
         // no copy may be left in flight into this block's shared memory: wait for the last phase
         // issued to each stage (already complete unless a consumer gave up)
-        for (int s = 0; s < kStagesTB; ++s) {
+        for (int s = 0; s < kStages; ++s) {
             if (it <= s) continue;
-            const int64_t u_last = (it - 1 - s) / kStagesTB;
+            const int64_t u_last = (it - 1 - s) / kStages;
             if (!mbar_wait_bounded(&full[s], (uint32_t)u_last & 1u, kWaitNs) && lane == 0) atomicExch(err, 1);
         }
         return;
     }
 
-    // consumers: thread tid holds nodes x0 + 2 tid and x0 + 2 tid + 1 of the task's row
-    uint32_t* scr = stage0 + kStagesTB * kStageW + warp * kScratchW;
+    // consumers: of item c of a task, a lane holds nodes x0 + 64 c + 2 lane and the next
     typedef Packed<S> P;
-    const int xw = kHaloW + tid;
-    for (int64_t it = 0; it < nmine; ++it) {
-        const int s = (int)(it % kStagesTB);
-        if (!mbar_wait_bounded(&full[s], (uint32_t)(it / kStagesTB) & 1u, kWaitNs)) {
+    const int dy = (int)(G / nseg), dg = (int)(G % nseg);
+    ItemWalk i(warp, nseg);
+    for (; i.next((uint32_t)nmine, sg, dy, dg); i.c += kConsumerWarps) {
+        const uint32_t s = i.it % kStages;
+        if (!mbar_wait_bounded(&full[s], (i.it / kStages) & 1u, kWaitNs)) {
             atomicExch(err, 1);
             break;
         }
-        const int64_t t = t0 + it * G;
-        const int y = (int)(t / nseg), x0 = (int)(t % nseg) * kSegX;
-        const int T = min(kSegX, nx - x0);
-        const bool active = 2 * tid < T;
+        const int y = i.y, x = i.g * seg + 64 * i.c + 2 * lane;
+        const bool active = x < nx;
         {
             const bool bottom = (y == 0), top = (y == ny - 1);
-            const uint32_t* st = stage0 + s * kStageW;
+            const uint32_t* st = stage0 + s * kStageW + kHaloW + 32 * i.c + lane;
             // rows without a wall (all but two) take a path with no closure code
             auto body = [&](auto walls) {
                 constexpr bool W = decltype(walls)::value;
+                uint32_t u[kSlots];
                 if (active) {
 #pragma unroll
                     for (int k = 0; k < kSlots; ++k) {
                         const int a = dir_of(k), ex = ex9(a), ey = ey9(a);
                         const bool wall = W && ((ey == 1 && bottom) || (ey == -1 && top));
                         const uint32_t* row = st + k * kSlotW;
-                        uint32_t w;
                         if (wall || ex == 0)
-                            w = row[xw];
+                            u[k] = row[0];
                         else if (ex == 1)  // x <- x - 1 (high half of the word before), x + 1 <- x
-                            w = __byte_perm(row[xw - 1], row[xw], 0x5432);
+                            u[k] = __byte_perm(row[-1], row[0], 0x5432);
                         else  // x <- x + 1, x + 1 <- x + 2 (low half of the word after)
-                            w = __byte_perm(row[xw], row[xw + 1], 0x5432);
-                        scr[k * 32 + lane] = w;  // this lane's column of the warp's scratch
+                            u[k] = __byte_perm(row[0], row[1], 0x5432);
                     }
                 }
-                // the warp's words are in its scratch: the stage goes back to the producer before the
+                // the words are in registers: the stage goes back to the producer before the
                 // collision and the stores
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&empty[s]);
                 if (!active) return;
                 float2 v[kSlots];
 #pragma unroll
-                for (int k = 0; k < kSlots; ++k) {
-                    const uint32_t w = scr[k * 32 + lane];
-                    v[k] = P::pair(w);
-                }
+                for (int k = 0; k < kSlots; ++k) v[k] = P::pair(u[k]);
                 float2 f[9], gx[5], gy[5];
 #pragma unroll
                 for (int a = 0; a < 9; ++a) f[a] = v[a];
@@ -226,16 +246,13 @@ __global__ void __launch_bounds__(kThreads, 1) step_kernel_staged(const S* __res
                 }
                 // moment closure, moments, equilibria and collision for both nodes
                 close_collide_pair<CLOSURE, COUPLING, W>(f, gx, gy, p, bottom, top);
-                const int64_t q = ((int64_t)y * nx + x0) / 2 + tid;  // the pair's word in every plane
-                uint32_t* fo = reinterpret_cast<uint32_t*>(fout);
-                uint32_t* go = reinterpret_cast<uint32_t*>(gout);
-                const int64_t NP = N / 2;
+                const uint32_t q = 2u * ((uint32_t)y * nx + x);  // bytes: at most 2^30 nodes
 #pragma unroll
-                for (int a = 0; a < 9; ++a) fo[a * NP + q] = P::pack(f[a].x, f[a].y);
+                for (int a = 0; a < 9; ++a) put_word(out, a, q, P::pack(f[a].x, f[a].y));
 #pragma unroll
-                for (int a = 0; a < 5; ++a) go[a * NP + q] = P::pack(gx[a].x, gx[a].y);
+                for (int a = 0; a < 5; ++a) put_word(out, 9 + a, q, P::pack(gx[a].x, gx[a].y));
 #pragma unroll
-                for (int a = 0; a < 5; ++a) go[(5 + a) * NP + q] = P::pack(gy[a].x, gy[a].y);
+                for (int a = 0; a < 5; ++a) put_word(out, 14 + a, q, P::pack(gy[a].x, gy[a].y));
             };
             if (bottom || top)
                 body(std::true_type{});
@@ -245,11 +262,10 @@ __global__ void __launch_bounds__(kThreads, 1) step_kernel_staged(const S* __res
     }
 }
 
-
 // Phase 0 of the in-place pair of steps (lks_aa.cuh) for 16-bit storage, staged the same way.  The
 // rows are interleaved (32-bit word w of a row holds nodes x = w and x = w + nx/2), so a shift by one
 // node is a shift by one word, with the two halves swapped across the periodic row edge.  A task is
-// kSegX/2 words of one row; the producer stages, for each slot, the words the task's nodes pull from
+// up to kSegX/2 words of one row; the producer stages, for each slot, the words the task's nodes pull from
 // (row y - e_y; link wall rows their own row of the opposite plane; moment wall rows nothing) with
 // 16-byte halos as above.  Each consumer thread takes one word (two nodes), collides them as a
 // float2 and pushes every direction b into plane bbar at x + e_b (a direction that would leave
@@ -258,26 +274,26 @@ __global__ void __launch_bounds__(kThreads, 1) step_kernel_staged(const S* __res
 // that node (its push of direction cbar), after its read; halo words a task stages but does not use
 // belong to other nodes, and it never writes them.
 template <typename S, int CLOSURE, int COUPLING>
-__global__ void __launch_bounds__(kThreads, 1) step_kernel_aa_staged(S* __restrict__ fb, S* __restrict__ gb,
-                                                                      const StepParams<float> p, int* err) {
+__global__ void __launch_bounds__(kThreads, 1) step_kernel_aa_staged(const S* fb, const S* gb,
+                                                                      const SlotPlanes out, const StepParams<float> p,
+                                                                      const Segments sg, int* err) {
     extern __shared__ __align__(128) unsigned char sm[];
     uint64_t* full = reinterpret_cast<uint64_t*>(sm);
-    uint64_t* empty = full + kStagesTB;
+    uint64_t* empty = full + kStages;
     uint32_t* stage0 = reinterpret_cast<uint32_t*>(sm + 128);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int ny = p.ny, H = p.nx / 2;              // words per row
     const int64_t NP = p.N / 2;                     // words per plane
-    constexpr int kSegW = kSegX / 2;
-    const int nseg = (H + kSegW - 1) / kSegW;
+    const int nseg = sg.n, segw = 32 * sg.items;
     const int64_t ntask = (int64_t)ny * nseg;
     const int64_t G = gridDim.x, t0 = blockIdx.x;
     const int64_t nmine = t0 < ntask ? (ntask - 1 - t0) / G + 1 : 0;
-    uint32_t* fw = reinterpret_cast<uint32_t*>(fb);
-    uint32_t* gw = reinterpret_cast<uint32_t*>(gb);
+    const uint32_t* fw = reinterpret_cast<const uint32_t*>(fb);
+    const uint32_t* gw = reinterpret_cast<const uint32_t*>(gb);
     if (tid == 0) {
-        for (int s = 0; s < kStagesTB; ++s) {
+        for (int s = 0; s < kStages; ++s) {
             mbar_init(&full[s], 1);
-            mbar_init(&empty[s], kConsumerWarps);
+            mbar_init(&empty[s], sg.items);
         }
         mbar_init_fence();
     }
@@ -292,15 +308,15 @@ __global__ void __launch_bounds__(kThreads, 1) step_kernel_aa_staged(S* __restri
         const uint32_t* bw = base + (int64_t)plane_of(k, opp9(a)) * NP;
         int64_t it = 0;
         for (; it < nmine; ++it) {
-            const int s = (int)(it % kStagesTB);
-            const int64_t u = it / kStagesTB;
+            const int s = (int)(it % kStages);
+            const int64_t u = it / kStages;
             if (u > 0 && !mbar_wait_bounded(&empty[s], (uint32_t)(u - 1) & 1u, kWaitNs)) {
                 if (lane == 0) atomicExch(err, 1);
                 break;
             }
             const int64_t t = t0 + it * G;
-            const int y = (int)(t / nseg), w0 = (int)(t % nseg) * kSegW;
-            const int TW = min(kSegW, H - w0);
+            const int y = (int)(t / nseg), w0 = (int)(t % nseg) * segw;
+            const int TW = min(segw, H - w0);
             const bool wall = (ey == 1 && y == 0) || (ey == -1 && y == ny - 1);
             uint32_t* dst = stage0 + s * kStageW + k * kSlotW;
             // this lane's copies: (global word offset, shared word offset, words)
@@ -331,49 +347,45 @@ __global__ void __launch_bounds__(kThreads, 1) step_kernel_aa_staged(S* __restri
             if (n1) bulk_g2s(dst + d1, src + g1, 4u * n1, &full[s]);
             if (n2) bulk_g2s(dst + d2, src + g2, 4u * n2, &full[s]);
         }
-        for (int s = 0; s < kStagesTB; ++s) {
+        for (int s = 0; s < kStages; ++s) {
             if (it <= s) continue;
-            const int64_t u_last = (it - 1 - s) / kStagesTB;
+            const int64_t u_last = (it - 1 - s) / kStages;
             if (!mbar_wait_bounded(&full[s], (uint32_t)u_last & 1u, kWaitNs) && lane == 0) atomicExch(err, 1);
         }
         return;
     }
 
-    uint32_t* scr = stage0 + kStagesTB * kStageW + warp * kScratchW;
     typedef Packed<S> P;
-    const int xw = kHaloW + tid;
-    for (int64_t it = 0; it < nmine; ++it) {
-        const int s = (int)(it % kStagesTB);
-        if (!mbar_wait_bounded(&full[s], (uint32_t)(it / kStagesTB) & 1u, kWaitNs)) {
+    const int dy = (int)(G / nseg), dg = (int)(G % nseg);
+    ItemWalk i(warp, nseg);
+    for (; i.next((uint32_t)nmine, sg, dy, dg); i.c += kConsumerWarps) {
+        const uint32_t s = i.it % kStages;
+        if (!mbar_wait_bounded(&full[s], (i.it / kStages) & 1u, kWaitNs)) {
             atomicExch(err, 1);
             break;
         }
-        const int64_t t = t0 + it * G;
-        const int y = (int)(t / nseg), w0 = (int)(t % nseg) * kSegW;
-        const int TW = min(kSegW, H - w0);
-        const bool active = tid < TW;
+        const int y = i.y, w = i.g * segw + 32 * i.c + lane;  // the lane's word in its row
+        const bool active = w < H;
         {
             const bool bottom = (y == 0), top = (y == ny - 1);
-            const uint32_t* st = stage0 + s * kStageW;
-            const int w = w0 + tid;                           // the thread's word in its row
+            const uint32_t* st = stage0 + s * kStageW + kHaloW + 32 * i.c + lane;
             const bool sm = (w == 0), sp = (w == H - 1);      // halves swap across the row edge
             const int wm = sm ? H - 1 : w - 1, wp = sp ? 0 : w + 1;
             auto body = [&](auto walls) {
                 constexpr bool W = decltype(walls)::value;
+                uint32_t u[kSlots];
                 if (active) {
 #pragma unroll
                     for (int k = 0; k < kSlots; ++k) {
                         const int a = dir_of(k), ex = ex9(a), ey = ey9(a);
                         const bool wall = W && ((ey == 1 && bottom) || (ey == -1 && top));
                         const uint32_t* row = st + k * kSlotW;
-                        uint32_t u;
                         if (wall || ex == 0)
-                            u = row[xw];
+                            u[k] = row[0];
                         else if (ex == 1)  // nodes x - 1: the word before (swapped across the left edge)
-                            u = sm ? __byte_perm(row[xw - 1], 0, 0x1032) : row[xw - 1];
+                            u[k] = sm ? __byte_perm(row[-1], 0, 0x1032) : row[-1];
                         else  // nodes x + 1: the word after (swapped across the right edge)
-                            u = sp ? __byte_perm(row[xw + 1], 0, 0x1032) : row[xw + 1];
-                        scr[k * 32 + lane] = u;
+                            u[k] = sp ? __byte_perm(row[1], 0, 0x1032) : row[1];
                     }
                 }
                 // release the stage at once, as the two-buffer kernel does
@@ -382,10 +394,7 @@ __global__ void __launch_bounds__(kThreads, 1) step_kernel_aa_staged(S* __restri
                 if (!active) return;
                 float2 v[kSlots];
 #pragma unroll
-                for (int k = 0; k < kSlots; ++k) {
-                    const uint32_t u = scr[k * 32 + lane];
-                    v[k] = P::pair(u);
-                }
+                for (int k = 0; k < kSlots; ++k) v[k] = P::pair(u[k]);
                 float2 f[9], gx[5], gy[5];
 #pragma unroll
                 for (int a = 0; a < 9; ++a) f[a] = v[a];
@@ -412,42 +421,44 @@ __global__ void __launch_bounds__(kThreads, 1) step_kernel_aa_staged(S* __restri
                 }
                 close_collide_pair<CLOSURE, COUPLING, W>(f, gx, gy, p, bottom, top);
                 // push: direction b -> plane bbar at x + e_b; through a wall -> plane b, own word
-                const int64_t rc = (int64_t)y * H, rs = rc - H, rn = rc + H;
-                auto put = [&](uint32_t* at, bool swap, float2 q) { *at = swap ? P::pack(q.y, q.x) : P::pack(q.x, q.y); };
-                put(fw + 0 * NP + rc + w, false, f[0]);
-                put(fw + 3 * NP + rc + wp, sp, f[1]);
-                put(fw + 1 * NP + rc + wm, sm, f[3]);
-                put(gw + 0 * NP + rc + w, false, gx[0]);
-                put(gw + 3 * NP + rc + wp, sp, gx[1]);
-                put(gw + 1 * NP + rc + wm, sm, gx[3]);
-                put(gw + 5 * NP + rc + w, false, gy[0]);
-                put(gw + 8 * NP + rc + wp, sp, gy[1]);
-                put(gw + 6 * NP + rc + wm, sm, gy[3]);
+                const uint32_t rc = (uint32_t)y * H, rs = rc - H, rn = rc + H;
+                auto put = [&](int k, uint32_t at, bool swap, float2 q) {
+                    put_word(out, k, 4u * at, swap ? P::pack(q.y, q.x) : P::pack(q.x, q.y));
+                };
+                put(0, rc + w, false, f[0]);
+                put(3, rc + wp, sp, f[1]);
+                put(1, rc + wm, sm, f[3]);
+                put(9, rc + w, false, gx[0]);
+                put(12, rc + wp, sp, gx[1]);
+                put(10, rc + wm, sm, gx[3]);
+                put(14, rc + w, false, gy[0]);
+                put(17, rc + wp, sp, gy[1]);
+                put(15, rc + wm, sm, gy[3]);
                 if (!top) {
-                    put(fw + 4 * NP + rn + w, false, f[2]);
-                    put(fw + 7 * NP + rn + wp, sp, f[5]);
-                    put(fw + 8 * NP + rn + wm, sm, f[6]);
-                    put(gw + 4 * NP + rn + w, false, gx[2]);
-                    put(gw + 9 * NP + rn + w, false, gy[2]);
+                    put(4, rn + w, false, f[2]);
+                    put(7, rn + wp, sp, f[5]);
+                    put(8, rn + wm, sm, f[6]);
+                    put(13, rn + w, false, gx[2]);
+                    put(18, rn + w, false, gy[2]);
                 } else {
-                    put(fw + 2 * NP + rc + w, false, f[2]);
-                    put(fw + 5 * NP + rc + w, false, f[5]);
-                    put(fw + 6 * NP + rc + w, false, f[6]);
-                    put(gw + 2 * NP + rc + w, false, gx[2]);
-                    put(gw + 7 * NP + rc + w, false, gy[2]);
+                    put(2, rc + w, false, f[2]);
+                    put(5, rc + w, false, f[5]);
+                    put(6, rc + w, false, f[6]);
+                    put(11, rc + w, false, gx[2]);
+                    put(16, rc + w, false, gy[2]);
                 }
                 if (!bottom) {
-                    put(fw + 2 * NP + rs + w, false, f[4]);
-                    put(fw + 5 * NP + rs + wm, sm, f[7]);
-                    put(fw + 6 * NP + rs + wp, sp, f[8]);
-                    put(gw + 2 * NP + rs + w, false, gx[4]);
-                    put(gw + 7 * NP + rs + w, false, gy[4]);
+                    put(2, rs + w, false, f[4]);
+                    put(5, rs + wm, sm, f[7]);
+                    put(6, rs + wp, sp, f[8]);
+                    put(11, rs + w, false, gx[4]);
+                    put(16, rs + w, false, gy[4]);
                 } else {
-                    put(fw + 4 * NP + rc + w, false, f[4]);
-                    put(fw + 7 * NP + rc + w, false, f[7]);
-                    put(fw + 8 * NP + rc + w, false, f[8]);
-                    put(gw + 4 * NP + rc + w, false, gx[4]);
-                    put(gw + 9 * NP + rc + w, false, gy[4]);
+                    put(4, rc + w, false, f[4]);
+                    put(7, rc + w, false, f[7]);
+                    put(8, rc + w, false, f[8]);
+                    put(13, rc + w, false, gx[4]);
+                    put(18, rc + w, false, gy[4]);
                 }
             };
             if (bottom || top)
@@ -489,52 +500,48 @@ cudaError_t prepare_typed(int inplace, int* blocks) {
     int b[4] = {0, 0, 0, 0};
     cudaError_t e;
     if (inplace) {
-        e = prepare_kernel(step_kernel_aa_staged<S, 0, 0>, &b[0], kSmemTB);
-        if (e == cudaSuccess) e = prepare_kernel(step_kernel_aa_staged<S, 1, 0>, &b[1], kSmemTB);
-        if (e == cudaSuccess) e = prepare_kernel(step_kernel_aa_staged<S, 0, 1>, &b[2], kSmemTB);
-        if (e == cudaSuccess) e = prepare_kernel(step_kernel_aa_staged<S, 1, 1>, &b[3], kSmemTB);
+        e = prepare_kernel(step_kernel_aa_staged<S, 0, 0>, &b[0], kSmem);
+        if (e == cudaSuccess) e = prepare_kernel(step_kernel_aa_staged<S, 1, 0>, &b[1], kSmem);
+        if (e == cudaSuccess) e = prepare_kernel(step_kernel_aa_staged<S, 0, 1>, &b[2], kSmem);
+        if (e == cudaSuccess) e = prepare_kernel(step_kernel_aa_staged<S, 1, 1>, &b[3], kSmem);
     } else {
-        e = prepare_kernel(step_kernel_staged<S, 0, 0>, &b[0], kSmemTB);
-        if (e == cudaSuccess) e = prepare_kernel(step_kernel_staged<S, 1, 0>, &b[1], kSmemTB);
-        if (e == cudaSuccess) e = prepare_kernel(step_kernel_staged<S, 0, 1>, &b[2], kSmemTB);
-        if (e == cudaSuccess) e = prepare_kernel(step_kernel_staged<S, 1, 1>, &b[3], kSmemTB);
+        e = prepare_kernel(step_kernel_staged<S, 0, 0>, &b[0], kSmem);
+        if (e == cudaSuccess) e = prepare_kernel(step_kernel_staged<S, 1, 0>, &b[1], kSmem);
+        if (e == cudaSuccess) e = prepare_kernel(step_kernel_staged<S, 0, 1>, &b[2], kSmem);
+        if (e == cudaSuccess) e = prepare_kernel(step_kernel_staged<S, 1, 1>, &b[3], kSmem);
     }
     *blocks = std::min(std::min(b[0], b[1]), std::min(b[2], b[3]));
     return e;
 }
 
 template <typename S>
+SlotPlanes planes_of(S* f, S* g, int64_t N) {
+    SlotPlanes d;
+    for (int k = 0; k < kSlots; ++k) d.slot[k] = k < 9 ? f + k * N : g + (k - 9) * N;
+    return d;
+}
+
+template <typename S>
 void launch_typed_aa_staged(void* f, void* g, const StepParams<float>& p, int closure, const StagedStep& ss,
                             cudaStream_t st) {
-    const int64_t ntask = (int64_t)p.ny * ((p.nx / 2 + kSegX / 2 - 1) / (kSegX / 2));
-    const unsigned grid = (unsigned)std::min<int64_t>(ntask, ss.grid);
+    const Segments sg = segments_of(p.nx);
+    const unsigned grid = (unsigned)std::min<int64_t>((int64_t)p.ny * sg.n, ss.grid);
     S* fb = (S*)f;
     S* gb = (S*)g;
-    if (p.coupling == 0) {
-        if (closure == 0) launch_pdl(step_kernel_aa_staged<S, 0, 0>, grid, kThreads, kSmemTB, st, fb, gb, p, ss.err);
-        else launch_pdl(step_kernel_aa_staged<S, 1, 0>, grid, kThreads, kSmemTB, st, fb, gb, p, ss.err);
-    } else {
-        if (closure == 0) launch_pdl(step_kernel_aa_staged<S, 0, 1>, grid, kThreads, kSmemTB, st, fb, gb, p, ss.err);
-        else launch_pdl(step_kernel_aa_staged<S, 1, 1>, grid, kThreads, kSmemTB, st, fb, gb, p, ss.err);
-    }
+    const auto kernel = p.coupling == 0 ? (closure == 0 ? step_kernel_aa_staged<S, 0, 0> : step_kernel_aa_staged<S, 1, 0>)
+                                        : (closure == 0 ? step_kernel_aa_staged<S, 0, 1> : step_kernel_aa_staged<S, 1, 1>);
+    launch_pdl(kernel, grid, kThreads, kSmem, st, (const S*)fb, (const S*)gb, planes_of(fb, gb, p.N), p, sg, ss.err);
 }
 
 template <typename S>
 void launch_typed_staged(const void* fin, const void* gin, void* fout, void* gout, const StepParams<float>& p,
                          int closure, const StagedStep& ss, cudaStream_t st) {
-    const int64_t ntask = (int64_t)p.ny * ((p.nx + kSegX - 1) / kSegX);
-    const unsigned grid = (unsigned)std::min<int64_t>(ntask, ss.grid);
-    const S* fi = (const S*)fin;
-    const S* gi = (const S*)gin;
-    S* fo = (S*)fout;
-    S* go = (S*)gout;
-    if (p.coupling == 0) {
-        if (closure == 0) launch_pdl(step_kernel_staged<S, 0, 0>, grid, kThreads, kSmemTB, st, fi, gi, fo, go, p, ss.err);
-        else launch_pdl(step_kernel_staged<S, 1, 0>, grid, kThreads, kSmemTB, st, fi, gi, fo, go, p, ss.err);
-    } else {
-        if (closure == 0) launch_pdl(step_kernel_staged<S, 0, 1>, grid, kThreads, kSmemTB, st, fi, gi, fo, go, p, ss.err);
-        else launch_pdl(step_kernel_staged<S, 1, 1>, grid, kThreads, kSmemTB, st, fi, gi, fo, go, p, ss.err);
-    }
+    const Segments sg = segments_of(p.nx);
+    const unsigned grid = (unsigned)std::min<int64_t>((int64_t)p.ny * sg.n, ss.grid);
+    const auto kernel = p.coupling == 0 ? (closure == 0 ? step_kernel_staged<S, 0, 0> : step_kernel_staged<S, 1, 0>)
+                                        : (closure == 0 ? step_kernel_staged<S, 0, 1> : step_kernel_staged<S, 1, 1>);
+    launch_pdl(kernel, grid, kThreads, kSmem, st, (const S*)fin, (const S*)gin, planes_of((S*)fout, (S*)gout, p.N), p,
+               sg, ss.err);
 }
 
 }  // namespace
