@@ -158,6 +158,7 @@ StepParams<double> make_step_params(int nx, int ny, int closure, double tau_f, d
     s.sw5 = s.src_coef * 3.0 * Fx * (1.0 / 36.0);
     s.src3 = 3.0 * s.src_coef;
     s.ov = s.omega_f / 36.0;
+    s.kl = 3.0 * s.src_coef / 36.0;
     s.kv = 3.0 * s.src_coef * Fx / 36.0;
     s.cm = 0.25 * s.omega_f;
     s.coupling = coupling;

@@ -86,7 +86,7 @@ __device__ __forceinline__ StepParams<C> to_compute(const StepParams<double>& d)
     o.owm0 = (C)d.owm0; o.owm1 = (C)d.owm1;
     o.sw0 = (C)d.sw0; o.sw1 = (C)d.sw1; o.sw5 = (C)d.sw5;
     o.src3 = (C)d.src3; o.coupling = d.coupling;
-    if constexpr (sizeof(C) == 8) o.ov = d.ov, o.kv = d.kv, o.cm = d.cm;
+    if constexpr (sizeof(C) == 8) o.ov = d.ov, o.kv = d.kv, o.cm = d.cm, o.kl = d.kl;
     o.bot.r = (C)d.bot.r; o.bot.bc = (C)d.bot.bc; o.bot.kx = (C)d.bot.kx; o.bot.du = (C)d.bot.du; o.bot.U = (C)d.bot.U;
     o.top.r = (C)d.top.r; o.top.bc = (C)d.top.bc; o.top.kx = (C)d.top.kx; o.top.du = (C)d.top.du; o.top.U = (C)d.top.U;
     return o;
