@@ -592,12 +592,12 @@ __global__ void __launch_bounds__(256) step3_flat_kernel(const S* fin, const S* 
 // warps are given anyway; warps held to one task's eight shares, with the stage kept until the stores,
 // left two of five stages out of flight.  256 x 128 x 96 BF16, us a step: 91.1 with eight warps a task, 91.4
 // with eleven on shares, 88.7 with stages given back early, 86.3 with the destination planes as parameters
-// (FP16 87.0).
+// and 85.6 with four stages instead of five (three: 86.3).  FP16 85.5; 256^3 BF16 424, with five stages 428.
 constexpr int kTaskNodes3 = 512;                 // nodes of a task: consumer threads x 2
 constexpr int kItems3 = kTaskNodes3 / 64;        // a consumer warp takes 64 nodes at a time
 constexpr int kConsumerWarps3 = 11;
 constexpr int kThreads3 = (kConsumerWarps3 + 1) * 32;  // consumers + the producer warp
-constexpr int kStages3 = 5;
+constexpr int kStages3 = 4;
 constexpr int kStageElems3 = 40 * kTaskNodes3;   // a slot takes kTaskNodes3 elements of a stage
 constexpr uint64_t kWaitNs = 1000000000ull;  // 1 s
 
