@@ -1,7 +1,7 @@
 """Benchmark of the fused LKS-MHD collide-stream step on GB300.
 
 Default workload (one "step" = one time step of the whole lattice: pull-stream, wall closures,
-moments, equilibria, collision and store in one fused kernel): shear-driven Hartmann-Couette channel, 4096 x 4096 nodes, periodic in x,
+moments, equilibria, collision and store, three of them per pass of the fused row kernel): shear-driven Hartmann-Couette channel, 4096 x 4096 nodes, periodic in x,
 moment-based Shercliff closure on both walls (c = 1), top wall at U_w = 0.05, Ha = 20,
 tau_f = tau_m = 0.8, rest start, FP32 deviation storage.  Inputs (2.5 GB of populations) are far
 larger than the 129 MB L2, so no flush is needed between steps.
@@ -86,6 +86,17 @@ def _ncu_traffic(storage, n):
         if st == storage and kh == _kernel_hash():
             return b * (n * n) / nodes
     return None
+
+
+def _passes(storage, n, steps, inplace=False):
+    """(passes over the populations, kernel launches) of lks_step(steps) on an n x n lattice.  FP32 and, with
+    two buffers, 16-bit lattices of 2048^2 and more take three steps per pass, what is left over one by one;
+    an in-place pass first saves the edges of its blocks in a launch of its own."""
+    fused = n >= 2048 and (storage == "f32" if inplace else storage != "f64")
+    if not fused:
+        return steps, steps
+    k = steps // 3 - (steps // 3 & 1 if inplace else 0)
+    return k + steps - 3 * k, (2 * k if inplace else k) + steps - 3 * k
 
 
 class ClockSampler:
@@ -299,13 +310,18 @@ def bench_ours(args):
     per_launch = t / args.steps
     peak, peak_kind = _peaks()
     bpn = BYTES_PER_NODE[args.storage]
-    achieved = bpn * nodes / per_launch / 1e9
-    traffic = None if args.inplace else _ncu_traffic(args.storage, n)
+    # bytes: one read and one write of the populations per pass, of one step or of three
+    passes, launches = _passes(args.storage, n, args.steps, args.inplace)
+    achieved = bpn * nodes * passes / t / 1e9
+    traffic = None if args.inplace or passes < args.steps else _ncu_traffic(args.storage, n)
     roofline = {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
                 "frac": round(achieved / peak, 4), "traffic": traffic,
                 "peak_source": "%s (MEASURED_PEAKS.json hbm_gbs)" % peak_kind if peak_kind == "measured" else
                 "fallback 6.8 TB/s",
-                "algorithmic_bytes_per_launch": bpn * nodes, "kernel": ("step_kernel_aa<%s,moment> (both phases)" if args.inplace else "step_kernel<%s,moment>")
+                "algorithmic_bytes_per_launch": bpn * nodes, "passes": passes, "steps": args.steps,
+                "step_by_step": round(bpn * nodes / per_launch / 1e9, 1),
+                "kernel": ("rows_kernel<%s,moment> (three steps per pass)" if passes < args.steps else
+                           "step_kernel_aa<%s,moment> (both phases)" if args.inplace else "step_kernel<%s,moment>")
                 % args.storage}
     # sanity: the state must still be finite (lks_residual reports a non-finite state as LKS_EUNSTABLE)
     lat.residual()
@@ -424,7 +440,7 @@ def bench_ours(args):
         kl = max(10, min(args.steps, 2000))
         tl = max_over_ranks(_time_steps(ll, kl, stream))
         vl = nodes * kl * ws / tl / 1e6
-        al = 152 * nodes / (tl / kl) / 1e9
+        al = 152 * nodes * _passes("f32", n, kl)[0] / tl / 1e9
         extra["lorentz_f32"] = {"value": round(vl, 1), "unit": UNIT, "steps": kl,
                                 "roofline": {"bound": "hbm", "achieved": round(al, 1), "peak": peak, "unit": "GB/s",
                                              "frac": round(al / peak, 4)}}
@@ -440,7 +456,7 @@ def bench_ours(args):
             kr += kr & 1
             tr = max_over_ranks(_time_steps(lr, kr, stream))
             vr = nodes * kr * ws / tr / 1e6
-            ar = BYTES_PER_NODE[st] * nodes / (tr / kr) / 1e9
+            ar = BYTES_PER_NODE[st] * nodes * _passes(st, n, kr, inplace)[0] / tr / 1e9
             extra[key] = {"value": round(vr, 1), "unit": UNIT, "steps": kr,
                           "roofline": {"bound": "hbm", "achieved": round(ar, 1), "peak": peak, "unit": "GB/s",
                                        "frac": round(ar / peak, 4)}}
@@ -490,7 +506,7 @@ def bench_ours(args):
                 "warmup": args.warmup, "ms_per_step": round(per_launch * 1e3, 4), "higher_is_better": True,
                 "scaling": "weak", "vs_baseline": None, "dtype": "f32" if args.storage != "f64" else "f64",
                 "data": "synthetic", "config": _workload(args), "roofline": roofline, "cpu_baseline": cpu,
-                "e2e": e2e, "gpu_launches": args.steps, "clocks": clocks,
+                "e2e": e2e, "gpu_launches": launches, "clocks": clocks,
                 "parallelism": "replicas" if ws > 1 else "single GPU"}
         line.update(extra)
         print(json.dumps(line), flush=True)
@@ -947,7 +963,7 @@ def bench_duct(args):
                       "c_hartmann": 0.5, "c_side": 0.1, "Ha": 20.0,
                       "l2": "inputs larger than L2" if bpn * nodes > 129e6 else "inputs within L2"},
            "roofline": {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
-                        "frac": round(achieved / peak, 4), "kernel": "step3_duct_kernel<%s>" % storage}}
+                        "frac": round(achieved / peak, 4), "kernel": "step3_flat_kernel<%s>" % storage}}
     lat.close()
     print(json.dumps(out), flush=True)
     return 0
@@ -1081,13 +1097,13 @@ def bench_c1(args):
     return 0
 
 
-# FP64 arithmetic per bulk node per step in collide_node, counted from the source with an FMA as
-# 2 flops: moments and 1/rho (Newton) 40, equilibrium set-up 23, nine directions 116, g 33.
-FP64_FLOPS_PER_NODE = 212
-# FP64 pipe instructions per node of the FP64 step kernel (ncu sm__inst_executed_pipe_fp64.sum x 32
-# / nodes at 2048^2) and the pipe's nominal rate (1.25 TFLOP/s = 0.625e12 DFMA/s on GB300)
-FP64_PIPE_INSTR_PER_NODE = 153
-FP64_PIPE_INSTR_PER_NODE_3D = 336
+# FP64 arithmetic per node of the FP64 step kernel without a body force (ncu
+# smsp__sass_thread_inst_executed_op_d{add,mul,fma}_pred_on.sum at 2048^2, an FMA as 2 flops)
+FP64_FLOPS_PER_NODE = 141
+# FP64 pipe instructions per node of the same kernels (ncu sm__inst_executed_pipe_fp64.sum x 32 / nodes;
+# 2D at 2048^2, 3D at 128^3) and the pipe's nominal rate (1.25 TFLOP/s = 0.625e12 DFMA/s on GB300)
+FP64_PIPE_INSTR_PER_NODE = 105
+FP64_PIPE_INSTR_PER_NODE_3D = 222
 FP64_PIPE_PEAK = 0.625e12
 
 
