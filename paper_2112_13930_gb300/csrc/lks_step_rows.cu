@@ -624,8 +624,8 @@ cudaError_t plan_rows(int storage, int closure, const StepParams<double>& p, int
     rp->strip = rp->chunk = rp->edge = 0;
     if (storage == 0 || (storage >= 2 && nx % 2 != 0) || nx < 64) return cudaSuccess;
     if (inplace) {
-        // FP32 only: the interleaved rows of 16-bit storage ran at 64 (BF16) and 58 (FP16) GLUPS against 67 and 83 in AA
-        // pairs (2056 x 1500).  Plane strides are 32-bit.
+        // FP32 only: the interleaved rows of 16-bit storage ran at 64 (BF16) and 58 (FP16) GLUPS at 2056 x 1500
+        // against 72 and 71 in AA pairs.  Plane strides are 32-bit.
         if (storage != 1 || (int64_t)nx * ny * 4 >= (int64_t)1 << 32) return cudaSuccess;
         return plan_typed<InplaceF32>(closure, coupling, force, nx, ny, rp);
     }
