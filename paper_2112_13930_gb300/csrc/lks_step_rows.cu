@@ -37,10 +37,18 @@ namespace {
 // Rows of the first and last chunk, whose blocks test every row for a wall and run about 1.5 times as
 // long a row, as a share of the others'.
 constexpr double kEdgeShare = 0.65;
-// Fewest rows of a chunk: each block also computes kRowSteps - 1 rows beyond either end, so that short
-// chunks lose to single steps (FP32 at 1000 x 513, 7 rows: 53.6 GLUPS against 57.4, 512^2, 4 rows: 43 against
-// 49; at 1000^2, 12 rows: 75 against 43.  FP16 at 512^2, 3 rows: 34 against 50, 1000^2, 9 rows: 69 against 68).
+// Fewest rows of a chunk.  A pass costs about the same per row and block whatever the fit, kRowSteps - 1 rows more
+// per chunk than it stores, so its rate is the share of the computed nodes that are the lattice's own (the plan's
+// use) times 95-129 GLUPS for FP32, 107-133 for BF16, 105-115 for FP16 (measured over widths of 70 to 2048 and
+// chunks of 4 to 106 rows).  Single steps: 43-57 (FP32), 45-73 (16-bit) while both buffers fit in L2, 39-45 and 44-57
+// from memory.  GLUPS, fused against single: FP32 1000 x 513 (use 0.59) 53.6 / 57.4, 132 x 2800 (0.38) 39.7 / 42.9,
+// 264 x 4000 (0.60, from memory) 67.7 / 41.1, 132 x 40000 (0.50, from memory) 64.7 / 40.3; FP16 1500 x 700 (0.61)
+// 64.6 / 68.5, 900 x 1100 (0.64) 70.6 / 64.1, 264 x 2500 (0.39) 42.0 / 48.2; BF16 520 x 1500 (0.50) 59.4 / 59.2.
 constexpr int kRowMinChunk = 8;
+constexpr double kUseL2 = 0.62, kUseMemory = 0.47;
+// In place the saved edges and the blocks' far pulls cost more, the AA pairs less: 1000^2 (0.73, in L2) 35 against 60,
+// 2000 x 800 (0.78) 43.6 / 43.1, 2056 x 1500 (0.88) 55.7 / 43.1, 4096^2 68.4 / 45.0; 250 x 3000 (0.55, in L2) 23 / 54.
+constexpr double kUseInPlace = 0.8;
 // Rows fetched into L2 ahead of their first use (no prefetch: FP16 92.8 instead of 100.3 GLUPS).
 constexpr int kAhead = 2;
 
@@ -587,7 +595,7 @@ typedef Rows<float, OneNode<float>, true, F32S> InplaceF32;
 
 // Strips and chunks of the kernel R: as many blocks as are resident at once.
 template <typename R>
-static cudaError_t plan_typed(int closure, int coupling, bool force, int nx, int ny, RowsPlan* rp) {
+static cudaError_t plan_typed(int closure, int coupling, bool force, int nx, int ny, double least, RowsPlan* rp) {
     int dev = 0, sms = 0, blocks = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -611,7 +619,8 @@ static cudaError_t plan_typed(int closure, int coupling, bool force, int nx, int
             if (2 * (int64_t)edge + (int64_t)(slots - 2) * chunk >= ny) break;
         }
     }
-    if (chunk < kRowMinChunk) return cudaSuccess;
+    const double use = (double)nx * ny / ((double)slots * strips * R::kThreads * R::kNodes * (chunk + kRowSteps - 1));
+    if (chunk < kRowMinChunk || use < least) return cudaSuccess;
     rp->strip = strip;
     rp->chunk = chunk;
     rp->edge = edge;
@@ -623,15 +632,21 @@ cudaError_t plan_rows(int storage, int closure, const StepParams<double>& p, int
     const bool force = (float)p.Fx != 0.0f;
     rp->strip = rp->chunk = rp->edge = 0;
     if (storage == 0 || (storage >= 2 && nx % 2 != 0) || nx < 64) return cudaSuccess;
+    int dev = 0, l2 = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev);
+    if (e != cudaSuccess) return e;
+    const bool memory = (int64_t)(inplace ? 19 : 38) * storage_bytes(storage) * nx * ny > l2;
     if (inplace) {
         // FP32 only: the interleaved rows of 16-bit storage ran at 64 (BF16) and 58 (FP16) GLUPS at 2056 x 1500
         // against 72 and 71 in AA pairs.  Plane strides are 32-bit.
-        if (storage != 1 || (int64_t)nx * ny * 4 >= (int64_t)1 << 32) return cudaSuccess;
-        return plan_typed<InplaceF32>(closure, coupling, force, nx, ny, rp);
+        if (storage != 1 || !memory || (int64_t)nx * ny * 4 >= (int64_t)1 << 32) return cudaSuccess;
+        return plan_typed<InplaceF32>(closure, coupling, force, nx, ny, kUseInPlace, rp);
     }
-    if (storage == 1) return plan_typed<RowsF32>(closure, coupling, force, nx, ny, rp);
-    if (storage == 2) return plan_typed<RowsBf16>(closure, coupling, force, nx, ny, rp);
-    return plan_typed<RowsF16>(closure, coupling, force, nx, ny, rp);
+    const double least = memory ? kUseMemory : kUseL2;
+    if (storage == 1) return plan_typed<RowsF32>(closure, coupling, force, nx, ny, least, rp);
+    if (storage == 2) return plan_typed<RowsBf16>(closure, coupling, force, nx, ny, least, rp);
+    return plan_typed<RowsF16>(closure, coupling, force, nx, ny, least, rp);
 }
 
 size_t rows_workspace(int nx, int ny, const RowsPlan& rp) {

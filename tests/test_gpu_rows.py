@@ -1,15 +1,16 @@
 """Three fused steps per pass over memory (lks_step_rows.cu) against single steps, bit for bit: step(n)
 takes n // 3 fused passes and n % 3 single steps, n calls of step(1) only single ones.  Sizes: the
 narrowest row (one block wraps around it), one block's width and one column more (two strips), a
-ragged last strip, and chunks of eight rows, the fewest that take the fused kernel, up to many."""
+ragged last strip, and chunks of eight rows, the fewest that take the fused kernel, up to many.  Where half of a
+block's columns are idle, the lattice is larger than L2, as the fused kernel asks."""
 import numpy as np
 import pytest
 
 pytestmark = pytest.mark.gpu
 
 # nx (columns of one node for FP32, of two for 16-bit storage), ny: 760 FP32 or 608 16-bit blocks are resident
-SIZES = {"f32": [(64, 5700), (128, 6000), (129, 3100), (1001, 1300)],
-         "bf16": [(64, 4600), (256, 4900), (258, 2500), (1034, 1100)]}
+SIZES = {"f32": [(64, 40000), (128, 6000), (129, 20000), (1001, 1300)],
+         "bf16": [(128, 40000), (256, 4900), (258, 20000), (1034, 1200)]}
 SIZES["f16"] = SIZES["bf16"]
 
 
@@ -47,11 +48,11 @@ def test_fused_steps_equal_single_steps_bitwise(lks, storage, closure, coupling,
 @pytest.mark.parametrize("closure", ["link", "moment"])
 @pytest.mark.parametrize("coupling", ["maxwell", "lorentz"])
 def test_fused_steps_in_place_equal_two_buffer_single_steps_bitwise(lks, closure, coupling):
-    """One buffer (FP32): fused passes come in twos (6 steps), the rest in AA pairs.  (124, 6000) is one strip whose
-    halo columns wrap onto itself, (125, 3100) a second strip of one column's width, (1001, 1307) a last chunk of
-    one row."""
+    """One buffer (FP32, larger than L2): fused passes come in twos (6 steps), the rest in AA pairs.  (124, 14000) is one
+    strip whose halo columns wrap onto itself, (247, 7100) two strips, (1001, 2600) a ragged last strip, (1001, 2527) a
+    last chunk of one row, (2056, 900) the shortest chunks."""
     storage = "f32"
-    for nx, ny in SIZES[storage] + [(124, 6000), (125, 3100), (1001, 1307)]:
+    for nx, ny in [(124, 14000), (247, 7100), (1001, 2640), (1001, 2563), (2056, 900)]:
         kw = dict(closure=closure, storage=storage, coupling=coupling, seed=5, perturb_amp=1e-2)
         a = lks.Lattice(nx, ny, 0.7, 0.9, 0.02, 2e-5, inplace=True, **kw)
         b = lks.Lattice(nx, ny, 0.7, 0.9, 0.02, 2e-5, **kw)
