@@ -17,7 +17,7 @@
 namespace lks {
 
 // ROWS2D: grid (ceil(nx/256), ny), the column and row come from the block indices; otherwise a
-// 1D grid over n = y*nx + x (narrow lattices), split with one 32-bit division.
+// 1D grid over n = y*nx + x (rows2d says when), split with one 32-bit division.
 template <typename S, typename C, int CLOSURE, int COUPLING, bool ROWS2D>
 __global__ void __launch_bounds__(256) step_kernel(const S* fin, const S* gin, S* fout, S* gout,
                                                    const StepParams<C> p) {
@@ -184,9 +184,6 @@ __global__ void __launch_bounds__(256, CLOSURE == 0 ? 3 : 4) step_kernel_pair(co
     for (int a = 0; a < 5; ++a) go[(5 + a) * NP + q] = P::pack(gyA[a], gyB[a]);
 }
 
-// A row-per-grid-row layout when rows are wide enough to fill blocks and ny fits gridDim.y.
-static bool rows2d(int row_items, int ny) { return row_items >= 64 && ny <= 65535; }
-
 template <typename S, bool R2>
 static void launch_pair_grid(const S* fi, const S* gi, S* fo, S* go, const StepParams<float>& p, int closure,
                              dim3 grid, unsigned block, cudaStream_t st) {
@@ -203,7 +200,7 @@ template <typename S>
 static cudaError_t launch_pair(const void* fin, const void* gin, void* fout, void* gout, const StepParams<float>& p,
                                int closure, cudaStream_t st) {
     const int npr = p.nx / 2;
-    const bool flat = !rows2d(npr, p.ny);
+    const bool flat = !rows2d(npr, p.ny, p.N);
     const unsigned block = block_f32(flat ? p.N / 2 : npr, flat ? 1 : p.ny);
     if (!flat)
         launch_pair_grid<S, true>((const S*)fin, (const S*)gin, (S*)fout, (S*)gout, p, closure,
@@ -230,10 +227,10 @@ template <typename S, typename C>
 static cudaError_t launch_typed(const void* fin, const void* gin, void* fout, void* gout, const StepParams<C>& p,
                                 int closure, cudaStream_t st) {
     // FP64 is bound by the FP64 pipe, where the grid shape changes nothing (3.55 GLUPS at 4096^2
-    // either way): it keeps the 1D grid, and its 2D kernels are not instantiated.  Its blocks are
+    // either way with the collision by directions): it keeps the 1D grid, and its 2D kernels are not instantiated.  Its blocks are
     // small (block_f64), so that small lattices use as many SMs as they can
     if constexpr (sizeof(C) == 4) {
-        if (rows2d(p.nx, p.ny)) {
+        if (rows2d(p.nx, p.ny, p.N)) {
             const unsigned block = block_f32(p.nx, p.ny);
             launch_typed_grid<S, C, true>((const S*)fin, (const S*)gin, (S*)fout, (S*)gout, p, closure,
                                           dim3((p.nx + block - 1) / block, p.ny), block, st);

@@ -1,7 +1,7 @@
 // lks_step_aa.cu -- kernels of the in-place (one-buffer) step; the per-node work and the proof
 // that it reproduces the two-buffer step are in lks_aa.cuh.  Same thread layout as the two-buffer
-// kernel: consecutive x positions in consecutive threads, a 2D grid (row = blockIdx.y) for wide
-// FP32 / 16-bit lattices and a 1D grid otherwise.
+// kernel: consecutive x positions in consecutive threads, a 2D grid (row = blockIdx.y) or a 1D
+// grid as rows2d says.
 #include "lks_aa.cuh"
 #include "lks_internal.h"
 #include "lks_packed.cuh"
@@ -245,7 +245,7 @@ template <typename S, typename C, int PHASE>
 static cudaError_t launch_aa_typed(void* f, void* g, const StepParams<C>& p, int closure, cudaStream_t st) {
     // as in the two-buffer step: FP64 is FP64-pipe-bound and keeps the 1D grid of small blocks
     if constexpr (sizeof(C) == 4) {
-        if (p.nx >= 64 && p.ny <= 65535) {
+        if (rows2d(p.nx, p.ny, p.N)) {
             const unsigned block = block_f32(p.nx, p.ny);
             launch_aa_grid<S, C, PHASE, true>((S*)f, (S*)g, p, closure, dim3((p.nx + block - 1) / block, p.ny), block, st);
             return cudaGetLastError();
@@ -272,7 +272,7 @@ static void launch_aa_pair_grid(S* f, S* g, const StepParams<float>& p, int clos
 template <typename S, int PHASE>
 static cudaError_t launch_aa_pair(void* f, void* g, const StepParams<float>& p, int closure, cudaStream_t st) {
     const int npr = p.nx / 2;
-    const bool flat = !(npr >= 64 && p.ny <= 65535);
+    const bool flat = !rows2d(npr, p.ny, p.N);
     const unsigned block = block_f32(flat ? p.N / 2 : npr, flat ? 1 : p.ny);
     if (!flat)
         launch_aa_pair_grid<S, PHASE, true>((S*)f, (S*)g, p, closure, dim3((npr + block - 1) / block, p.ny), block, st);

@@ -41,7 +41,7 @@ constexpr double kEdgeShare = 0.65;
 // per chunk than it stores, so its rate is the share of the computed nodes that are the lattice's own (the plan's
 // use) times 95-129 GLUPS for FP32, 107-133 for BF16, 105-115 for FP16 (measured over widths of 70 to 2048 and
 // chunks of 4 to 106 rows).  Single steps: 43-57 (FP32), 45-73 (16-bit) while both buffers fit in L2, 39-45 and 44-57
-// from memory.  GLUPS, fused against single: FP32 1000 x 513 (use 0.59) 53.6 / 57.4, 132 x 2800 (0.38) 39.7 / 42.9,
+// from memory.  GLUPS, fused against single: FP32 1000 x 513 (use 0.59) 53.6 / 57.4, 132 x 2800 (0.38) 39.7 / 50.3,
 // 264 x 4000 (0.60, from memory) 67.7 / 41.1, 132 x 40000 (0.50, from memory) 64.7 / 40.3; FP16 1500 x 700 (0.61)
 // 64.6 / 68.5, 900 x 1100 (0.64) 70.6 / 64.1, 264 x 2500 (0.39) 42.0 / 48.2; BF16 520 x 1500 (0.50) 59.4 / 59.2.
 constexpr int kRowMinChunk = 8;
