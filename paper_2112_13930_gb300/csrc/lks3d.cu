@@ -1090,7 +1090,10 @@ cudaError_t launch_step3(lks3_handle* h, int src, cudaStream_t st) {
         const S* gi = (const S*)h->g[src];
         S* fo = (S*)h->f[src ^ 1];
         S* go = (S*)h->g[src ^ 1];
-        const bool flat = sizeof(C) == 8 || (p.nx + 63) / 64 * 64 * 2 > 3 * p.nx;  // else a grid row per row
+        // The flattened index for rows that fill blocks badly or are not aligned (rows2d; us a step, grid rows / flat:
+        // FP32 150 x 70 x 50 31.9 / 26.9, 187 x 100 x 60 63.4 / 54.9, FP16 250 x 90 x 60 76.5 / 70.5), else a grid
+        // row per row.
+        const bool flat = sizeof(C) == 8 || (p.nx + 63) / 64 * 64 * 2 > 3 * p.nx || !lks::rows2d(p.nx, p.ny, q.N);
         const unsigned block = sizeof(C) == 8 ? lks::block_f64(q.N)
                                : flat ? lks::block_f32(q.N, 1)
                                // large channels run at the HBM rate, idle lanes or not (160 x 129 x 200: 194 us a step
