@@ -73,10 +73,11 @@ inline unsigned block_f32(int64_t items, int64_t rows) {
 // flattened index?  The latter costs a division but no idle lanes, and its own-node loads and its stores stay
 // aligned where rows do not start on a 32-byte sector (us a step, grid rows / flat: FP32 132 x 2800 8.6 / 7.3,
 // 270 x 900 5.9 / 5.4, 777 x 555 9.3 / 8.8, in place 1001 x 800 14.8 / 13.5, BF16 270 x 1200 7.7 / 6.3; where they do:
-// FP32 96 x 3000 5.7 / 6.1, 520 x 700 7.1 / 7.3).  Large lattices keep grid rows: BF16 in place 1001 x 3000 44.5 / 55.2,
-// FP16 1500 x 1500 27.5 / 29.4.
+// FP32 96 x 3000 5.7 / 6.1, 520 x 700 7.1 / 7.3).  Large lattices keep grid rows (BF16 in place 1001 x 3000 44.5 / 55.2,
+// FP16 1500 x 1500 27.5 / 29.4), and so do wide rows, few of which end with the moment closure's long wall row (FP32
+// 2500 x 75 4.97 / 5.35, 3001 x 60 5.20 / 5.39).
 inline bool rows2d(int items, int ny, int64_t N) {
-    return items >= 64 && ny <= 65535 && (items % 8 == 0 || N >= (int64_t)1 << 21);
+    return items >= 64 && ny <= 65535 && (items % 8 == 0 || items >= 1024 || N >= (int64_t)1 << 21);
 }
 
 // Bytes per stored population for each lks_storage value.
