@@ -9,8 +9,8 @@
 // of the opposite plane; a moment-closure wall row fetches nothing for the slots it reconstructs) into one
 // of the shared-memory stages, with a 16-byte halo on each side for the x-shifted slots (periodic in x:
 // wrapped copies at the row ends), completing on the stage's `full` mbarrier.  The consumer warps take
-// the tasks' nodes 64 at a time: a lane reads 19 words (two x-adjacent nodes; byte_perm for the x shift)
-// into registers, the warp arrives on the stage's `empty` mbarrier, so that the producer refills it
+// the tasks' nodes 64 at a time (lks_ring.cuh): a lane reads 19 words (two x-adjacent nodes; byte_perm for the x
+// shift) into registers, the warp arrives on the stage's `empty` mbarrier, so that the producer refills it
 // while the warp computes, and then come the wall closure, the collision as one float2 (packed FP32x2
 // arithmetic) and 19 packed words stored.  Rows without a wall run a path with no closure code.  Every
 // wait is bounded (kWaitNs); one that runs out sets *err and ends that warp's loop, and the producer
@@ -34,6 +34,7 @@
 #include "lks_packed.cuh"
 #include "lks_pair.cuh"
 #include "lks_pdl.cuh"
+#include "lks_ring.cuh"
 
 namespace lks {
 namespace {
@@ -67,22 +68,31 @@ inline Segments segments_of(int nx) {
     return {n, ((nx + n - 1) / n + 63) / 64};
 }
 
-// A consumer warp's walk over the items of its block's tasks t0, t0 + G, ...: every kConsumerWarps-th item.
-struct ItemWalk {
-    uint32_t it;  // task of the block
-    int c, y, g;  // item of the task, the task's row and segment
-    __device__ __forceinline__ ItemWalk(int warp, int nseg) : it(0), c(warp), y(blockIdx.x / nseg), g(blockIdx.x % nseg) {}
-    __device__ __forceinline__ bool next(uint32_t ntask, const Segments& sg, int dy, int dg) {
-        while (c >= sg.items) {
-            c -= sg.items;
-            ++it;
+// The row and segment of task t0 + k G, for k = 0, 1, ... in order.
+struct TaskAt {
+    uint32_t k;
+    int y, g;  // row, segment
+    __device__ __forceinline__ explicit TaskAt(int nseg) : k(0), y(blockIdx.x / nseg), g(blockIdx.x % nseg) {}
+    __device__ __forceinline__ void to(uint32_t it, int nseg, int dy, int dg) {
+        for (; k < it; ++k) {
             y += dy;
             g += dg;
-            if (g >= sg.n) g -= sg.n, ++y;
+            if (g >= nseg) g -= nseg, ++y;
         }
-        return it < ntask;
     }
 };
+
+// A consumer warp's part in a task in which it has no item (lks_ring.cuh).
+__device__ __forceinline__ bool pass_task(uint64_t* full, uint64_t* empty, uint32_t it, int lane, int* err) {
+    const uint32_t s = it % kStages;
+    if (!mbar_wait_bounded(&full[s], (it / kStages) & 1u, kWaitNs)) {
+        atomicExch(err, 1);
+        return false;
+    }
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&empty[s]);
+    return true;
+}
 
 // D2Q9 (f) and D2Q5 (g) directions of slot k: k < 9 is f_k, 9..13 is g_x,k-9, 14..18 is g_y,k-14.
 __host__ __device__ constexpr int dir_of(int k) { return k < 9 ? k : (k < 14 ? k - 9 : k - 14); }
@@ -110,7 +120,7 @@ __global__ void __launch_bounds__(kThreads, 1) step_kernel_staged(const S* __res
     if (tid == 0) {
         for (int s = 0; s < kStages; ++s) {
             mbar_init(&full[s], 1);
-            mbar_init(&empty[s], sg.items);
+            mbar_init(&empty[s], ring_arrivals(sg.items, kConsumerWarps));
         }
         mbar_init_fence();
     }
@@ -181,14 +191,17 @@ __global__ void __launch_bounds__(kThreads, 1) step_kernel_staged(const S* __res
     // consumers: of item c of a task, a lane holds nodes x0 + 64 c + 2 lane and the next
     typedef Packed<S> P;
     const int dy = (int)(G / nseg), dg = (int)(G % nseg);
-    ItemWalk i(warp, nseg);
-    for (; i.next((uint32_t)nmine, sg, dy, dg); i.c += kConsumerWarps) {
+    const auto skip = [&](uint32_t it) -> bool { return pass_task(full, empty, it, lane, err); };
+    ItemWalk<kConsumerWarps> i(warp);
+    TaskAt at(nseg);
+    for (; i.next((uint32_t)nmine, sg.items, skip); i.c += kConsumerWarps) {
+        at.to(i.it, nseg, dy, dg);
         const uint32_t s = i.it % kStages;
         if (!mbar_wait_bounded(&full[s], (i.it / kStages) & 1u, kWaitNs)) {
             atomicExch(err, 1);
             break;
         }
-        const int y = i.y, x = i.g * seg + 64 * i.c + 2 * lane;
+        const int y = at.y, x = at.g * seg + 64 * i.c + 2 * lane;
         const bool active = x < nx;
         {
             const bool bottom = (y == 0), top = (y == ny - 1);
@@ -293,7 +306,7 @@ __global__ void __launch_bounds__(kThreads, 1) step_kernel_aa_staged(const S* fb
     if (tid == 0) {
         for (int s = 0; s < kStages; ++s) {
             mbar_init(&full[s], 1);
-            mbar_init(&empty[s], sg.items);
+            mbar_init(&empty[s], ring_arrivals(sg.items, kConsumerWarps));
         }
         mbar_init_fence();
     }
@@ -357,14 +370,17 @@ __global__ void __launch_bounds__(kThreads, 1) step_kernel_aa_staged(const S* fb
 
     typedef Packed<S> P;
     const int dy = (int)(G / nseg), dg = (int)(G % nseg);
-    ItemWalk i(warp, nseg);
-    for (; i.next((uint32_t)nmine, sg, dy, dg); i.c += kConsumerWarps) {
+    const auto skip = [&](uint32_t it) -> bool { return pass_task(full, empty, it, lane, err); };
+    ItemWalk<kConsumerWarps> i(warp);
+    TaskAt at(nseg);
+    for (; i.next((uint32_t)nmine, sg.items, skip); i.c += kConsumerWarps) {
+        at.to(i.it, nseg, dy, dg);
         const uint32_t s = i.it % kStages;
         if (!mbar_wait_bounded(&full[s], (i.it / kStages) & 1u, kWaitNs)) {
             atomicExch(err, 1);
             break;
         }
-        const int y = i.y, w = i.g * segw + 32 * i.c + lane;  // the lane's word in its row
+        const int y = at.y, w = at.g * segw + 32 * i.c + lane;  // the lane's word in its row
         const bool active = w < H;
         {
             const bool bottom = (y == 0), top = (y == ny - 1);
