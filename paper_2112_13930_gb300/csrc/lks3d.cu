@@ -31,6 +31,7 @@
 #include "lks_internal.h"
 #include "lks_packed.cuh"
 #include "lks_pdl.cuh"
+#include "lks_ring.cuh"
 #include "lks_vec.cuh"
 
 using lks::load_s;
@@ -578,7 +579,7 @@ __global__ void __launch_bounds__(256) step3_flat_kernel(const S* fin, const S* 
 // each slot with one bulk copy of R' nx elements (two where the task holds a wall row and e_y != 0:
 // that row takes the node's own row of the opposite plane), one slot per lane, into one of
 // kStages3 shared-memory stages, completing on the stage's `full` barrier.  The periodic x pull is
-// an index wrap within the staged row.  The consumer warps take the tasks' nodes 64 at a time: a lane
+// an index wrap within the staged row.  The consumer warps take the tasks' nodes 64 at a time (lks_ring.cuh): a lane
 // reads its slots into registers (two x-adjacent nodes, x even, so one 32-bit word of a staged row per
 // slot), arrives on the stage's `empty` barrier, which the producer waits for before it refills the
 // stage, and then computes both nodes as one float2 (packed FP32 arithmetic), storing one word per
@@ -626,7 +627,7 @@ __global__ void __launch_bounds__(kThreads3, 1) step3_staged_kernel(const S* __r
     if (tid == 0) {
         for (int s = 0; s < kStages3; ++s) {
             lks::mbar_init(&full[s], 1);
-            lks::mbar_init(&empty[s], kItems3);
+            lks::mbar_init(&empty[s], lks::ring_arrivals(kItems3, kConsumerWarps3));
         }
         lks::mbar_init_fence();
     }
@@ -695,14 +696,24 @@ __global__ void __launch_bounds__(kThreads3, 1) step3_staged_kernel(const S* __r
     // consumers: of item c of a task (nodes 64 c ..), a lane holds nodes x, x + 1 (x even) of task row j
     typedef lks::Packed<S> P;
     const int nw = nx / 2;  // words per row
-    const uint32_t nitem = (uint32_t)nmine * kItems3;  // a block's share of at most 2^31 nodes' rows
-    for (uint32_t q = warp; q < nitem; q += kConsumerWarps3) {
-        const uint32_t it = q / kItems3, s = it % kStages3;
+    const auto skip = [&](uint32_t it) -> bool {  // a task in which the warp has no item (lks_ring.cuh)
+        const uint32_t s = it % kStages3;
+        if (!lks::mbar_wait_bounded(&full[s], (it / kStages3) & 1u, kWaitNs)) {
+            atomicExch(err, 1);
+            return false;
+        }
+        __syncwarp();
+        if (lane == 0) lks::mbar_arrive(&empty[s]);
+        return true;
+    };
+    lks::ItemWalk<kConsumerWarps3> q(warp);
+    for (; q.next((uint32_t)nmine, kItems3, skip); q.c += kConsumerWarps3) {
+        const uint32_t it = q.it, s = it % kStages3;
         if (!lks::mbar_wait_bounded(&full[s], (it / kStages3) & 1u, kWaitNs)) {
             atomicExch(err, 1);
             break;
         }
-        const int i = (int)(q % kItems3) * 64 + 2 * lane;
+        const int i = q.c * 64 + 2 * lane;
         const int j = i / nx, x = i - j * nx;
         const int xw = x / 2, xwm = xw == 0 ? nw - 1 : xw - 1, xwp = xw == nw - 1 ? 0 : xw + 1;
         const uint32_t t = (uint32_t)t0 + it * (uint32_t)G;

@@ -111,8 +111,9 @@ def ring(tmp_path_factory):
     return str(d / "ring")
 
 
-# 2D: 15 consumer warps, three stages, rows of 1024 nodes and more have 9 to 16 items a task
-@pytest.mark.parametrize("warps,first,last", [(15, 1, 17)])
+# 2D: 15 consumer warps, three stages, rows of 1024 nodes and more have 9 to 16 items a task; 3D: 11 consumer warps,
+# four stages, 8 items a task
+@pytest.mark.parametrize("warps,first,last", [(15, 1, 17), (11, 8, 8)])
 def test_every_wait_of_the_ring_is_exact(ring, warps, first, last):
     r = subprocess.run([ring, str(warps), str(first), str(last)], capture_output=True, text=True)
     assert r.returncode == 0, r.stdout
