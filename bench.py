@@ -88,17 +88,6 @@ def _ncu_traffic(storage, n):
     return None
 
 
-def _passes(storage, n, steps, inplace=False):
-    """(passes over the populations, kernel launches) of lks_step(steps) on an n x n lattice.  FP32 and, with
-    two buffers, 16-bit lattices of 2048^2 and more take three steps per pass, what is left over one by one;
-    an in-place pass first saves the edges of its blocks in a launch of its own."""
-    fused = n >= 2048 and (storage == "f32" if inplace else storage != "f64")
-    if not fused:
-        return steps, steps
-    k = steps // 3 - (steps // 3 & 1 if inplace else 0)
-    return k + steps - 3 * k, (2 * k if inplace else k) + steps - 3 * k
-
-
 class ClockSampler:
     """nvidia-smi clock/throttle samples during the timed region."""
 
@@ -311,7 +300,7 @@ def bench_ours(args):
     peak, peak_kind = _peaks()
     bpn = BYTES_PER_NODE[args.storage]
     # bytes: one read and one write of the populations per pass, of one step or of three
-    passes, launches = _passes(args.storage, n, args.steps, args.inplace)
+    passes, launches = lat.step_plan(args.steps)
     achieved = bpn * nodes * passes / t / 1e9
     traffic = None if args.inplace or passes < args.steps else _ncu_traffic(args.storage, n)
     roofline = {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
@@ -440,7 +429,7 @@ def bench_ours(args):
         kl = max(10, min(args.steps, 2000))
         tl = max_over_ranks(_time_steps(ll, kl, stream))
         vl = nodes * kl * ws / tl / 1e6
-        al = 152 * nodes * _passes("f32", n, kl)[0] / tl / 1e9
+        al = 152 * nodes * ll.step_plan(kl)[0] / tl / 1e9
         extra["lorentz_f32"] = {"value": round(vl, 1), "unit": UNIT, "steps": kl,
                                 "roofline": {"bound": "hbm", "achieved": round(al, 1), "peak": peak, "unit": "GB/s",
                                              "frac": round(al / peak, 4)}}
@@ -456,7 +445,7 @@ def bench_ours(args):
             kr += kr & 1
             tr = max_over_ranks(_time_steps(lr, kr, stream))
             vr = nodes * kr * ws / tr / 1e6
-            ar = BYTES_PER_NODE[st] * nodes * _passes(st, n, kr, inplace)[0] / tr / 1e9
+            ar = BYTES_PER_NODE[st] * nodes * lr.step_plan(kr)[0] / tr / 1e9
             extra[key] = {"value": round(vr, 1), "unit": UNIT, "steps": kr,
                           "roofline": {"bound": "hbm", "achieved": round(ar, 1), "peak": peak, "unit": "GB/s",
                                        "frac": round(ar / peak, 4)}}

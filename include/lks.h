@@ -160,9 +160,14 @@ lks_status lks_set_walls(lks_handle* h, double c_bottom, double c_top, double u_
  * the whole call in one launch of one thread-block cluster; large FP32 and 16-bit ones take three
  * steps per pass over memory, the n % 3 left over one by one; all others a kernel per step.  The
  * result has the same bits either way.  Launches run as captured CUDA graphs of 64, 32, ..., 2 of
- * them (built on first use, rebuilt after lks_set_walls) plus at most one direct launch.  n must be
+ * them (built on first use, rebuilt after lks_set_walls), the few left over directly.  n must be
  * even for an in-place handle (LKS_EINVAL). */
 lks_status lks_step(lks_handle* h, int64_t n);
+
+/* What lks_step(h, n) would launch: *passes over the populations (each reads and writes all of them once
+ * in device memory, for one step or for several) and *launches of kernels.  Either may be NULL.  No
+ * device work. */
+lks_status lks_step_plan(const lks_handle* h, int64_t n, int64_t* passes, int64_t* launches);
 
 /* Steps taken since lks_create / lks_set_state. */
 int64_t lks_steps_taken(const lks_handle* h);

@@ -275,6 +275,22 @@ cudaError_t launch_once(lks_handle* h, int src, cudaStream_t st) {
     return step_once(h, src, st);
 }
 
+// The steps of lks_step(h, n), in the order they are taken: `resident` in launches of up to kResidentSteps of a
+// resident lattice, `launches` launches of launch_steps(h) each (as graphs where there are enough), `single` one by
+// one.
+struct StepSplit {
+    int64_t resident, launches, single;
+};
+StepSplit split_steps(const lks_handle* h, int64_t n) {
+    StepSplit s = {0, 0, 0};
+    if (h->resident.ctas && n > 1) s.resident = n % kResidentSteps == 1 ? n - 1 : n;
+    n -= s.resident;
+    s.launches = n / launch_steps(h);
+    if (h->rows_work) s.launches &= ~(int64_t)1;  // in place the rest is taken in pairs of steps
+    s.single = n - s.launches * launch_steps(h);
+    return s;
+}
+
 // Capture kGraphLaunches[size] launches starting from buffer `start` into an executable graph.
 cudaError_t build_graph(lks_handle* h, int size, int start) {
     cudaGraph_t graph = nullptr;
@@ -472,8 +488,9 @@ lks_status lks_step(lks_handle* h, int64_t n) {
     if (!h) return fail(nullptr, LKS_EINVAL, "handle is NULL");
     if (n < 0) return fail(h, LKS_EINVAL, "n must be >= 0");
     if (h->p.inplace && (n & 1)) return fail(h, LKS_EINVAL, "an in-place handle steps in pairs: n must be even");
-    while (h->resident.ctas && n > 1) {
-        const int64_t k = n < kResidentSteps ? n : kResidentSteps;
+    const StepSplit split = split_steps(h, n);
+    for (int64_t left = split.resident; left > 0;) {
+        const int64_t k = left < kResidentSteps ? left : kResidentSteps;
         const int to = h->p.inplace ? 0 : (int)(h->cur ^ (k & 1));
         const int from = h->p.inplace ? 0 : h->cur;
         cudaError_t e = lks::launch_resident(h->p.storage, h->p.closure, h->f[from], h->g[from], h->f[to], h->g[to],
@@ -481,12 +498,10 @@ lks_status lks_step(lks_handle* h, int64_t n) {
         if (e != cudaSuccess) return cuda_fail(h, e, "step kernel launch");
         h->cur ^= (int)(k & 1);
         h->steps += k;
-        n -= k;
+        left -= k;
     }
     const int64_t per = launch_steps(h);
-    int64_t left = n / per;  // launches of `per` steps
-    if (h->rows_work) left &= ~(int64_t)1;  // in place the rest is taken in pairs of steps
-    n -= left * per;
+    int64_t left = split.launches;
     for (int g = 0; g < kGraphSizes && !h->graphs_disabled; ++g) {
         while (left >= kGraphLaunches[g] && !h->graphs_disabled) {
             if (!h->graph[g][h->cur]) {
@@ -509,12 +524,24 @@ lks_status lks_step(lks_handle* h, int64_t n) {
         if (!h->rows_work) h->cur ^= 1;
         h->steps += per;
     }
-    for (; n > 0; --n) {
+    for (int64_t k = split.single; k > 0; --k) {
         cudaError_t e = step_once(h, h->cur, h->stream);
         if (e != cudaSuccess) return cuda_fail(h, e, "step kernel launch");
         h->cur ^= 1;
         h->steps += 1;
     }
+    return LKS_OK;
+}
+
+lks_status lks_step_plan(const lks_handle* h, int64_t n, int64_t* passes, int64_t* launches) {
+    if (!h) return fail(nullptr, LKS_EINVAL, "handle is NULL");
+    lks_handle* hm = const_cast<lks_handle*>(h);
+    if (n < 0) return fail(hm, LKS_EINVAL, "n must be >= 0");
+    if (h->p.inplace && (n & 1)) return fail(hm, LKS_EINVAL, "an in-place handle steps in pairs: n must be even");
+    const StepSplit s = split_steps(h, n);
+    const int64_t all = (s.resident + kResidentSteps - 1) / kResidentSteps + s.launches + s.single;
+    if (passes) *passes = all;
+    if (launches) *launches = all + (h->rows_work ? s.launches : 0);  // and one that saves the blocks' edges
     return LKS_OK;
 }
 

@@ -62,6 +62,7 @@ SIGNATURES = {
     "lks_set_walls": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_double, ctypes.c_double, ctypes.c_double,
                                      ctypes.c_double]),
     "lks_step": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int64]),
+    "lks_step_plan": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int64, _i64p, _i64p]),
     "lks_steps_taken": (ctypes.c_int64, [ctypes.c_void_p]),
     "lks_moments": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int, _dp]),
     "lks_moments_device": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int, ctypes.c_void_p]),
@@ -188,6 +189,12 @@ class Lattice:
 
     def step(self, n=1):
         _check(load().lks_step(self._h, int(n)), self._h)
+
+    def step_plan(self, n):
+        """(passes over the populations, kernel launches) that step(n) would take."""
+        passes, launches = ctypes.c_int64(), ctypes.c_int64()
+        _check(load().lks_step_plan(self._h, int(n), ctypes.byref(passes), ctypes.byref(launches)), self._h)
+        return passes.value, launches.value
 
     @property
     def steps(self):
