@@ -1,8 +1,12 @@
-"""lks_step_plan: what lks_step launches.  A pass is one launch, three steps in a fused pass, all steps of a resident
-lattice in one up to 16384."""
+"""lks_step_plan: what lks_step launches.  The lattices that other tests take through the fused rows and the resident
+kernel do take them (their comparisons with single steps would pass without), and the counts are those of the rules:
+a pass is one launch, three steps in a fused pass, all steps of a resident lattice in one up to 16384."""
 import ctypes
 
 import pytest
+
+from test_gpu_resident import SIZES as RESIDENT
+from test_gpu_rows import SIZES as ROWS
 
 pytestmark = pytest.mark.gpu
 
@@ -24,6 +28,24 @@ def _plan(lks, nx, ny, storage, n, closure="link", coupling="maxwell", fx=2e-5, 
         return lat.step_plan(n)
     finally:
         lat.close()
+
+
+@pytest.mark.parametrize("storage", ["f32", "bf16", "f16"])
+@pytest.mark.parametrize("closure", ["link", "moment"])
+@pytest.mark.parametrize("coupling,fx", [("maxwell", 2e-5), ("maxwell", 0.0), ("lorentz", 2e-5)])
+def test_lattices_of_the_rows_test_are_fused(lks, storage, closure, coupling, fx):
+    for nx, ny in ROWS[storage]:
+        assert _plan(lks, nx, ny, storage, 10, closure, coupling, fx) == (4, 4), (nx, ny)  # 3 + 3 + 3 + 1
+
+
+@pytest.mark.parametrize("coupling", ["maxwell", "lorentz"])
+@pytest.mark.parametrize("storage", ["f64", "f32", "bf16", "f16"])
+def test_lattices_of_the_resident_test_are_resident(lks, storage, coupling):
+    for nx, ny in RESIDENT[storage]:
+        assert _plan(lks, nx, ny, storage, 12, coupling=coupling) == (1, 1), (nx, ny)
+        assert _plan(lks, nx, ny, storage, 12, coupling=coupling, inplace=True) == (1, 1), (nx, ny)
+        assert _plan(lks, nx, ny, storage, 16385, coupling=coupling) == (2, 2)  # a launch and a single step
+        assert _plan(lks, nx, ny, storage, 2 * 16384 + 2, coupling=coupling) == (3, 3)
 
 
 def test_counts(lks):
