@@ -138,10 +138,13 @@ cudaError_t launch_rows(int storage, int closure, const void* fin, const void* g
 // where it does not apply.  fin / fout: the buffers before and after `steps` steps (they may be the same);
 // ilv as interleave_row.
 constexpr int kResidentThreads = 1024;  // FP64: half
-// Most nodes: the lattice then has 16 SMs, so that above these single steps on all SMs are faster (us a step,
-// resident against single: FP32 64 x 120 1.17 / 1.41, 64 x 190 1.44 / 1.40; BF16 96 x 96 1.41 / 2.2; FP64 from
-// 129 nodes a CTA on two warps share a sub-partition).
+// Most nodes: above these single steps on all SMs are faster (us a step, resident against single: FP32 64 x 120
+// 1.17 / 1.41, 64 x 190 1.44 / 1.40; BF16 96 x 96 1.41 / 2.2).  For FP64 also most nodes of a CTA, which with fewer
+// rows than 16 are more than a 16th of the lattice: from 129 on two warps share a sub-partition (link closure: 8 x 256,
+// 128 a CTA, 4.73 / 4.98, 128 x 16 5.02 / 4.96; 7 x 289, 133, 6.44 / 5.28, 200 x 8, 200, 8.13 / 5.05, 160 x 3, 320,
+// 11.2 / 4.9).  FP32 and 16-bit CTAs of few wide rows meet the shared-memory limit first (250 x 8 1.17 / 1.70).
 constexpr int64_t kResidentNodesF64 = 2048, kResidentNodesF32 = 10240, kResidentNodes16 = 12288;
+constexpr int kResidentCtaNodesF64 = 128;
 constexpr int kResidentQuads = 2;  // groups of 32 nodes a CTA, four warps each (FP64, Maxwell coupling)
 struct ResidentPlan {
     int ctas, threads, rows_max, quads;

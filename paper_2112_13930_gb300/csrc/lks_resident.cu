@@ -111,6 +111,7 @@ cudaError_t plan_resident(int storage, int closure, int coupling, int nx, int ny
     while (ctas > ny) ctas /= 2;
     rp->rows_max = (ny + ctas - 1) / ctas;
     const int nodes = rp->rows_max * nx;
+    if (storage == 0 && nodes > kResidentCtaNodesF64) return cudaSuccess;
     rp->threads = std::min(storage == 0 ? kResidentThreads / 2 : kResidentThreads, (nodes + 31) / 32 * 32);
     rp->smem = (size_t)2 * 19 * nx * (rp->rows_max + 2) * storage_bytes(storage);
     if (storage == 0 && coupling == 0 && nodes <= 32 * kResidentQuads) {

@@ -3,6 +3,7 @@ kernel do take them (their comparisons with single steps would pass without), an
 a pass is one launch, three steps in a fused pass, all steps of a resident lattice in one up to 16384."""
 import ctypes
 
+import numpy as np
 import pytest
 
 from test_gpu_resident import SIZES as RESIDENT
@@ -42,10 +43,35 @@ def test_lattices_of_the_rows_test_are_fused(lks, storage, closure, coupling, fx
 @pytest.mark.parametrize("storage", ["f64", "f32", "bf16", "f16"])
 def test_lattices_of_the_resident_test_are_resident(lks, storage, coupling):
     for nx, ny in RESIDENT[storage]:
+        if (storage, nx, ny) == ("f64", 7, 289):  # 133 nodes a CTA
+            assert _plan(lks, nx, ny, storage, 12, coupling=coupling) == (12, 12)
+            continue
         assert _plan(lks, nx, ny, storage, 12, coupling=coupling) == (1, 1), (nx, ny)
         assert _plan(lks, nx, ny, storage, 12, coupling=coupling, inplace=True) == (1, 1), (nx, ny)
         assert _plan(lks, nx, ny, storage, 16385, coupling=coupling) == (2, 2)  # a launch and a single step
         assert _plan(lks, nx, ny, storage, 2 * 16384 + 2, coupling=coupling) == (3, 3)
+
+
+@pytest.mark.parametrize("closure", ["link", "moment"])
+@pytest.mark.parametrize("coupling", ["maxwell", "lorentz"])
+def test_fp64_ctas_hold_at_most_128_nodes(lks, closure, coupling):
+    """128 nodes a CTA are resident, bit for bit with single steps; one row or column more is not, nor are lattices of
+    few wide rows, whose CTAs are few."""
+    for nx, ny in [(8, 256), (128, 16), (128, 8), (128, 3)]:
+        a, b = (lks.Lattice(nx, ny, 0.7, 0.9, 0.02, 2e-5, closure, "f64", seed=5, perturb_amp=1e-2, coupling=coupling)
+                for _ in range(2))
+        for lat in (a, b):
+            lat.set_walls(0.4, 3.0, 0.02, -0.04)
+        n = 7
+        assert a.step_plan(n) == ((1, 1) if ny > 3 else (n, n))
+        a.step(n)
+        for _ in range(n):
+            b.step(1)
+        assert all(np.array_equal(x, y) for x, y in zip(a.get_state(), b.get_state())), (nx, ny)
+        a.close()
+        b.close()
+    for nx, ny in [(129, 8), (43, 44), (160, 3), (200, 8), (20, 100)]:
+        assert _plan(lks, nx, ny, "f64", 12, closure, coupling) == (12, 12), (nx, ny)
 
 
 def test_counts(lks):
