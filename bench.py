@@ -268,7 +268,7 @@ def bench_ours(args):
 
     def make(storage, nn=n, inplace=False):
         lat = lks.Lattice(nn, nn, phys["tau_f"], phys["tau_m"], phys["B0"], phys["Fx"], "moment", storage,
-                          inplace=inplace)
+                          inplace=inplace, workspace=inplace)
         lat.set_walls(phys["c"], phys["c"], 0.0, phys["u_w"])
         return lat
 
@@ -301,6 +301,8 @@ def bench_ours(args):
     bpn = BYTES_PER_NODE[args.storage]
     # bytes: one read and one write of the populations per pass, of one step or of three
     passes, launches = lat.step_plan(args.steps)
+    # what in-place fused passes take beyond the handle's footprint
+    workspace = lat.nbytes - lks.footprint_bytes(n, n, "moment", args.storage, inplace=args.inplace)
     achieved = bpn * nodes * passes / t / 1e9
     traffic = None if args.inplace or passes < args.steps else _ncu_traffic(args.storage, n)
     roofline = {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
@@ -497,6 +499,8 @@ def bench_ours(args):
                 "data": "synthetic", "config": _workload(args), "roofline": roofline, "cpu_baseline": cpu,
                 "e2e": e2e, "gpu_launches": launches, "clocks": clocks,
                 "parallelism": "replicas" if ws > 1 else "single GPU"}
+        if args.inplace:
+            line["config"]["workspace_bytes"] = workspace
         line.update(extra)
         print(json.dumps(line), flush=True)
     if ws > 1:

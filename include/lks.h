@@ -120,10 +120,7 @@ typedef struct lks_params {
                               the second reads and writes only the node's own slots), half
                               the population memory at the same bytes per step and the
                               same results bit for bit; lks_step and lks_run_to_steady then
-                              take even step counts (LKS_EINVAL otherwise).  A large FP32
-                              in-place handle also allocates a workspace for the edges of
-                              its kernel's blocks (8 % of the populations at 4096 x 4096)
-                              when it is created; where that fails it steps without.  With 16-bit
+                              take even step counts (LKS_EINVAL otherwise).  With 16-bit
                               storage and even nx the in-place buffer keeps each row
                               interleaved (32-bit word w holds nodes x = w and x = w + nx/2);
                               lks_moments, lks_get_state and lks_set_state present and take
@@ -138,6 +135,17 @@ typedef struct lks_handle lks_handle;
  * residual snapshot, reduction and profile buffers); 0 if the parameters are
  * invalid.  Used for admission control. */
 size_t lks_footprint_bytes(const lks_params* p);
+
+/* Device bytes of a workspace with which an in-place handle takes three steps per pass over memory (FP32,
+ * larger than L2: 8 % of the populations at 4096 x 4096, 5 to 37 % over all sizes that have one);
+ * 0 for every other handle.  Not part of lks_footprint_bytes: without one the handle steps in pairs. */
+size_t lks_workspace_bytes(const lks_handle* h);
+
+/* Lend the handle `bytes` >= lks_workspace_bytes(h) bytes of device memory, 256-byte aligned, for the
+ * steps enqueued from now on: the results are the same bit for bit.  The memory must outlive the handle
+ * or be taken back first (dev = NULL, bytes = 0), and the steps enqueued with it must have finished before it
+ * is used otherwise.  LKS_EINVAL for a handle that has no use for it, or for too few or unaligned bytes. */
+lks_status lks_set_workspace(lks_handle* h, void* dev, size_t bytes);
 
 /* Validate p, allocate (or carve dev_buffer), and enqueue the initial state:
  * equilibria at rho = 1, B = (0, B0), u = u0, where u0 = 0 or, if
@@ -158,9 +166,10 @@ lks_status lks_set_walls(lks_handle* h, double c_bottom, double c_top, double u_
 /* Enqueue n >= 0 fused collide-stream steps (pull-stream, wall closures, moments, equilibria,
  * collision and store in one kernel).  Asynchronous.  Small lattices (up to about 1e4 nodes) take
  * the whole call in one launch of one thread-block cluster; large FP32 and 16-bit ones take three
- * steps per pass over memory, the n % 3 left over one by one; all others a kernel per step.  The
+ * steps per pass over memory, the n % 3 left over one by one (in place: FP32 with a workspace,
+ * lks_set_workspace, six steps per two passes); all others a kernel per step.  The
  * result has the same bits either way.  Launches run as captured CUDA graphs of 64, 32, ..., 2 of
- * them (built on first use, rebuilt after lks_set_walls), the few left over directly.  n must be
+ * them (built on first use, rebuilt after lks_set_walls and lks_set_workspace), the few left over directly.  n must be
  * even for an in-place handle (LKS_EINVAL). */
 lks_status lks_step(lks_handle* h, int64_t n);
 

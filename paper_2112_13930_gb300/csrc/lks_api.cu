@@ -206,8 +206,8 @@ struct lks_handle {
     bool staged = false;              // 16-bit, nx % 8 == 0, nx >= 1024: the staged kernels
     lks::StagedStep ss = {nullptr, 0};
     lks::ResidentPlan resident = {0, 0, 0, 0, 0};  // ctas > 0: all steps of a call in one launch
-    void* rows_work = nullptr;        // in-place handles: the fused steps' workspace
-    lks::RowsPlan rows = {0, 0, 0};     // strip > 0: kRowSteps steps per launch
+    lks::RowsPlan rows = {0, 0, 0};   // strip > 0: kRowSteps steps per launch (in place: with rows_work)
+    void* rows_work = nullptr;        // the workspace lent to an in-place handle
     double c_bot = 0.0, c_top = 0.0, u_bot = 0.0, u_top = 0.0;
     StepParams<double> sp;
     int64_t steps = 0;
@@ -267,9 +267,11 @@ cudaError_t step_once(lks_handle* h, int src, cudaStream_t st) {
 }
 
 // Steps per launch of a graph, and one such launch from buffer (in place: phase) `src`.
-int launch_steps(const lks_handle* h) { return h->rows.strip ? lks::kRowSteps : 1; }
+int launch_steps(const lks_handle* h) {
+    return h->rows.strip && (!h->p.inplace || h->rows_work) ? lks::kRowSteps : 1;
+}
 cudaError_t launch_once(lks_handle* h, int src, cudaStream_t st) {
-    if (h->rows.strip)
+    if (launch_steps(h) > 1)
         return lks::launch_rows(h->p.storage, h->p.closure, h->f[src], h->g[src], h->f[src ^ 1], h->g[src ^ 1], h->sp,
                                 h->rows, h->rows_work, st);
     return step_once(h, src, st);
@@ -447,12 +449,6 @@ lks_status lks_create(const lks_params* p, lks_handle** out) {
     if (e == cudaSuccess) e = lks::plan_resident(p->storage, p->closure, p->coupling, p->nx, p->ny, &h->resident);
     if (e == cudaSuccess && !h->resident.ctas)
         e = lks::plan_rows(p->storage, p->closure, h->sp, p->inplace, &h->rows);
-    if (e == cudaSuccess && p->inplace && h->rows.strip &&
-        cudaMalloc(&h->rows_work, lks::rows_workspace(p->nx, p->ny, h->rows)) != cudaSuccess) {
-        cudaGetLastError();  // no room for it: pairs of single steps
-        h->rows_work = nullptr;
-        h->rows.strip = 0;
-    }
     if (e != cudaSuccess) {
         lks_destroy(h);
         return cuda_fail(nullptr, e, "lks_create");
@@ -467,6 +463,25 @@ lks_status lks_create(const lks_params* p, lks_handle** out) {
         return cuda_fail(nullptr, e, "lks_create: init kernel");
     }
     *out = h;
+    return LKS_OK;
+}
+
+size_t lks_workspace_bytes(const lks_handle* h) {
+    return h && h->p.inplace && h->rows.strip ? lks::rows_workspace(h->p.nx, h->p.ny, h->rows) : 0;
+}
+
+lks_status lks_set_workspace(lks_handle* h, void* dev, size_t bytes) {
+    if (!h) return fail(nullptr, LKS_EINVAL, "handle is NULL");
+    const size_t need = lks_workspace_bytes(h);
+    if (dev) {
+        if (!need) return fail(h, LKS_EINVAL, "the handle has no use for a workspace (lks_workspace_bytes() is 0)");
+        if (bytes < need || ((uintptr_t)dev % kAlign) != 0)
+            return fail(h, LKS_EINVAL, "the workspace is smaller than lks_workspace_bytes() or not 256-byte aligned");
+    } else if (bytes) {
+        return fail(h, LKS_EINVAL, "the workspace is NULL but its size is not 0");
+    }
+    h->rows_work = dev;
+    drop_graphs(h);
     return LKS_OK;
 }
 
@@ -752,7 +767,6 @@ lks_status lks_destroy(lks_handle* h) {
     if (h->stream || h->base) cudaStreamSynchronize(h->stream);
     drop_graphs(h);
     if (h->state_stage) cudaFree(h->state_stage);
-    if (h->rows_work) cudaFree(h->rows_work);
     if (h->owns && h->base) cudaFree(h->base);
     if (h->host_small) cudaFreeHost(h->host_small);
     if (h->cap_stream) cudaStreamDestroy(h->cap_stream);

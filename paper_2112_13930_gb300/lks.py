@@ -58,6 +58,8 @@ class LksParams(ctypes.Structure):
 _PP = ctypes.POINTER(LksParams)
 SIGNATURES = {
     "lks_footprint_bytes": (ctypes.c_size_t, [_PP]),
+    "lks_workspace_bytes": (ctypes.c_size_t, [ctypes.c_void_p]),
+    "lks_set_workspace": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_size_t]),
     "lks_create": (ctypes.c_int, [_PP, ctypes.POINTER(ctypes.c_void_p)]),
     "lks_set_walls": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_double, ctypes.c_double, ctypes.c_double,
                                      ctypes.c_double]),
@@ -144,8 +146,10 @@ class Lattice:
     """One channel lattice resident on the GPU (a wrapped lks_handle)."""
 
     def __init__(self, nx, ny, tau_f, tau_m, B0, Fx=0.0, closure="link", storage="f64", seed=0, perturb_amp=0.0,
-                 stream=None, torch_memory=True, coupling="maxwell", inplace=False):
-        """inplace=True: one population buffer updated in place, steps in pairs (even counts)."""
+                 stream=None, torch_memory=True, coupling="maxwell", inplace=False, workspace=False):
+        """inplace=True: one population buffer updated in place, steps in pairs (even counts).
+        workspace=True: also hold the device memory with which a large FP32 in-place lattice takes three steps per
+        pass (lks_workspace_bytes; none for other lattices)."""
         import torch
         L = load()
         self.nx, self.ny = int(nx), int(ny)
@@ -174,6 +178,13 @@ class Lattice:
             raise LksError(status, msg.decode() if msg else "")
         self._h = h
         self.params = p
+        self._work = None
+        if workspace:
+            n = int(L.lks_workspace_bytes(h))
+            if n:
+                self._work = torch.empty(n, dtype=torch.uint8, device=stream.device)
+                _check(L.lks_set_workspace(h, self._work.data_ptr(), n), h)
+                self.nbytes += n
 
     @property
     def a(self):
@@ -280,7 +291,7 @@ class Lattice:
         if getattr(self, "_h", None) is not None and self._h.value:
             load().lks_destroy(self._h)
             self._h = None
-            self._buf = None
+            self._buf = self._work = None
 
     def __del__(self):
         try:
