@@ -164,13 +164,14 @@ lks_status lks_create(const lks_params* p, lks_handle** out);
 lks_status lks_set_walls(lks_handle* h, double c_bottom, double c_top, double u_bottom, double u_top);
 
 /* Enqueue n >= 0 fused collide-stream steps (pull-stream, wall closures, moments, equilibria,
- * collision and store in one kernel).  Asynchronous.  Small lattices (up to about 1e4 nodes) take
- * the whole call in one launch of one thread-block cluster; large FP32 and 16-bit ones take three
- * steps per pass over memory, the n % 3 left over one by one (in place: FP32 with a workspace,
- * lks_set_workspace, six steps per two passes); all others a kernel per step.  The
- * result has the same bits either way.  Launches run as captured CUDA graphs of 64, 32, ..., 2 of
- * them (built on first use, rebuilt after lks_set_walls and lks_set_workspace), the few left over directly.  n must be
- * even for an in-place handle (LKS_EINVAL). */
+ * collision and store in one kernel).  Asynchronous.  Small lattices (up to about 1e4 nodes) take a
+ * call of a dozen steps or more (the largest of them: a hundred) in one launch of one thread-block
+ * cluster; large FP32 and 16-bit ones take three steps per pass over memory, the n % 3 left over one
+ * by one (in place: FP32 with a workspace, lks_set_workspace, six steps per two passes); all others a
+ * kernel per step.  The result has the same bits either way.  Launches run as captured CUDA graphs
+ * of 64, 32, ..., 2 of them (built on first use, rebuilt after lks_set_walls and
+ * lks_set_workspace), the few left over directly.  n must be even for an in-place handle
+ * (LKS_EINVAL). */
 lks_status lks_step(lks_handle* h, int64_t n);
 
 /* What lks_step(h, n) would launch: *passes over the populations (each reads and writes all of them once

@@ -205,7 +205,7 @@ struct lks_handle {
     int* flag = nullptr;
     bool staged = false;              // 16-bit, nx % 8 == 0, nx >= 1024: the staged kernels
     lks::StagedStep ss = {nullptr, 0};
-    lks::ResidentPlan resident = {0, 0, 0, 0, 0};  // ctas > 0: all steps of a call in one launch
+    lks::ResidentPlan resident = {};  // ctas > 0: the steps of a call, `least` or more, in one launch
     lks::RowsPlan rows = {0, 0, 0};   // strip > 0: kRowSteps steps per launch (in place: with rows_work)
     void* rows_work = nullptr;        // the workspace lent to an in-place handle
     double c_bot = 0.0, c_top = 0.0, u_bot = 0.0, u_top = 0.0;
@@ -285,7 +285,7 @@ struct StepSplit {
 };
 StepSplit split_steps(const lks_handle* h, int64_t n) {
     StepSplit s = {0, 0, 0};
-    if (h->resident.ctas && n > 1) s.resident = n % kResidentSteps == 1 ? n - 1 : n;
+    if (h->resident.ctas && n >= h->resident.least) s.resident = n % kResidentSteps == 1 ? n - 1 : n;
     n -= s.resident;
     s.launches = n / launch_steps(h);
     if (h->rows_work) s.launches &= ~(int64_t)1;  // in place the rest is taken in pairs of steps

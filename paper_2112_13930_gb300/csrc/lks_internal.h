@@ -147,9 +147,20 @@ constexpr int64_t kResidentNodesF64 = 2048, kResidentNodesF32 = 10240, kResident
 constexpr int kResidentCtaNodesF64 = 128;
 constexpr int kResidentQuads = 2;  // groups of 32 nodes a CTA, four warps each (FP64, Maxwell coupling)
 struct ResidentPlan {
-    int ctas, threads, rows_max, quads;
+    int ctas, threads, rows_max, quads, least;
     size_t smem;
 };
+// Fewest steps of a call that are taken in the cluster: starting it, loading the bands and storing them takes 12 us and
+// more, and a step there saves less over one on all SMs the more nodes there are.  us a call, resident / single steps:
+// FP32 4 x 65 (least 12) 8 steps 20.6 / 16.5, 12 steps 22.7 / 26.7; 16 x 128 (16) 16 steps 28.8 / 26.7, 20 steps 30.9 /
+// 35.0; 64 x 64 (28) 20 steps 35.0 / 32.9, 32 steps 45.3 / 47.2; 64 x 128 (79) 64 steps 92.3 / 90.3, 96 steps 129 / 137.
+// 16-bit 64 x 128 (28) 16 steps 39.1 / 34.9, 20 steps 43.2 / 45.2; 110 x 110 (48) 32 steps 80.0 / 73.5, 48 steps 109 / 111.
+// FP64 4 x 65 (4) 2 steps 18.6 / 12.5, 4 steps 22.7 / 22.7; 4 x 257 (14) 8 steps 46.3 / 43.1, 12 steps 62.7 / 67.7; 8 x
+// 256 (45) 32 steps 168 / 162, 48 steps 243 / 244.
+inline int resident_least(int storage, int64_t N) {
+    const int64_t n2 = N * N;
+    return (int)(storage == 0 ? 4 + n2 / 100000 : 12 + n2 / (storage == 1 ? 1000000 : 4000000));
+}
 cudaError_t plan_resident(int storage, int closure, int coupling, int nx, int ny, ResidentPlan* rp);
 cudaError_t launch_resident(int storage, int closure, const void* fin, const void* gin, void* fout, void* gout,
                             const StepParams<double>& pd, const ResidentPlan& rp, int ilv, int steps, cudaStream_t st);

@@ -104,7 +104,7 @@ struct Resident {
 }  // namespace
 
 cudaError_t plan_resident(int storage, int closure, int coupling, int nx, int ny, ResidentPlan* rp) {
-    *rp = ResidentPlan{0, 0, 0, 0, 0};
+    *rp = ResidentPlan{};
     const int64_t N = (int64_t)nx * ny;
     if (N > (storage == 0 ? kResidentNodesF64 : (storage == 1 ? kResidentNodesF32 : kResidentNodes16))) return cudaSuccess;
     int ctas = N <= 512 && storage != 0 ? 8 : 16;
@@ -121,6 +121,7 @@ cudaError_t plan_resident(int storage, int closure, int coupling, int nx, int ny
     }
     if (rp->smem > kResidentSmem) return cudaSuccess;
     rp->ctas = ctas;
+    rp->least = resident_least(storage, N);
     switch (storage) {
         case 0: return Resident<double, double>::prepare(closure, coupling, rp);
         case 1: return Resident<float, float>::prepare(closure, coupling, rp);
