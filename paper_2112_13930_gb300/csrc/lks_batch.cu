@@ -846,7 +846,14 @@ cudaError_t ensure_graph(lks_batch* b) {
 // instance and for FP64, which the FP64 pipe bounds either way.  Rounded up, so that few graphs are built.
 // Threads: one per node of the largest band while the blocks that share an SM fit its registers, at least
 // the T that a check uses.
-void choose_band(lks_batch* b, int nwork) {
+// A launch loads the bands and stores them, and a check stores them first (12-35 us in all) in place of what a step
+// gains on chip: with fewer than kBandSteps steps from one to the next the other kernel is faster.  us a launch,
+// resident / not, FP32: 38 instances of 4 x 33 .. 255 8 steps 53 / 45, 16 steps 55 / 64, 32 steps 78 / 102; 38 of 16 x 64
+// .. 159 8 steps 79 / 56, 16 steps 92 / 90, 32 steps 128 / 142; 18 of 64 x 64 (256 threads) 16 steps 102 / 83, 24 steps 117 /
+// 117; 192 steps with a check every 8, 16 and 32 steps there 1.22, 1.06 and 0.94 times the other kernel's time, over
+// 21 sets of sizes, threads and storage types 0.55-1.32, 0.42-1.09 and 0.35-0.94 times.
+constexpr int64_t kBandSteps = 16;
+void choose_band(lks_batch* b, int nwork, int64_t quantum) {
     b->band_cap = 0;
     b->band_threads = 0;
     if (b->CS == 1 || b->cfg.storage == 0) return;
@@ -854,13 +861,16 @@ void choose_band(lks_batch* b, int nwork) {
     const size_t per_sm = ((size_t)nwork * b->CS + b->nsm - 1) / b->nsm;
     size_t most = 0;
     int nodes = 0;
+    int64_t every = quantum;  // fewest steps from one load or store of the bands to the next
     for (int k = 0; k < nwork; ++k) {
         const Slot& s = b->slots[b->h_work[k]];
+        every = std::min<int64_t>(every, s.inst.check_every);
         const size_t need = band_bytes(s.nx, s.ny, sb, b->CS);
         if (need == 0) return;
         most = std::max(most, need);
         nodes = std::max(nodes, (s.ny + b->CS - 1) / b->CS * s.nx);
     }
+    if (every < kBandSteps) return;
     most = (most + 8191) / 8192 * 8192;
     if (red_bytes(b->T) + most > kMaxBand || per_sm * (most + red_bytes(b->T) + 2048) > 226 * 1024) return;
     b->band_cap = most;
@@ -1046,7 +1056,7 @@ lks_status lks_batch_run(lks_batch* b, int64_t quantum, int32_t* n_running) {
         b->h_ctl->nwork = nwork;
         b->h_ctl->pad = 0;
         b->h_ctl->quantum = quantum;
-        choose_band(b, nwork);
+        choose_band(b, nwork, quantum);
         cudaError_t e = ensure_graph(b);
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(b->d_work, b->h_work, nwork * sizeof(int32_t), cudaMemcpyHostToDevice, b->stream);
