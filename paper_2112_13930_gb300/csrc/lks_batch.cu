@@ -637,6 +637,15 @@ struct Slot {
     int nx = 0, ny = 0;
     InstDev inst;  // as admitted; what a launch changes (cur, steps, state, ...) is in h_res
 };
+// A captured launch and the shape it was captured for.  With a batch's membership the shape changes back and forth
+// (band_cap and band_threads follow the largest instance and the number of instances), and a new graph costs 20 us: two
+// shapes in turn at a quantum of 100 steps 329-336 us a launch with one graph kept, 313 without a change.
+struct BatchGraph {
+    int T = 0, G = 0, CS = 0, band_threads = 0;
+    size_t band_cap = 0;
+    cudaGraphExec_t exec = nullptr;
+};
+constexpr int kBatchGraphs = 8;
 // Device staging a batch keeps for readouts and states: allocating and freeing it on each call, and reading the
 // instance's record back, were a third of the profiles of a small instance (46 -> 31 us for 32 x 33 FP32).
 // Calls above it allocate theirs and give it back.
@@ -665,10 +674,11 @@ struct lks_batch {
     int T = 256, G = 1, CS = 1;
     double* d_stage = nullptr;   // at most kStageKeep bytes, on first use
     size_t stage_bytes = 0;
-    cudaGraphExec_t graph = nullptr;
-    int graph_T = 0, graph_G = 0, graph_CS = 0;
-    size_t band_cap = 0, graph_band_cap = 0;  // shared memory for a resident instance's band; 0: not resident
-    int band_threads = 0, graph_band_threads = 0;
+    size_t band_cap = 0;  // shared memory for a resident instance's band; 0: not resident
+    int band_threads = 0;
+    BatchGraph graphs[kBatchGraphs];
+    int next_graph = 0;  // the one given up when a new one is built
+    cudaGraphExec_t graph = nullptr;  // the current shape's among them
     std::string err;
 };
 
@@ -801,13 +811,16 @@ cudaError_t enqueue_launch(lks_batch* b, cudaStream_t st) {
 }
 
 cudaError_t ensure_graph(lks_batch* b) {
-    if (b->graph && b->graph_T == b->T && b->graph_G == b->G && b->graph_CS == b->CS &&
-        b->graph_band_cap == b->band_cap && b->graph_band_threads == b->band_threads)
-        return cudaSuccess;
-    if (b->graph) {
-        cudaGraphExecDestroy(b->graph);
-        b->graph = nullptr;
-    }
+    for (const BatchGraph& k : b->graphs)
+        if (k.exec && k.T == b->T && k.G == b->G && k.CS == b->CS && k.band_cap == b->band_cap &&
+            k.band_threads == b->band_threads) {
+            b->graph = k.exec;
+            return cudaSuccess;
+        }
+    BatchGraph& slot = b->graphs[b->next_graph];
+    if (slot.exec) cudaGraphExecDestroy(slot.exec);  // no launch is in flight: lks_batch_run waits for its own
+    slot = BatchGraph{};
+    b->graph = nullptr;
     const size_t smem = (size_t)b->G * 4 * (b->T / 32) * sizeof(double);
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(kernel_for(b->cfg), cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -829,15 +842,19 @@ cudaError_t ensure_graph(lks_batch* b) {
         return le;
     }
     if (e != cudaSuccess) return e;
-    e = cudaGraphInstantiate(&b->graph, g, 0);
+    e = cudaGraphInstantiate(&slot.exec, g, 0);
     cudaGraphDestroy(g);
-    if (e == cudaSuccess) {
-        b->graph_T = b->T;
-        b->graph_G = b->G;
-        b->graph_CS = b->CS;
-        b->graph_band_cap = b->band_cap;
-        b->graph_band_threads = b->band_threads;
+    if (e != cudaSuccess) {
+        slot.exec = nullptr;
+        return e;
     }
+    slot.T = b->T;
+    slot.G = b->G;
+    slot.CS = b->CS;
+    slot.band_cap = b->band_cap;
+    slot.band_threads = b->band_threads;
+    b->graph = slot.exec;
+    b->next_graph = (b->next_graph + 1) % kBatchGraphs;
     return e;
 }
 
@@ -1284,7 +1301,8 @@ lks_status lks_batch_memory(const lks_batch* b, size_t* free_bytes, size_t* used
 lks_status lks_batch_destroy(lks_batch* b) {
     if (!b) return LKS_OK;
     cudaStreamSynchronize(b->stream);
-    if (b->graph) cudaGraphExecDestroy(b->graph);
+    for (const BatchGraph& k : b->graphs)
+        if (k.exec) cudaGraphExecDestroy(k.exec);
     if (b->owns && b->pool) cudaFree(b->pool);
     cudaFree(b->d_tab);
     cudaFree(b->d_res);

@@ -41,3 +41,22 @@ def test_cuts_of_the_same_steps_are_equal_bitwise(batch, storage, coupling, inpl
         for quanta in ([240], [16, 14, 40, 2, 68, 100]):
             for w, g in zip(want, solve(quanta, check_every)):
                 assert np.array_equal(w[0], g[0]) and np.array_equal(w[1], g[1]) and w[2:] == g[2:], (check_every, quanta)
+
+
+def test_more_shapes_than_kept_graphs(batch):
+    """A batch keeps the graphs of eight shapes: twelve in turn, twice, give the states of one shape bit for bit."""
+    descs = [batch.make_desc(nx, ny, "link", 0.7, 0.9, 0.02, 2e-5, 0.4, 3.0, seed=k, perturb_amp=1e-2, tol=1e-30,
+                             check_every=100, max_steps=10**6) for k, (nx, ny) in enumerate(SIZES)]
+    shapes = [(T, 1, C) for T in (32, 64, 128, 256) for C in (1, 4, 8)]
+    a, b = (batch.Batch("f32", max_instances=8, pool_bytes=64 << 20, threads_per_group=128, cluster_ctas=8)
+            for _ in range(2))
+    sa, sb = [a.add(d) for d in descs], [b.add(d) for d in descs]
+    for shape in shapes + shapes[::-1] + shapes[:2] * 2:
+        a.set_shape(*shape)
+        a.run(20)
+        b.run(20)
+    for x, y in zip(sa, sb):
+        assert a.result(x)[:2] == b.result(y)[:2] == (batch.INST_RUNNING, 20 * 28)
+        assert all(np.array_equal(p, q) for p, q in zip(a.get_state(x), b.get_state(y)))
+    a.close()
+    b.close()
