@@ -277,6 +277,12 @@ cudaError_t launch_once(lks_handle* h, int src, cudaStream_t st) {
     return step_once(h, src, st);
 }
 
+bool capturing(cudaStream_t st) {
+    cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &s) != cudaSuccess) cudaGetLastError();
+    return s == cudaStreamCaptureStatusActive;
+}
+
 // The steps of lks_step(h, n), in the order they are taken: `resident` in launches of up to kResidentSteps of a
 // resident lattice, `launches` launches of launch_steps(h) each (as graphs where there are enough), `single` one by
 // one.
@@ -285,7 +291,9 @@ struct StepSplit {
 };
 StepSplit split_steps(const lks_handle* h, int64_t n) {
     StepSplit s = {0, 0, 0};
-    if (h->resident.ctas && n >= h->resident.least) s.resident = n % kResidentSteps == 1 ? n - 1 : n;
+    // a cluster launch is a node of the caller's graph; graphs cannot be instantiated while it is captured
+    if (h->resident.ctas && n > 1 && (n >= h->resident.least || capturing(h->stream)))
+        s.resident = n % kResidentSteps == 1 ? n - 1 : n;
     n -= s.resident;
     s.launches = n / launch_steps(h);
     if (h->rows_work) s.launches &= ~(int64_t)1;  // in place the rest is taken in pairs of steps
