@@ -522,7 +522,8 @@ __device__ __forceinline__ void step3_node(const S* fin, const S* gin, S* fout, 
         for (int k = 0; k < 40; ++k) {
             const int a = slot_dir3(k);
             if (EYa(a) != 1) continue;
-            v[k] = wall_in3<C, C>(p, true, false, k, lks::Loader<S, C, false>::ld((k < 19 ? fin : gin) + slot_plane3(k, opp(a)) * N + n));
+            const S* own = (k < 19 ? fin : gin) + slot_plane3(k, opp(a)) * N + n;
+            v[k] = wall_in3<C, C>(p, true, false, k, lks::Loader<S, C, false>::ld(own));
         }
     }
     if (top) {  // entering along e_y = -1: 4, 8, 9, 16, 18; 4
@@ -530,7 +531,8 @@ __device__ __forceinline__ void step3_node(const S* fin, const S* gin, S* fout, 
         for (int k = 0; k < 40; ++k) {
             const int a = slot_dir3(k);
             if (EYa(a) != -1) continue;
-            v[k] = wall_in3<C, C>(p, false, true, k, lks::Loader<S, C, false>::ld((k < 19 ? fin : gin) + slot_plane3(k, opp(a)) * N + n));
+            const S* own = (k < 19 ? fin : gin) + slot_plane3(k, opp(a)) * N + n;
+            v[k] = wall_in3<C, C>(p, false, true, k, lks::Loader<S, C, false>::ld(own));
         }
     }
     if (SIDE && (back || front)) {  // entering along e_z = +1 at z = 0, e_z = -1 at z = nz-1
@@ -539,7 +541,8 @@ __device__ __forceinline__ void step3_node(const S* fin, const S* gin, S* fout, 
             const int a = slot_dir3(k), ey = EYa(a), ez = EZa(a);
             if (!((ez == 1 && back) || (ez == -1 && front))) continue;
             if ((ey == 1 && bottom) || (ey == -1 && top)) continue;  // closed by the y wall above
-            v[k] = side_in3<C, C>(p, ez == 1, k, lks::Loader<S, C, false>::ld((k < 19 ? fin : gin) + slot_plane3(k, opp(a)) * N + n));
+            const S* own = (k < 19 ? fin : gin) + slot_plane3(k, opp(a)) * N + n;
+            v[k] = side_in3<C, C>(p, ez == 1, k, lks::Loader<S, C, false>::ld(own));
         }
     }
     collide3<C, C>(p, [&](int k) -> C { return v[k]; },
@@ -582,7 +585,7 @@ __global__ void __launch_bounds__(256) step3_flat_kernel(const S* fin, const S* 
 // an index wrap within the staged row.  The consumer warps take the tasks' nodes 64 at a time (lks_ring.cuh): a lane
 // reads its slots into registers (two x-adjacent nodes, x even, so one 32-bit word of a staged row per
 // slot), arrives on the stage's `empty` barrier, which the producer waits for before it refills the
-// stage, and then computes both nodes as one float2 (packed FP32 arithmetic), storing one word per
+// stage (with eight items a task, a warp has none in one task of four or so and only arrives there), and then computes both nodes as one float2 (packed FP32 arithmetic), storing one word per
 // plane.  Each slot takes a fixed kTaskNodes3 elements of a stage, so the slot offsets are constants.
 // Rows must be 16-byte aligned: nx a multiple of 8, and nx <= kTaskNodes3.  A wait that runs out
 // (kWaitNs) sets *err and ends that warp's loop; the producer then waits, within the same limit, for

@@ -865,10 +865,10 @@ cudaError_t ensure_graph(lks_batch* b) {
 // the T that a check uses.
 // A launch loads the bands and stores them, and a check stores them first (12-35 us in all) in place of what a step
 // gains on chip: with fewer than kBandSteps steps from one to the next the other kernel is faster.  us a launch,
-// resident / not, FP32: 38 instances of 4 x 33 .. 255 8 steps 53 / 45, 16 steps 55 / 64, 32 steps 78 / 102; 38 of 16 x 64
-// .. 159 8 steps 79 / 56, 16 steps 92 / 90, 32 steps 128 / 142; 18 of 64 x 64 (256 threads) 16 steps 102 / 83, 24 steps 117 /
-// 117; 192 steps with a check every 8, 16 and 32 steps there 1.22, 1.06 and 0.94 times the other kernel's time, over
-// 21 sets of sizes, threads and storage types 0.55-1.32, 0.42-1.09 and 0.35-0.94 times.
+// resident / not, FP32: 38 instances of 4 x 33 .. 255 8 steps 53 / 45, 16 steps 55 / 64, 32 steps 78 / 102; 38 of
+// 16 x 64 .. 159 8 steps 79 / 56, 16 steps 92 / 90, 32 steps 128 / 142; 18 of 64 x 64 (256 threads) 16 steps 102 / 83,
+// 24 steps 117 / 117; 192 steps with a check every 8, 16 and 32 steps there 1.22, 1.06 and 0.94 times the other
+// kernel's time, over 21 sets of sizes, threads and storage types 0.55-1.32, 0.42-1.09 and 0.35-0.94 times.
 constexpr int64_t kBandSteps = 16;
 void choose_band(lks_batch* b, int nwork, int64_t quantum) {
     b->band_cap = 0;

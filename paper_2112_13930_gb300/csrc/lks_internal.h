@@ -73,9 +73,9 @@ inline unsigned block_f32(int64_t items, int64_t rows) {
 // flattened index?  The latter costs a division but no idle lanes, and its own-node loads and its stores stay
 // aligned where rows do not start on a 32-byte sector (us a step, grid rows / flat: FP32 132 x 2800 8.6 / 7.3,
 // 270 x 900 5.9 / 5.4, 777 x 555 9.3 / 8.8, in place 1001 x 800 14.8 / 13.5, BF16 270 x 1200 7.7 / 6.3; where they do:
-// FP32 96 x 3000 5.7 / 6.1, 520 x 700 7.1 / 7.3).  Large lattices keep grid rows (BF16 in place 1001 x 3000 44.5 / 55.2,
-// FP16 1500 x 1500 27.5 / 29.4), and so do wide rows, few of which end with the moment closure's long wall row (FP32
-// 2500 x 75 4.97 / 5.35, 3001 x 60 5.20 / 5.39).
+// FP32 96 x 3000 5.7 / 6.1, 520 x 700 7.1 / 7.3).  Large lattices keep grid rows (BF16 in place 1001 x 3000 44.5 /
+// 55.2, FP16 1500 x 1500 27.5 / 29.4), and so do wide rows, few of which end with the moment closure's long wall row
+// (FP32 2500 x 75 4.97 / 5.35, 3001 x 60 5.20 / 5.39).
 inline bool rows2d(int items, int ny, int64_t N) {
     return items >= 64 && ny <= 65535 && (items % 8 == 0 || items >= 1024 || N >= (int64_t)1 << 21);
 }
@@ -121,9 +121,9 @@ cudaError_t launch_step_aa(int storage, int closure, int phase, void* f, void* g
                            cudaStream_t st, const StagedStep* ss = nullptr);
 
 // kRowSteps fused steps per pass over memory (lks_step_rows.cu): FP32 and 16-bit storage.  kRowSteps is odd,
-// so that a fused pass of a two-buffer handle moves the state to the other buffer as that many single steps do.  strip: columns per block (words of two nodes for 16-bit storage), 0 where the
-// kernel does not apply; chunk: rows per block; edge: rows of the blocks at the bottom wall (at the top
-// wall: what is left).
+// so that a fused pass of a two-buffer handle moves the state to the other buffer as that many single steps do.
+// strip: columns per block (words of two nodes for 16-bit storage), 0 where the kernel does not apply; chunk: rows
+// per block; edge: rows of the blocks at the bottom wall (at the top wall: what is left).
 constexpr int kRowSteps = 3;
 struct RowsPlan {
     int strip, chunk, edge;
@@ -150,13 +150,14 @@ struct ResidentPlan {
     int ctas, threads, rows_max, quads, least;
     size_t smem;
 };
-// Fewest steps of a call that are taken in the cluster: starting it, loading the bands and storing them takes 12 us and
-// more, and a step there saves less over one on all SMs the more nodes there are.  us a call, resident / single steps:
-// FP32 4 x 65 (least 12) 8 steps 20.6 / 16.5, 12 steps 22.7 / 26.7; 16 x 128 (16) 16 steps 28.8 / 26.7, 20 steps 30.9 /
-// 35.0; 64 x 64 (28) 20 steps 35.0 / 32.9, 32 steps 45.3 / 47.2; 64 x 128 (79) 64 steps 92.3 / 90.3, 96 steps 129 / 137.
-// 16-bit 64 x 128 (28) 16 steps 39.1 / 34.9, 20 steps 43.2 / 45.2; 110 x 110 (48) 32 steps 80.0 / 73.5, 48 steps 109 / 111.
-// FP64 4 x 65 (4) 2 steps 18.6 / 12.5, 4 steps 22.7 / 22.7; 4 x 257 (14) 8 steps 46.3 / 43.1, 12 steps 62.7 / 67.7; 8 x
-// 256 (45) 32 steps 168 / 162, 48 steps 243 / 244.
+// Fewest steps of a call that are taken in the cluster: starting it, loading the bands and storing them takes 12 us
+// and more, and a step there saves less over one on all SMs the more nodes there are.  us a call, resident / single
+// steps (in brackets: the least):
+//   FP32 4 x 65 (12) 8 steps 20.6 / 16.5, 12 steps 22.7 / 26.7; 16 x 128 (16) 16 steps 28.8 / 26.7, 20 steps 30.9 /
+//   35.0; 64 x 64 (28) 20 steps 35.0 / 32.9, 32 steps 45.3 / 47.2; 64 x 128 (79) 64 steps 92.3 / 90.3, 96 steps 129 /
+//   137; 16-bit 64 x 128 (28) 16 steps 39.1 / 34.9, 20 steps 43.2 / 45.2; 110 x 110 (48) 32 steps 80.0 / 73.5, 48 steps
+//   109 / 111; FP64 4 x 65 (4) 2 steps 18.6 / 12.5, 4 steps 22.7 / 22.7; 4 x 257 (14) 8 steps 46.3 / 43.1, 12 steps
+//   62.7 / 67.7; 8 x 256 (45) 32 steps 168 / 162, 48 steps 243 / 244.
 inline int resident_least(int storage, int64_t N) {
     const int64_t n2 = N * N;
     return (int)(storage == 0 ? 4 + n2 / 100000 : 12 + n2 / (storage == 1 ? 1000000 : 4000000));
@@ -186,7 +187,8 @@ cudaError_t launch_node_moments(int storage, const void* f, const void* g, int64
 
 // Residual partial sums: nblk blocks write partial[4*blk + k] = (sum du^2, sum u^2, sum db^2, sum b^2)
 // and refresh the snapshot snap[0..N) = u_x, snap[N..2N) = B_x; then one block reduces in fixed order
-// into out[0..4), device or page-locked host memory.  residual_blocks(N) never exceeds kResidualMaxBlocks (8 blocks per SM on 152 SMs).
+// into out[0..4), device or page-locked host memory.  residual_blocks(N) never exceeds kResidualMaxBlocks
+// (8 blocks per SM on 152 SMs).
 constexpr int kResidualMaxBlocks = 1216;
 int residual_blocks(int64_t N);
 

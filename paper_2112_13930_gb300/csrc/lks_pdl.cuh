@@ -6,8 +6,8 @@
 //
 // No kernel triggers its successor before it exits (griddepcontrol.launch_dependents at the start was
 // slower: blocks that wait take the SMs the running kernel left free and then share them, duct 27 us a
-// step).  The fused row kernel and the two-node kernels of 16-bit storage are launched plainly: they
-// gained nothing and lost 1-2 % to the loads below.
+// step).  The fused row kernel and the two-node kernel of 16-bit storage with two buffers are launched plainly:
+// they gained nothing and lost 1-2 % to the loads below.
 //
 // After the wait, loads are plain (coherent) ones: the read-only path is defined for data that nobody
 // writes during the kernel's lifetime, which here begins while the predecessor still writes.
@@ -22,7 +22,8 @@ __device__ __forceinline__ void pdl_wait() {
 
 // Launch `kernel`, which calls pdl_wait() before its first access, so that it may start early.
 template <typename... P, typename... A>
-inline cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t st, A... args) {
+inline cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t st,
+                              A... args) {
     cudaLaunchConfig_t lc = {};
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;

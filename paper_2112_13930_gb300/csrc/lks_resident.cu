@@ -11,9 +11,9 @@ namespace {
 constexpr size_t kResidentSmem = 200 * 1024;  // most dynamic shared memory of a CTA
 
 template <typename S, typename C, int CLOSURE, int COUPLING>
-__global__ void __launch_bounds__(sizeof(C) == 8 ? kResidentThreads / 2 : kResidentThreads) resident_kernel(const S* fin, const S* gin, S* fout, S* gout,
-                                                                    const StepParams<C> p, int rows_max, int ilv,
-                                                                    int steps) {
+__global__ void __launch_bounds__(sizeof(C) == 8 ? kResidentThreads / 2 : kResidentThreads)
+    resident_kernel(const S* fin, const S* gin, S* fout, S* gout, const StepParams<C> p, int rows_max, int ilv,
+                    int steps) {
     extern __shared__ __align__(16) unsigned char res_sm[];
     cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
     Band<S> band;
@@ -80,7 +80,8 @@ struct Resident {
         int clusters = 0;
         // the limit is the function's, shared by every handle: always the same value
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kResidentSmem);
-        if (e == cudaSuccess && rp->ctas > 8) e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        if (e == cudaSuccess && rp->ctas > 8)
+            e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         if (e == cudaSuccess) {
             config(&lc, at, *rp, nullptr);
             e = cudaOccupancyMaxActiveClusters(&clusters, k, &lc);
@@ -96,8 +97,8 @@ struct Resident {
         cudaLaunchConfig_t lc = {};
         cudaLaunchAttribute at[1];
         config(&lc, at, rp, st);
-        return cudaLaunchKernelEx(&lc, kernel(closure, p.coupling, rp.quads > 0), (const S*)fin, (const S*)gin, (S*)fout, (S*)gout, p,
-                                  rp.rows_max, ilv, steps);
+        return cudaLaunchKernelEx(&lc, kernel(closure, p.coupling, rp.quads > 0), (const S*)fin, (const S*)gin,
+                                  (S*)fout, (S*)gout, p, rp.rows_max, ilv, steps);
     }
 };
 
@@ -106,7 +107,8 @@ struct Resident {
 cudaError_t plan_resident(int storage, int closure, int coupling, int nx, int ny, ResidentPlan* rp) {
     *rp = ResidentPlan{};
     const int64_t N = (int64_t)nx * ny;
-    if (N > (storage == 0 ? kResidentNodesF64 : (storage == 1 ? kResidentNodesF32 : kResidentNodes16))) return cudaSuccess;
+    if (N > (storage == 0 ? kResidentNodesF64 : (storage == 1 ? kResidentNodesF32 : kResidentNodes16)))
+        return cudaSuccess;
     int ctas = N <= 512 && storage != 0 ? 8 : 16;
     while (ctas > ny) ctas /= 2;
     rp->rows_max = (ny + ctas - 1) / ctas;

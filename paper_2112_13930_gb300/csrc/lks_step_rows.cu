@@ -5,7 +5,8 @@
 // level 1 (the first step) of row r from global memory, level 2 of row r - 1 from the level-1
 // rows it has just made, and so on; only the last level is stored.  Every level is the ordinary
 // step (pull, wall closures, collision, rounding to the storage type), so the state after kRowSteps
-// steps has the bits of as many single steps.
+// steps has the bits of as many single steps (but for the sign of a zero: without a body force the source terms,
+// + 0, are left out, so a population of -0 may stay one).
 //
 // What the next level pulls from a level: populations with e_x = 0 come from the thread's own
 // column and stay in registers (as storage words: the row above needs none of them back, the
@@ -20,9 +21,11 @@
 // In place (one population buffer) a block overwrites rows and columns that its neighbours still have to
 // pull from.  A copy kernel therefore saves kRowSteps rows or columns on either side of every block
 // boundary first, and pulls that leave the block's own area read the copies.  Inside the area a row is
-// stored two rows after its last pull.  The pass leaves the natural layout, as a pair of AA steps does.  FP32
-// 4096^2 in place: 45.0 -> 68.4 GLUPS, 2056 x 1500: 43.1 -> 55.7 (two buffers: 98 and 95): the copies take 7 %, and
-// the warp with the block's edges holds up the others at the barriers.
+// stored two rows after its last pull.  The pass leaves the natural layout, as a pair of AA steps does.  The copies
+// live in a workspace that the caller lends (lks_set_workspace).  FP32 in place, GLUPS, AA pairs -> fused with a body
+// force / without one: 4096^2 45.2 -> 69.0 / 74.9, 2056 x 1500 43.3 -> 55.4 / 59.0, 2056 x 900 42.6 -> 47.7 / 51.0 (two
+// buffers, fused: 4096^2 97.8 / 100.8, 2056 x 1500 96.1 / 102.5): the copies take 7 %, and the warp with the block's
+// edges holds up the others at the barriers.
 #include <algorithm>
 #include <type_traits>
 
@@ -198,7 +201,9 @@ struct Kept {
     W a0[3], a2[3], a4[3], b2[3], b5, b6;
 };
 
-__device__ __forceinline__ int ey9(int a) { return a == 2 || a == 5 || a == 6 ? 1 : (a == 4 || a == 7 || a == 8 ? -1 : 0); }
+__device__ __forceinline__ int ey9(int a) {
+    return a == 2 || a == 5 || a == 6 ? 1 : (a == 4 || a == 7 || a == 8 ? -1 : 0);
+}
 __device__ __forceinline__ int ey5(int a) { return a == 2 ? 1 : (a == 4 ? -1 : 0); }
 
 // The planes of both buffers (f0..8, gx0..4, gy0..4).  As kernel parameters their addresses are uniform
@@ -280,14 +285,16 @@ __global__ void __launch_bounds__(TB, MINB) rows_kernel(const __grid_constant__ 
             const int vm = v < 0 ? v + ncol : (v >= ncol ? v - ncol : v);
             const int b = (int)blockIdx.y - (y < y0 ? 1 : 0), k = y - (y < y0 ? y0 : y1) + T;
             q.ps = 2 * T * pitch;
-            q.f = (const char*)io.rows + ((uint64_t)(unsigned)(b * 19) * q.ps + (unsigned)k * pitch + vm * (unsigned)sizeof(W));
+            q.f = (const char*)io.rows +
+                  ((uint64_t)(unsigned)(b * 19) * q.ps + (unsigned)k * pitch + vm * (unsigned)sizeof(W));
             q.g = q.f + 9 * (uint64_t)q.ps;
             return q;
         }
         const bool left = v < x0, out = left || v >= x0 + w;
         const int b = left ? blockIdx.x : (blockIdx.x + 1 == gridDim.x ? 0 : blockIdx.x + 1);
         const unsigned saved = 2 * T * sizeof(W) * ny, plane = pitch * ny;
-        const unsigned at_out = (unsigned)y * (2 * T * sizeof(W)) + (v - (left ? x0 : x0 + w) + T) * (unsigned)sizeof(W);
+        const unsigned at_out = (unsigned)y * (2 * T * sizeof(W)) +
+                                (v - (left ? x0 : x0 + w) + T) * (unsigned)sizeof(W);
         const unsigned at_own = (unsigned)y * pitch + v * (unsigned)sizeof(W);
         const char* base = (const char*)io.cols + (uint64_t)(unsigned)(b * 19) * saved;
         const unsigned at = out ? at_out : at_own;
@@ -483,7 +490,8 @@ __global__ void __launch_bounds__(TB, MINB) rows_kernel(const __grid_constant__ 
                      min((px + (t % lines) * (128 / (int)sizeof(W))), ncol - 1) * (int)sizeof(W);
     auto prefetch = [&](int r) {
         const int y = r + kAhead - pey;
-        if (pa < 19 && y >= 0 && y < ny) asm volatile("prefetch.global.L2 [%0];" ::"l"(pf + (uint64_t)((unsigned)y * pitch)));
+        if (pa < 19 && y >= 0 && y < ny)
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(pf + (uint64_t)((unsigned)y * pitch)));
     };
     auto up = [&]() {  // the slots move up one row
         W* q = q0;
@@ -573,7 +581,8 @@ struct Rows {
         if (INPLACE) {
             typedef typename N::W W;
             W *rows = (W*)work, *cols = rows + halos.rows;
-            rows_save_kernel<W><<<dim3(19 * (halos.chunks - 1 + halos.strips), 8), 256, 0, st>>>(io, ncol, p.ny, rp, rows, cols);
+            rows_save_kernel<W><<<dim3(19 * (halos.chunks - 1 + halos.strips), 8), 256, 0, st>>>(io, ncol, p.ny, rp,
+                                                                                                rows, cols);
             io.rows = rows;
             io.cols = cols;
         }

@@ -21,8 +21,9 @@
 // tasks four words long; and 17 warps have 96 registers, too few to hold the words, so they went through
 // a scratch area.  Fifteen warps and the producer have 128.  Three stages: two starve the warps, four and
 // five put more reads among the writes than DRAM likes.  us a step, before -> after: BF16 in place
-// 2056 x 1500 46.2 -> 42.7, 4096^2 205.5 -> 204.0 (two stages 223, five 214.5), 3000^2 113.8 -> 113.0
-// (126, 118); two buffers 1024 x 1000 16.1 -> 14.3, 4096 x 150 10.7 -> 9.8, 2056 x 400 FP16 16.7 -> 14.3.
+// 2056 x 1500 47.8 -> 43.1, 4096^2 206 -> 203 (two stages 223, five 214.5), 3000^2 113.9 -> 112.9 (126, 118); two
+// buffers BF16 1024 x 1000 16.1 -> 15.3, 4096 x 150 10.7 -> 10.2, 2056 x 400 FP16 16.8 -> 14.6.  A warp's wait for the
+// tasks it has no item in is among these times (1 % of them at 11 items a task).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -96,8 +97,12 @@ __device__ __forceinline__ bool pass_task(uint64_t* full, uint64_t* empty, uint3
 
 // D2Q9 (f) and D2Q5 (g) directions of slot k: k < 9 is f_k, 9..13 is g_x,k-9, 14..18 is g_y,k-14.
 __host__ __device__ constexpr int dir_of(int k) { return k < 9 ? k : (k < 14 ? k - 9 : k - 14); }
-__host__ __device__ constexpr int ex9(int a) { return (a == 1 || a == 5 || a == 8) ? 1 : (a == 3 || a == 6 || a == 7) ? -1 : 0; }
-__host__ __device__ constexpr int ey9(int a) { return (a == 2 || a == 5 || a == 6) ? 1 : (a == 4 || a == 7 || a == 8) ? -1 : 0; }
+__host__ __device__ constexpr int ex9(int a) {
+    return (a == 1 || a == 5 || a == 8) ? 1 : (a == 3 || a == 6 || a == 7) ? -1 : 0;
+}
+__host__ __device__ constexpr int ey9(int a) {
+    return (a == 2 || a == 5 || a == 6) ? 1 : (a == 4 || a == 7 || a == 8) ? -1 : 0;
+}
 __host__ __device__ constexpr int opp9(int a) { return a == 0 ? 0 : (a <= 4 ? (a + 1) % 4 + 1 : (a + 1) % 4 + 5); }
 // plane of slot k's population table for direction a (f: a; g_x: a; g_y: 5 + a)
 __host__ __device__ constexpr int plane_of(int k, int a) { return k < 9 ? a : (k < 14 ? a : 5 + a); }
@@ -544,8 +549,9 @@ void launch_typed_aa_staged(void* f, void* g, const StepParams<float>& p, int cl
     const unsigned grid = (unsigned)std::min<int64_t>((int64_t)p.ny * sg.n, ss.grid);
     S* fb = (S*)f;
     S* gb = (S*)g;
-    const auto kernel = p.coupling == 0 ? (closure == 0 ? step_kernel_aa_staged<S, 0, 0> : step_kernel_aa_staged<S, 1, 0>)
-                                        : (closure == 0 ? step_kernel_aa_staged<S, 0, 1> : step_kernel_aa_staged<S, 1, 1>);
+    const auto kernel = p.coupling == 0
+                            ? (closure == 0 ? step_kernel_aa_staged<S, 0, 0> : step_kernel_aa_staged<S, 1, 0>)
+                            : (closure == 0 ? step_kernel_aa_staged<S, 0, 1> : step_kernel_aa_staged<S, 1, 1>);
     launch_pdl(kernel, grid, kThreads, kSmem, st, (const S*)fb, (const S*)gb, planes_of(fb, gb, p.N), p, sg, ss.err);
 }
 
