@@ -170,8 +170,8 @@ lks_status lks_set_walls(lks_handle* h, double c_bottom, double c_top, double u_
  * by one (in place: FP32 with a workspace, lks_set_workspace, six steps per two passes); all others a
  * kernel per step.  The result has the same bits either way.  Launches run as captured CUDA graphs
  * of 64, 32, ..., 2 of them (built on first use, rebuilt after lks_set_walls and
- * lks_set_workspace), the few left over directly.  n must be even for an in-place handle
- * (LKS_EINVAL). */
+ * lks_set_workspace), the few left over directly; on a stream that the caller captures all go out
+ * directly and become nodes of its graph.  n must be even for an in-place handle (LKS_EINVAL). */
 lks_status lks_step(lks_handle* h, int64_t n);
 
 /* What lks_step(h, n) would launch: *passes over the populations (each reads and writes all of them once

@@ -277,12 +277,6 @@ cudaError_t launch_once(lks_handle* h, int src, cudaStream_t st) {
     return step_once(h, src, st);
 }
 
-bool capturing(cudaStream_t st) {
-    cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &s) != cudaSuccess) cudaGetLastError();
-    return s == cudaStreamCaptureStatusActive;
-}
-
 // The steps of lks_step(h, n), in the order they are taken: `resident` in launches of up to kResidentSteps of a
 // resident lattice, `launches` launches of launch_steps(h) each (as graphs where there are enough), `single` one by
 // one.
@@ -291,14 +285,18 @@ struct StepSplit {
 };
 StepSplit split_steps(const lks_handle* h, int64_t n) {
     StepSplit s = {0, 0, 0};
-    // a cluster launch is a node of the caller's graph; graphs cannot be instantiated while it is captured
-    if (h->resident.ctas && n > 1 && (n >= h->resident.least || capturing(h->stream)))
-        s.resident = n % kResidentSteps == 1 ? n - 1 : n;
+    if (h->resident.ctas && n >= h->resident.least) s.resident = n % kResidentSteps == 1 ? n - 1 : n;
     n -= s.resident;
     s.launches = n / launch_steps(h);
     if (h->rows_work) s.launches &= ~(int64_t)1;  // in place the rest is taken in pairs of steps
     s.single = n - s.launches * launch_steps(h);
     return s;
+}
+
+bool capturing(cudaStream_t st) {
+    cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &s) != cudaSuccess) cudaGetLastError();
+    return s == cudaStreamCaptureStatusActive;
 }
 
 // Capture kGraphLaunches[size] launches starting from buffer `start` into an executable graph.
@@ -525,7 +523,9 @@ lks_status lks_step(lks_handle* h, int64_t n) {
     }
     const int64_t per = launch_steps(h);
     int64_t left = split.launches;
-    for (int g = 0; g < kGraphSizes && !h->graphs_disabled; ++g) {
+    // graphs cannot be instantiated while the caller captures the stream: the launches become nodes of its graph
+    const bool direct = left > 1 && capturing(h->stream);
+    for (int g = 0; g < kGraphSizes && !h->graphs_disabled && !direct; ++g) {
         while (left >= kGraphLaunches[g] && !h->graphs_disabled) {
             if (!h->graph[g][h->cur]) {
                 cudaError_t e = build_graph(h, g, h->cur);
